@@ -223,7 +223,8 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
   const size_t o_dPhi = take((size_t)B * phi_walker_stride(s, 1) * sizeof(Det));
   const size_t o_gradc = take((size_t)s->prep.total * sizeof(Cmp));
   const size_t o_dP = take((size_t)sh.R * s->cfg.n_dets * N * sizeof(Cmp));
-  const size_t o_orbP = take(Mode::kMode == FN_BF16_MIXED ? (size_t)sh.R * 4 * s->cfg.n_dets * N * sizeof(float) : 0);
+  const size_t o_orbP = take((size_t)sh.R * 4 * s->cfg.n_dets * N * sizeof(Cmp));
+  // FP32/FP64: the envelope values of the full pass take dP's place (a buffer of the gradient)
   const size_t o_envv = take(Mode::kMode == FN_BF16_MIXED ? (size_t)sh.R * s->cfg.n_dets * N * sizeof(float) : 0);
   const bool bf16 = Mode::kMode == FN_BF16_MIXED;
   int max_k = 0;
@@ -243,7 +244,7 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
     ws->prep16 = b + o_prep16; ws->walk2 = b + o_walk2; ws->lp2 = (double*)(b + o_lp2);
     ws->scratch_d = (double*)(b + o_scr); ws->dX = b + o_dX; ws->dH = b + o_dH; ws->dZ = b + o_dZ;
     ws->dZw = b + o_dZw; ws->dHbar = b + o_dHbar; ws->dG = b + o_dG; ws->dPhi = b + o_dPhi;
-    ws->gradc = b + o_gradc; ws->dP = b + o_dP; ws->orbP = (float*)(b + o_orbP); ws->envv = (float*)(b + o_envv); ws->status = s->d_status; ws->counter = (int64_t*)(b + o_counter);
+    ws->gradc = b + o_gradc; ws->dP = b + o_dP; ws->orbP = b + o_orbP; ws->envv = b + (Mode::kMode == FN_BF16_MIXED ? o_envv : o_dP); ws->status = s->d_status; ws->counter = (int64_t*)(b + o_counter);
     ws->g16 = b + o_g16; ws->t16a = b + o_t16a; ws->t16b = b + o_t16b;
   }
   return off;

@@ -8,18 +8,16 @@
 //                      rows) and its spin means for every layer
 //   k_pair_*_mma       the same on warp-level BF16 MMAs with hi/lo splits (BF16 mode)
 //   k_spin_means_bf16  spin means of a BF16 stream-layer output (next mean-field input)
-//   k_gemm             tiled SIMT GEMM (mean-field term U [hbar_up, hbar_dn] + b)
-//   k_layer            one-electron layer GEMM over all tangent slabs with the fused
-//                      tanh forward-Laplacian epilogue, residual and next spin means
+//   simt::launch_gemm / launch_layer / launch_orbitals (fn_simt.cu)  FP32/FP64 mean-field
+//                      term U [hbar_up, hbar_dn] + b, stream layer and orbitals
 //   k_envelope_values  envelope values per (electron, orbital) for the tensor-core orbitals
-//   k_orbital_fixup    envelope-derivative terms of the tensor-core orbitals
-//   k_orbitals         orbital projection x envelope with the product rule (SIMT)
+//   k_orbital_fixup    envelope-derivative terms of the full pass's orbitals
 #include <algorithm>
 #include <vector>
 
 #include "fn_device.cuh"
-#include "fn_gemm.cuh"
 #include "fn_internal.cuh"
+#include "fn_simt_launch.cuh"
 
 namespace fn {
 
@@ -821,132 +819,11 @@ __global__ void __launch_bounds__(256) k_pair_full_mma(const Wlk* __restrict__ r
 }
 
 // ---------------------------------------------------------------------------------------
-// one-electron layer: for every 128-row walker tile and 64 output columns, loop over
-// the tangent slabs: value first (h = tanh z), then every gradient slab
-// ((1 - h^2) z_t, accumulating sum_t z_t^2), then the Laplacian slab
-// ((1 - h^2) z_lap - 2 h (1 - h^2) sum_t z_t^2); plus the residual and the spin means
-// of the output for the next layer.
-// ---------------------------------------------------------------------------------------
-struct LayerArgs {
-  const void* X; int ldx; int k_self;
-  const void* VsT;      // [k_self][h1]
-  const void* Mterm;    // [T][B][h1]
-  void* Y; int ldy;     // output [T][R][ldy]
-  int residual;
-  void* Hbar_out;       // [T][B][2 h1] or null
-  void* act_out;        // [R][h1] tanh values (value pass) or null
-  int h1;
-};
-
-template <typename Act, typename Cmp, bool FULL>
-__global__ void __launch_bounds__(256) k_layer(Shape sh, LayerArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Cmp* xs = (Cmp*)smem_raw;                // [32][132]
-  Cmp* ws = xs + 32 * 132;                 // [32][64]
-  Cmp* ys = ws + 32 * 64;                  // [128][65]
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int tile = blockIdx.x, n0 = blockIdx.y * 64;
-  const int64_t row0 = (int64_t)tile * 128;
-  const Act* X = (const Act*)a.X;
-  const Cmp* VsT = (const Cmp*)a.VsT;
-  const Cmp* Mt = (const Cmp*)a.Mterm;
-  Act* Y = (Act*)a.Y;
-  const int64_t xslab = sh.R * a.ldx, yslab = sh.R * a.ldy;
-  Cmp hv[8][4], sq[8][4];
-  int wv[8];
-  for (int q = 0; q < 8; ++q) {
-    const int rl = ty * 8 + q, wl = rl / sh.N;
-    const int w = tile * sh.wpt + wl;
-    wv[q] = (wl < sh.wpt && w < sh.B) ? w : -1;
-  }
-  for (int t = 0; t < sh.T; ++t) {
-    Cmp acc[8][4] = {};
-    const Act* Xt = X + t * xslab + row0 * a.ldx;
-    for (int k0 = 0; k0 < a.k_self; k0 += 32) {
-      for (int e = tid; e < 128 * 32; e += 256) {
-        const int rr = e / 32, kk = e % 32;
-        const int k = k0 + kk;
-        xs[kk * 132 + rr] = k < a.k_self ? (Cmp)ld(Xt + (int64_t)rr * a.ldx + k) : (Cmp)0;
-      }
-      for (int e = tid; e < 32 * 64; e += 256) {
-        const int kk = e / 64, nn = e % 64;
-        const int k = k0 + kk, n = n0 + nn;
-        ws[kk * 64 + nn] = (k < a.k_self && n < a.h1) ? VsT[(int64_t)k * a.h1 + n] : (Cmp)0;
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int kk = 0; kk < 32; ++kk) {
-        Cmp av[8], bv[4];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) av[q] = xs[kk * 132 + ty * 8 + q];
-#pragma unroll
-        for (int p = 0; p < 4; ++p) bv[p] = ws[kk * 64 + tx * 4 + p];
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-#pragma unroll
-          for (int p = 0; p < 4; ++p) acc[q][p] += av[q] * bv[p];
-      }
-      __syncthreads();
-    }
-    // epilogue
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int rl = ty * 8 + q;
-      const int64_t row = row0 + rl;
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        const int cl = tx * 4 + p, col = n0 + cl;
-        Cmp out = 0;
-        if (wv[q] >= 0 && col < a.h1) {
-          const Cmp z = acc[q][p] + Mt[((int64_t)t * sh.B + wv[q]) * a.h1 + col];
-          if (t == 0) {
-            const Cmp h = f_tanh(z);
-            hv[q][p] = h;
-            sq[q][p] = 0;
-            out = h;
-            if (a.act_out) ((Cmp*)a.act_out)[row * a.h1 + col] = h;
-          } else if (t < sh.T - 1) {
-            const Cmp h = hv[q][p];
-            out = ((Cmp)1 - h * h) * z;
-            sq[q][p] += z * z;
-          } else {
-            const Cmp h = hv[q][p], d = (Cmp)1 - h * h;
-            out = d * z - (Cmp)2 * h * d * sq[q][p];
-          }
-          if (a.residual) out += (Cmp)ld(X + t * xslab + row * a.ldx + col);
-          st(Y + t * yslab + row * a.ldy + col, out);
-        }
-        ys[rl * 65 + cl] = out;
-      }
-    }
-    if (a.Hbar_out) {
-      __syncthreads();
-      Act* Hb = (Act*)a.Hbar_out;
-      for (int e = tid; e < sh.wpt * 2 * 64; e += 256) {
-        const int wl = e / 128, s = (e / 64) % 2, cl = e % 64, col = n0 + cl;
-        const int w = tile * sh.wpt + wl;
-        if (w >= sh.B || col >= a.h1) continue;
-        const int lo = s ? sh.n_up : 0, hi = s ? sh.N : sh.n_up;
-        Cmp sum = 0;
-        for (int i = lo; i < hi; ++i) sum += ys[(wl * sh.N + i) * 65 + cl];
-        st(Hb + ((int64_t)t * sh.B + w) * 2 * a.h1 + s * a.h1 + col, hi > lo ? sum / (Cmp)(hi - lo) : (Cmp)0);
-      }
-      __syncthreads();
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------
 // orbitals: phi^{k}_i(r_j) = (w_ki . h_j + g_ki) * env_ki(r_j), with the product rule
 // over the tangent slabs; envelope derivatives only along r_j.
 // ---------------------------------------------------------------------------------------
-struct OrbArgs {
-  const void* HL;               // [T][R][h1]
-  const void* wT[2]; const void* g[2]; const void* pi[2]; const void* sig[2];
-  void* Phi;                    // [B][PW]
-  int64_t PW;                   // elements per walker
-  int h1, K, aniso;
-};
+using simt::LayerArgs;
+using simt::OrbArgs;
 
 // Envelope sum_m pi exp(-s_m) of orbital ko at electron position rj (Eq. 4), its gradient
 // along rj and its Laplacian.  Isotropic: s = sigma |d|; anisotropic: s = |Sigma d|, with
@@ -988,11 +865,11 @@ __device__ __forceinline__ void env_jet(const OrbArgs& a, int spin, int ko, cons
   *le_out = le;
 }
 
-// Envelope-derivative terms of the tensor-core orbital pass: on the slabs of the row's own
+// Envelope-derivative terms of the full pass: on the slabs of the row's own
 // coordinates phi += P_0 d_c env, on the Laplacian slab phi += 2 sum_c P_c d_c env + P_0 lap env.
-template <typename PhiT, typename Wlk>
+template <typename Cmp, typename PhiT, typename Wlk>
 __global__ void k_orbital_fixup(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbArgs a,
-                                const float* __restrict__ orbP) {
+                                const Cmp* __restrict__ orbP) {
   const int w = blockIdx.x / sh.N, j = blockIdx.x % sh.N;
   const int spin = j < sh.n_up ? 0 : 1;
   const int n_s = spin ? sh.n_dn : sh.n_up;
@@ -1001,18 +878,18 @@ __global__ void k_orbital_fixup(const Wlk* __restrict__ r, const double* __restr
   const int jj = j - (spin ? sh.n_up : 0);
   const int64_t row = tile_row(w, j, sh.N, sh.wpt);
   const int ldp = a.K * sh.N, poff = spin ? a.K * sh.n_up : 0;
-  float env, ge[3], le;
-  env_jet<float, Wlk>(a, spin, ko, r + ((int64_t)w * sh.N + j) * 3, nuc, sh.M, &env, ge, &le);
-  const float* pr = orbP + row * 4 * ldp + poff + ko;
-  const float P0 = pr[0];
+  Cmp env, ge[3], le;
+  env_jet<Cmp, Wlk>(a, spin, ko, r + ((int64_t)w * sh.N + j) * 3, nuc, sh.M, &env, ge, &le);
+  const Cmp* pr = orbP + row * 4 * ldp + poff + ko;
+  const Cmp P0 = pr[0];
   const int k = ko / n_s, i = ko % n_s;
   const int64_t nn = (int64_t)n_s * n_s;
   PhiT* base = (PhiT*)a.Phi + (int64_t)w * a.PW + (spin ? (int64_t)a.K * sh.T * sh.n_up * sh.n_up : 0) +
                (int64_t)k * sh.T * nn + i * n_s + jj;
-  float lap = P0 * le;
+  Cmp lap = P0 * le;
   for (int c = 0; c < 3; ++c) {
     base[(1 + 3 * j + c) * nn] += (PhiT)(P0 * ge[c]);
-    lap += 2.f * pr[(1 + c) * ldp] * ge[c];
+    lap += (Cmp)2 * pr[(1 + c) * ldp] * ge[c];
   }
   base[(sh.T - 1) * nn] += (PhiT)lap;
 }
@@ -1128,54 +1005,6 @@ __global__ void k_envelope_values_smem(const Wlk* __restrict__ r, const double* 
   }
 }
 
-template <typename Act, typename Cmp, typename PhiT, typename Wlk, bool FULL>
-__global__ void k_orbitals(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Cmp* hs = (Cmp*)smem_raw;     // [h1]
-  const int w = blockIdx.x / sh.N, j = blockIdx.x % sh.N;
-  const int spin = j < sh.n_up ? 0 : 1;
-  const int n_s = spin ? sh.n_dn : sh.n_up;
-  const int jj = j - (spin ? sh.n_up : 0);
-  const int n_ko = a.K * n_s;
-  const int ko = threadIdx.x;
-  const bool active = ko < n_ko;
-  const int64_t row = tile_row(w, j, sh.N, sh.wpt);
-  const Cmp* wT = (const Cmp*)a.wT[spin];
-  // envelope value, gradient along r_j and Laplacian
-  Cmp env = 0, ge[3] = {0, 0, 0}, le = 0;
-  const Wlk* rj = r + ((int64_t)w * sh.N + j) * 3;
-  if (active) env_jet<Cmp, Wlk>(a, spin, ko, rj, nuc, sh.M, &env, ge, &le);
-  const int k = active ? ko / n_s : 0, i = active ? ko % n_s : 0;
-  PhiT* out = (PhiT*)a.Phi + (int64_t)w * a.PW +
-             (spin ? (int64_t)a.K * sh.T * sh.n_up * sh.n_up : 0) + (int64_t)k * sh.T * n_s * n_s +
-             (int64_t)i * n_s + jj;
-  const int64_t tstride = (int64_t)n_s * n_s;
-  const int64_t hslab = sh.R * a.h1;
-  const Act* HL = (const Act*)a.HL;
-  Cmp p0 = 0, pj[3] = {0, 0, 0};
-  for (int t = 0; t < sh.T; ++t) {
-    for (int c = threadIdx.x; c < a.h1; c += blockDim.x) hs[c] = (Cmp)ld(HL + t * hslab + row * a.h1 + c);
-    __syncthreads();
-    if (active) {
-      Cmp p = t == 0 ? ((const Cmp*)a.g[spin])[ko] : (Cmp)0;
-      for (int c = 0; c < a.h1; ++c) p += hs[c] * wT[(int64_t)c * n_ko + ko];
-      Cmp phi;
-      if (t == 0) {
-        p0 = p;
-        phi = p * env;
-      } else if (t < sh.T - 1) {
-        const int e = (t - 1) / 3, c = (t - 1) % 3;
-        phi = p * env;
-        if (e == j) { pj[c] = p; phi += p0 * ge[c]; }
-      } else {
-        phi = p * env + (Cmp)2 * (pj[0] * ge[0] + pj[1] * ge[1] + pj[2] * ge[2]) + p0 * le;
-      }
-      out[t * tstride] = (PhiT)phi;
-    }
-    __syncthreads();
-  }
-}
-
 // ---------------------------------------------------------------------------------------
 // orchestration
 // ---------------------------------------------------------------------------------------
@@ -1253,8 +1082,9 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
                             (const float*)(prep + s->prep.b[l]), sh.B, 1, false, ws.status, st, sh.T * sh.B))
           const_cast<fn_system*>(s)->host_error = FN_ERR_CUDA;
       } else {
-        gemm<Act, Cmp, Cmp, Cmp>(st, sh.T * sh.B, h1, 2 * d.d_h, Hb, 2 * d.d_h, 1, prep + s->prep.UT[l], h1, 1,
-                                 (Cmp*)ws.Mterm, h1, 1, prep + s->prep.b[l], sh.B, 1, false);
+        simt::launch_gemm<Cmp>({(int64_t)sh.T * sh.B, h1, 2 * d.d_h, (const Cmp*)ws.Hbar[l], 2 * d.d_h,
+                                prep + s->prep.UT[l], h1, (Cmp*)ws.Mterm, h1, prep + s->prep.b[l], sh.B, 0},
+                               false, false, 1, s->sm_count, st);
       }
     }
     LayerArgs la{};
@@ -1283,15 +1113,7 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
       }
       continue;
     }
-    const size_t smem = sizeof(Cmp) * (32 * 132 + 32 * 64 + 128 * 65);
-    dim3 grid(sh.tiles, (h1 + 63) / 64);
-    if (full) {
-      cudaFuncSetAttribute(k_layer<Act, Cmp, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_layer<Act, Cmp, true><<<grid, 256, smem, st>>>(sh, la);
-    } else {
-      cudaFuncSetAttribute(k_layer<Act, Cmp, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_layer<Act, Cmp, false><<<grid, 256, smem, st>>>(sh, la);
-    }
+    simt::launch_layer<Cmp>(sh, la, s->sm_count, st);
   }
   {
     OrbArgs oa{};
@@ -1303,8 +1125,7 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
     oa.Phi = ws.Phi;
     oa.PW = phi_walker_stride(s, sh.T);
     oa.h1 = h1; oa.K = s->cfg.n_dets; oa.aniso = s->cfg.envelope == FN_ENV_ANISOTROPIC;
-    const int ko_max = s->cfg.n_dets * std::max(s->n_up, s->n_dn);
-    const int threads = (int)std::min<int64_t>(1024, round_up(ko_max, 32));
+    oa.walkers = walkers; oa.nuclei = s->d_nuclei; oa.envv = ws.envv; oa.orbP = ws.orbP;
     if (Mode::kMode == FN_BF16_MIXED) {
       {
       ProfScope ps(s->prof, full ? kProfOrbFull : kProfOrbValue, st);
@@ -1320,32 +1141,28 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         const unsigned gx = (unsigned)((per_walker + 255) / 256);
         const unsigned gy = (unsigned)std::max(1, std::min(sh.B, (s->sm_count * 8 + (int)gx - 1) / (int)gx));
         cudaFuncSetAttribute(k_envelope_values_smem<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)env_smem);
-        k_envelope_values_smem<Wlk><<<dim3(gx, gy), 256, env_smem, st>>>(r, s->d_nuclei, sh, oa, ws.envv);
+        k_envelope_values_smem<Wlk><<<dim3(gx, gy), 256, env_smem, st>>>(r, s->d_nuclei, sh, oa, (float*)ws.envv);
       } else {
-        k_envelope_values<Wlk><<<(unsigned)((n_env + 255) / 256), 256, 0, st>>>(r, s->d_nuclei, sh, oa, ws.envv);
+        k_envelope_values<Wlk><<<(unsigned)((n_env + 255) / 256), 256, 0, st>>>(r, s->d_nuclei, sh, oa, (float*)ws.envv);
       }
       const float* wb[2] = {(const float*)oa.g[0], (const float*)oa.g[1]};
       const float* pis[2] = {(const float*)oa.pi[0], (const float*)oa.pi[1]};
       const float* sgs[2] = {(const float*)oa.sig[0], (const float*)oa.sig[1]};
       if (!launch_orbitals_tc(sh, ws.HL, h1, (const __nv_bfloat16*)ws.prep16 + s->prep.W16, wb, pis, sgs,
-                              s->cfg.n_dets, oa.aniso, (const float*)walkers, s->d_nuclei, ws.Phi, oa.PW, ws.orbP,
-                              ws.envv, ws.status, st))
+                              s->cfg.n_dets, oa.aniso, (const float*)walkers, s->d_nuclei, ws.Phi, oa.PW,
+                              (float*)ws.orbP, (const float*)ws.envv, ws.status, st))
         const_cast<fn_system*>(s)->host_error = FN_ERR_CUDA;
       }
-      if (full) {
-        const int ko_max = s->cfg.n_dets * std::max(s->n_up, s->n_dn);
-        ProfScope ps2(s->prof, kProfOrbFix, st);
-        k_orbital_fixup<typename Mode::PhiT, Wlk><<<(unsigned)((int64_t)sh.B * sh.N), (unsigned)round_up(ko_max, 32), 0,
-                                                    st>>>(r, s->d_nuclei, sh, oa, ws.orbP);
-      }
-      return;
+    } else {
+      ProfScope ps(s->prof, full ? kProfOrbFull : kProfOrbValue, st);
+      simt::launch_orbitals<Cmp>(sh, oa, s->sm_count, st);
     }
-    ProfScope ps(s->prof, full ? kProfOrbFull : kProfOrbValue, st);
-    const size_t smem = sizeof(Cmp) * h1;
-    const unsigned blocks = (unsigned)((int64_t)sh.B * sh.N);
-    using PhiT = typename Mode::PhiT;
-    if (full) k_orbitals<Act, Cmp, PhiT, Wlk, true><<<blocks, threads, smem, st>>>(r, s->d_nuclei, sh, oa);
-    else k_orbitals<Act, Cmp, PhiT, Wlk, false><<<blocks, threads, smem, st>>>(r, s->d_nuclei, sh, oa);
+    if (full) {
+      const int ko_max = s->cfg.n_dets * std::max(s->n_up, s->n_dn);
+      ProfScope ps(s->prof, kProfOrbFix, st);
+      k_orbital_fixup<Cmp, typename Mode::PhiT, Wlk><<<(unsigned)((int64_t)sh.B * sh.N), (unsigned)round_up(ko_max, 32), 0,
+                                                       st>>>(r, s->d_nuclei, sh, oa, (const Cmp*)ws.orbP);
+    }
   }
 }
 

@@ -200,8 +200,8 @@ struct Workspace {
   void* dPhi = nullptr;          // [B][orbital block, value slab] (Det)
   void* gradc = nullptr;         // prepared-layout gradient accumulator (Cmp)
   void* dP = nullptr;            // [R][K (n_up + n_dn)] gradient wrt orbital projections (Cmp)
-  float* orbP = nullptr;         // [R][4][K N] projections for the orbital envelope fix-up (BF16 mode)
-  float* envv = nullptr;         // [R][K N] envelope values (BF16 mode)
+  void* orbP = nullptr;          // [R][4][K N] projections for the orbital envelope fix-up (Cmp)
+  void* envv = nullptr;          // [R][K N] envelope values (Cmp)
   // BF16-mode backward operands for the tensor-core GEMMs
   void* g16 = nullptr;           // [R][max(h1, ldWT)] bf16 copy of dZ or dP
   void* t16a = nullptr;          // [max(k_self, h1)][R] bf16 transposed activations (X_l^T, h_L^T)

@@ -88,7 +88,7 @@ static size_t value_pass_layout(const fn_system* s, int B, unsigned char* base, 
     ws->prep = base + o_prep;
     ws->prep16 = base + o_prep16;
     ws->status = s->d_status;            // kernels report into the handle's word, read by fn_sync
-    ws->envv = (float*)(base + o_envv);
+    ws->envv = base + o_envv;
     ws->base = base;
     ws->bytes = off;
     ws->cap_B = B;
