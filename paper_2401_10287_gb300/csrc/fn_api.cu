@@ -180,6 +180,15 @@ static void build_layout(fn_system* s) {
   }
   p.total = q;
   p.total16 = q16;
+  int64_t q3 = 0;
+  if (s->cfg.precision == FN_FP32 && h1 % 128 == 0) {
+    for (int l = 0; l < L; ++l) {
+      p.V3[l] = q3; q3 += (int64_t)h1 * 3 * round_up(s->layer[l].k_self, 64);
+      p.U3[l] = q3; q3 += (int64_t)h1 * 3 * round_up(2 * s->layer[l].d_h, 64);
+    }
+    for (int a = 0; a < 2; ++a) { p.W3[a] = q3; q3 += (int64_t)K * ns[a] * 3 * h1; }
+  }
+  p.total3 = q3;
 }
 
 template <class Mode>
@@ -211,6 +220,7 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
   const size_t o_Phi = take((size_t)B * phi_walker_stride(s, T) * sizeof(typename Mode::PhiT));
   const size_t o_prep = take((size_t)s->prep.total * sizeof(Cmp));
   const size_t o_prep16 = take((size_t)s->prep.total16 * sizeof(__nv_bfloat16));
+  const size_t o_prep3 = take((size_t)s->prep.total3 * sizeof(__nv_bfloat16));
   const size_t o_walk2 = take((size_t)B * N * 3 * sizeof(Wlk));
   const size_t o_lp2 = take((size_t)B * sizeof(double));
   const size_t o_scr = take((size_t)B * sizeof(double) * 2);
@@ -241,7 +251,7 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
       ws->gpair[l] = b + o_gp[l];
     }
     ws->HL = b + o_HL; ws->Mterm = b + o_M; ws->Phi = b + o_Phi; ws->prep = b + o_prep;
-    ws->prep16 = b + o_prep16; ws->walk2 = b + o_walk2; ws->lp2 = (double*)(b + o_lp2);
+    ws->prep16 = b + o_prep16; ws->prep3 = b + o_prep3; ws->walk2 = b + o_walk2; ws->lp2 = (double*)(b + o_lp2);
     ws->scratch_d = (double*)(b + o_scr); ws->dX = b + o_dX; ws->dH = b + o_dH; ws->dZ = b + o_dZ;
     ws->dZw = b + o_dZw; ws->dHbar = b + o_dHbar; ws->dG = b + o_dG; ws->dPhi = b + o_dPhi;
     ws->gradc = b + o_gradc; ws->dP = b + o_dP; ws->orbP = b + o_orbP; ws->envv = b + (Mode::kMode == FN_BF16_MIXED ? o_envv : o_dP); ws->status = s->d_status; ws->counter = (int64_t*)(b + o_counter);
@@ -500,7 +510,7 @@ fn_status fn_log_psi(fn_system_t s, const void* d_params, const void* d_walkers,
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
     const Shape sh = make_shape(s, B, 1);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, false, cs);
     launch_forward<Mode>(s, d_walkers, sh, false, cs);
     launch_det_energy<Mode>(s, d_walkers, sh, nullptr, d_log_psi, d_sign, false, cs);
     return 0;
@@ -517,7 +527,7 @@ fn_status fn_local_energy(fn_system_t s, const void* d_params, const void* d_wal
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
     const Shape sh = make_shape(s, B, 3 * s->N + 2);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, true, cs);
     launch_forward<Mode>(s, d_walkers, sh, false, cs);
     launch_det_energy<Mode>(s, d_walkers, sh, d_e_local, d_log_psi, d_sign, false, cs);
     return 0;
@@ -538,7 +548,7 @@ fn_status fn_mcmc_steps(fn_system_t s, const void* d_params, void* d_walkers, do
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
     const Shape sh = make_shape(s, B, 1);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, false, cs);
     for (int k = 0; k < n_steps; ++k) {
       const uint32_t step = (uint32_t)(step_offset + (uint64_t)k);
       launch_propose<Mode>(s, B, d_walkers, s->ws.walk2, step_size, seed, step, cs);
@@ -562,7 +572,7 @@ fn_status fn_energy_grad(fn_system_t s, const void* d_params, const void* d_walk
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
     const Shape sh = make_shape(s, B, 1);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, false, cs);
     launch_forward<Mode>(s, d_walkers, sh, true, cs);
     launch_det_energy<Mode>(s, d_walkers, sh, nullptr, s->ws.lp2, nullptr, true, cs);
     launch_energy_weights<Mode>(s, B, d_e_local, s->ws.scratch_d, d_e_mean, cs);
@@ -583,7 +593,7 @@ fn_status fn_log_psi_vjp(fn_system_t s, const void* d_params, const void* d_walk
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
     const Shape sh = make_shape(s, B, 1);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, false, cs);
     launch_forward<Mode>(s, d_walkers, sh, true, cs);
     launch_det_energy<Mode>(s, d_walkers, sh, nullptr, s->ws.lp2, nullptr, true, cs);
     launch_backward<Mode>(s, d_walkers, sh, d_weights, d_grad, cs);
@@ -652,7 +662,7 @@ fn_status fn_vmc_iteration(fn_system_t s, const fn_train_config* c, void* d_para
     using Mode = decltype(m);
     const Shape value = make_shape(s, B, 1);
     const Shape full = make_shape(s, B, 3 * s->N + 2);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, true, cs);
     // log|psi| of the persistent walkers under the current parameters
     launch_forward<Mode>(s, d_walkers, value, false, cs);
     launch_det_energy<Mode>(s, d_walkers, value, nullptr, d_log_psi, nullptr, false, cs);
@@ -704,7 +714,7 @@ fn_status fn_pretrain_grad(fn_system_t s, const void* d_params, const void* d_wa
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
     const Shape sh = make_shape(s, B, 1);
-    launch_prep_params<Mode>(s, d_params, cs);
+    launch_prep_params<Mode>(s, d_params, false, cs);
     launch_forward<Mode>(s, d_walkers, sh, true, cs);
     launch_pretrain_seed<Mode>(s, d_walkers, sh, d_loss, cs);
     launch_backward<Mode>(s, d_walkers, sh, s->ws.scratch_d, d_grad, cs);

@@ -18,6 +18,7 @@
 #include "fn_device.cuh"
 #include "fn_internal.cuh"
 #include "fn_simt_launch.cuh"
+#include "fn_x3.cuh"
 
 namespace fn {
 
@@ -127,14 +128,33 @@ fn_status upload_prep_descs(fn_system* s) {
   return FN_OK;
 }
 
+// FP32 local-energy passes run their contractions on the tensor cores (fn_x3.cu) when the width
+// fills its 128-column tiles; the value passes stay on the FMA pipe, where their few rows per
+// launch take less time than the preparation of the split weights would add to every call.
+template <class Mode> static bool use_x3(const fn_system* s, bool full) {
+  return Mode::kMode == FN_FP32 && full && s->prep.total3 > 0;
+}
+
 template <class Mode>
-void launch_prep_params(const fn_system* s, const void* params, cudaStream_t st) {
+void launch_prep_params(const fn_system* s, const void* params, bool full, cudaStream_t st) {
   using Par = typename Mode::Par; using Cmp = typename Mode::Cmp;
   dim3 grid(32, s->n_descs);
   ProfScope ps(s->prof, kProfPrep, st);
   k_prep<Par, Cmp><<<grid, 256, 0, st>>>((const Par*)params, (const CopyDesc*)s->d_descs, s->n_descs,
                                          (Cmp*)s->ws.prep,
                                          (__nv_bfloat16*)s->ws.prep16);
+  if (!use_x3<Mode>(s, full)) return;
+  x3::SplitList list{};
+  const int L = s->cfg.n_layers, h1 = s->cfg.h1, K = s->cfg.n_dets, ns[2] = {s->n_up, s->n_dn};
+  for (int l = 0; l < L; ++l) {
+    const LayerDims& d = s->layer[l];
+    const int64_t f_in = 3 * d.d_h + 2 * d.d_g;
+    list.e[list.n++] = {d.off_V, d.off_V + 3 * d.d_h, f_in, s->prep.V3[l], d.d_h, d.k_self, (int)round_up(d.k_self, 64), h1};
+    list.e[list.n++] = {d.off_V + d.d_h, 0, f_in, s->prep.U3[l], 2 * d.d_h, 2 * d.d_h, (int)round_up(2 * d.d_h, 64), h1};
+  }
+  for (int a = 0; a < 2; ++a)
+    if (ns[a]) list.e[list.n++] = {s->off_w[a], 0, h1, s->prep.W3[a], h1, h1, h1, K * ns[a]};
+  x3::launch_split_weights((const float*)params, list, s->ws.prep3, st);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -374,6 +394,16 @@ __global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Sh
     const int warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int col = 2 * lane, half0 = col < dg ? 0 : 1, half1 = col + 1 < dg ? 0 : 1;
     const int c0 = col - half0 * dg, c1 = col + 1 - half1 * dg;
+    // the pair of columns is one store where it starts at an even element (an odd h1 shifts it)
+    const bool even = (a.col0[l] & 1) == 0;
+    auto put2 = [&](Act* p, Cmp v0, Cmp v1) {
+      if (even) {
+        st2(p, v0, v1);
+      } else {
+        st(p, v0);
+        st(p + 1, v1);
+      }
+    };
     // d/dr_j slabs (j != i): -d g_ij / d r_i / n_spin(j) in j's spin half, 0 in the other
     for (int pp = warp; pp < n_i * sh.N; pp += n_warps) {
       const int e_i = pp / sh.N, jj = pp - e_i * sh.N;
@@ -385,8 +415,7 @@ __global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Sh
       for (int axis = 0; axis < 3; ++axis) {
         const Cmp* src = gs + (pp * 5 + 2 + axis) * 33;
         const Cmp v0 = half0 == sjj ? src[c0] * scale : (Cmp)0, v1 = half1 == sjj ? src[c1] * scale : (Cmp)0;
-        st2(Xc + (1 + 3 * jj + axis) * slab + row + col, v0, v1);
-        if (SplitValue<Act>::value) st2_lo(Xc + (sh.T + 1 + 3 * jj + axis) * slab + row + col, v0, v1);
+        put2(Xc + (1 + 3 * jj + axis) * slab + row + col, v0, v1);
       }
     }
     // value, Laplacian and d/dr_i rows: spin means over partners
@@ -401,8 +430,7 @@ __global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Sh
       const int t = qq == 0 ? 0 : (qq == 1 ? sh.T - 1 : 1 + 3 * ie + (qq - 2));
       const Cmp m0 = half0 ? dn0 * id : up0 * iu, m1 = half1 ? dn1 * id : up1 * iu;
       const int64_t o = tile_row(w, ie, sh.N, sh.wpt) * ldx + col;
-      st2(Xc + t * slab + o, m0, m1);
-      if (SplitValue<Act>::value) st2_lo(Xc + (sh.T + t) * slab + o, m0, m1);
+      put2(Xc + t * slab + o, m0, m1);
     }
     if (l == a.L - 1) break;
     __syncthreads();
@@ -544,6 +572,33 @@ __global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* __restrict__ Y,
     const int64_t off = ((int64_t)t * sh.B + w) * 2 * h1 + s2 * h1 + 8 * c8;
     *(uint4*)(Hbar + off) = o;
     *(uint4*)(Hbar + (int64_t)sh.T * sh.B * 2 * h1 + off) = ol;
+  }
+}
+
+// The same in FP32 (after the FP32 tensor-core layer): one thread per (slab, walker, spin, 4 columns).
+__global__ void k_spin_means_f32(Shape sh, const float* __restrict__ Y, int ldy, int h1, float* __restrict__ Hbar) {
+  const int g4 = h1 >> 2;
+  const int64_t n = (int64_t)sh.T * sh.B * 2 * g4;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int c4 = (int)(e % g4);
+    const int64_t rest = e / g4;
+    const int s2 = (int)(rest & 1);
+    const int64_t tw = rest >> 1;
+    const int w = (int)(tw % sh.B), t = (int)(tw / sh.B);
+    const int lo = s2 ? sh.n_up : 0, hi = s2 ? sh.N : sh.n_up;
+    const float* base = Y + ((int64_t)t * sh.R + tile_row(w, 0, sh.N, sh.wpt)) * ldy + 4 * c4;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i0 = lo; i0 < hi; i0 += 4) {
+      float4 u[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        u[k] = i0 + k < hi ? __ldg((const float4*)(base + (int64_t)(i0 + k) * ldy)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { acc.x += u[k].x; acc.y += u[k].y; acc.z += u[k].z; acc.w += u[k].w; }
+    }
+    const float d = (float)(hi - lo);
+    if (hi > lo) acc = make_float4(acc.x / d, acc.y / d, acc.z / d, acc.w / d);
+    *(float4*)(Hbar + ((int64_t)t * sh.B + w) * 2 * h1 + s2 * h1 + 4 * c4) = acc;
   }
 }
 
@@ -1069,6 +1124,9 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
       }
     }
   }
+  const bool x3 = use_x3<Mode>(s, full);
+  const __nv_bfloat16* prep3 = (const __nv_bfloat16*)ws.prep3;
+  bool ok = true;
   for (int l = 0; l < L; ++l) {
     const LayerDims& d = s->layer[l];
     // mean-field term M = Hbar_l U_l^T + b_l (bias on the value slab only)
@@ -1081,6 +1139,10 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         if (!launch_gemm_tc(sh.T * sh.B, 2 * d.d_h, Hb, 2 * d.d_h, U16, 4 * d.d_h, 2 * d.d_h, h1, (float*)ws.Mterm, h1,
                             (const float*)(prep + s->prep.b[l]), sh.B, 1, false, ws.status, st, sh.T * sh.B))
           const_cast<fn_system*>(s)->host_error = FN_ERR_CUDA;
+      } else if (x3) {
+        ok = x3::launch_gemm((int64_t)sh.T * sh.B, 2 * d.d_h, (const float*)Hb, 2 * d.d_h, prep3 + s->prep.U3[l],
+                             (int)round_up(2 * d.d_h, 64), h1, (float*)ws.Mterm, (const float*)(prep + s->prep.b[l]), sh.B,
+                             ws.status, s->sm_count, st) && ok;
       } else {
         simt::launch_gemm<Cmp>({(int64_t)sh.T * sh.B, h1, 2 * d.d_h, (const Cmp*)ws.Hbar[l], 2 * d.d_h,
                                 prep + s->prep.UT[l], h1, (Cmp*)ws.Mterm, h1, prep + s->prep.b[l], sh.B, 0},
@@ -1110,6 +1172,18 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)s->sm_count * 64);
         k_spin_means_bf16<<<blocks, 256, 0, st>>>(sh, (const __nv_bfloat16*)la.Y, la.ldy, h1,
                                                   (__nv_bfloat16*)la.Hbar_out);
+      }
+      continue;
+    }
+    if (x3) {
+      ok = x3::launch_layer(sh, (const float*)la.X, la.ldx, la.k_self, prep3 + s->prep.V3[l],
+                            (int)round_up(la.k_self, 64), (const float*)la.Mterm, (float*)la.Y, la.ldy, la.residual, h1,
+                            ws.status, s->sm_count, st) && ok;
+      if (!last) {
+        ProfScope pm(s->prof, kProfSpinMeans, st);
+        const int64_t n = (int64_t)sh.T * sh.B * 2 * (h1 / 4);
+        const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)s->sm_count * 64);
+        k_spin_means_f32<<<blocks, 256, 0, st>>>(sh, (const float*)la.Y, la.ldy, h1, (float*)la.Hbar_out);
       }
       continue;
     }
@@ -1153,10 +1227,19 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
                               (float*)ws.orbP, (const float*)ws.envv, ws.status, st))
         const_cast<fn_system*>(s)->host_error = FN_ERR_CUDA;
       }
+    } else if (x3) {
+      ProfScope ps(s->prof, kProfOrbFull, st);
+      simt::launch_envelope<float>(sh, oa, st);
+      for (int a = 0; a < 2; ++a)
+        if (a ? s->n_dn : s->n_up)
+          ok = x3::launch_orbitals(sh, a, (const float*)ws.HL, h1, prep3 + s->prep.W3[a], h1,
+                                   (const float*)(prep + s->prep.g[a]), oa.K, (float*)ws.Phi, oa.PW, (const float*)ws.envv,
+                                   (float*)ws.orbP, ws.status, s->sm_count, st) && ok;
     } else {
       ProfScope ps(s->prof, full ? kProfOrbFull : kProfOrbValue, st);
       simt::launch_orbitals<Cmp>(sh, oa, s->sm_count, st);
     }
+    if (!ok) const_cast<fn_system*>(s)->host_error = FN_ERR_CUDA;
     if (full) {
       const int ko_max = s->cfg.n_dets * std::max(s->n_up, s->n_dn);
       ProfScope ps(s->prof, kProfOrbFix, st);
@@ -1166,9 +1249,9 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
   }
 }
 
-template void launch_prep_params<ModeF64>(const fn_system*, const void*, cudaStream_t);
-template void launch_prep_params<ModeF32>(const fn_system*, const void*, cudaStream_t);
-template void launch_prep_params<ModeBF16>(const fn_system*, const void*, cudaStream_t);
+template void launch_prep_params<ModeF64>(const fn_system*, const void*, bool, cudaStream_t);
+template void launch_prep_params<ModeF32>(const fn_system*, const void*, bool, cudaStream_t);
+template void launch_prep_params<ModeBF16>(const fn_system*, const void*, bool, cudaStream_t);
 template void launch_forward<ModeF64>(const fn_system*, const void*, const Shape&, bool, cudaStream_t);
 template void launch_forward<ModeF32>(const fn_system*, const void*, const Shape&, bool, cudaStream_t);
 template void launch_forward<ModeBF16>(const fn_system*, const void*, const Shape&, bool, cudaStream_t);

@@ -162,6 +162,10 @@ struct PrepLayout {
   int64_t W16T;              // orbital projections transposed: rows h1, ld = ldWT (dh_L = dP W)
   int ldWT;                  // K (n_up + n_dn) rounded up to 64 (the hi part of a k-block never reaches the lo part)
   int64_t total16;
+  // FP32 mode with h1 a multiple of 128: three-part BF16 weights of the local-energy pass
+  // (fn_x3.cu), [rows][3][ld] with ld = the contraction length rounded up to 64
+  int64_t V3[kMaxLayers], U3[kMaxLayers], W3[2];
+  int64_t total3;
 };
 
 // One strided copy of the parameter preparation: blob -> internal layout.
@@ -185,6 +189,7 @@ struct Workspace {
   void* Phi = nullptr;           // [B][per-walker orbital block] (PhiT)
   void* prep = nullptr;          // prepared params (Cmp)
   void* prep16 = nullptr;        // bf16 weights
+  void* prep3 = nullptr;         // three-part bf16 weights (FP32 mode)
   void* walk2 = nullptr;         // proposal walkers [B][N][3] (Wlk)
   double* lp2 = nullptr;         // proposal log|psi| [B]
   double* scratch_d = nullptr;   // [B] doubles (per-walker weights etc.)
@@ -201,7 +206,7 @@ struct Workspace {
   void* gradc = nullptr;         // prepared-layout gradient accumulator (Cmp)
   void* dP = nullptr;            // [R][K (n_up + n_dn)] gradient wrt orbital projections (Cmp)
   void* orbP = nullptr;          // [R][4][K N] projections for the orbital envelope fix-up (Cmp)
-  void* envv = nullptr;          // [R][K N] envelope values (Cmp)
+  void* envv = nullptr;          // envelope values (Cmp): BF16 mode [R][K N], else [K N][R]
   // BF16-mode backward operands for the tensor-core GEMMs
   void* g16 = nullptr;           // [R][max(h1, ldWT)] bf16 copy of dZ or dP
   void* t16a = nullptr;          // [max(k_self, h1)][R] bf16 transposed activations (X_l^T, h_L^T)
@@ -267,7 +272,8 @@ Shape make_shape(const fn_system* s, int B, int T);
 int64_t phi_walker_stride(const fn_system* s, int T);   // elements per walker of Phi
 
 // ---- launchers (one instantiation per precision mode) --------------------------------
-template <class Mode> void launch_prep_params(const fn_system* s, const void* params, cudaStream_t st);
+// full: a local-energy pass follows (its FP32 tensor-core weights are prepared too)
+template <class Mode> void launch_prep_params(const fn_system* s, const void* params, bool full, cudaStream_t st);
 template <class Mode> void launch_forward(const fn_system* s, const void* walkers, const Shape& sh,
                                           bool keep_for_backward, cudaStream_t st);
 template <class Mode> void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,

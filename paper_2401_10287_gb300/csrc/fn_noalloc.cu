@@ -121,7 +121,7 @@ static fn_status log_psi_noalloc(fn_system* s, const void* params, const void* w
   s->ws = arena;
   s->prof = nullptr;
   const Shape sh = make_shape(s, B, 1);
-  launch_prep_params<Mode>(s, params, st);
+  launch_prep_params<Mode>(s, params, false, st);
   launch_forward<Mode>(s, walkers, sh, false, st);
   launch_det_energy<Mode>(s, walkers, sh, nullptr, log_psi, sign, false, st);
   s->ws = saved;

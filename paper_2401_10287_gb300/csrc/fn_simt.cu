@@ -40,7 +40,7 @@ __device__ __forceinline__ void store_group(T* p, int live, const T (&v)[Vec<T>:
 // ring keeps loading across slabs, the spin means of the output are summed in electron
 // order from a staged copy.
 // Bound by the FMA pipe: N2 network at 4096 walkers, 104 -> 35 ms per FP32 local-energy
-// call for its four layers (1.26 TFLOP).
+// call for its four layers (1.26 TFLOP); that width now takes the tensor cores (fn_x3.cu).
 // ---------------------------------------------------------------------------------------
 template <typename T, int TM, int TN, int WM, bool FULL, bool VEC>
 __global__ void __launch_bounds__(32 * WM) k_layer(Shape sh, LayerArgs a, int wps, int subs) {
@@ -186,10 +186,12 @@ void launch_layer(const Shape& sh, const LayerArgs& a, int sm_count, cudaStream_
 // per slab), and the own-coordinate and Laplacian envelope terms are added afterwards from
 // the projections kept in orbP (k_orbital_fixup).
 // ---------------------------------------------------------------------------------------
-template <typename T> __device__ __forceinline__ T env_value(const T* pi, const T* sig, int aniso, int M, const T* d) {
+// sum_m pi_m exp(-|sigma_m d_m|); d[q * ld] = coordinate q mod 3 of the distance to nucleus q / 3
+template <typename T>
+__device__ __forceinline__ T env_value(const T* pi, const T* sig, int aniso, int M, const T* d, int ld) {
   T env = 0;
   for (int m = 0; m < M; ++m) {
-    const T d0 = d[3 * m], d1 = d[3 * m + 1], d2 = d[3 * m + 2];
+    const T d0 = d[3 * m * ld], d1 = d[(3 * m + 1) * ld], d2 = d[(3 * m + 2) * ld];
     T s;
     if (!aniso) {
       s = sig[m] * f_sqrt(d0 * d0 + d1 * d1 + d2 * d2);
@@ -204,19 +206,24 @@ template <typename T> __device__ __forceinline__ T env_value(const T* pi, const 
   return env;
 }
 
-// Envelope values of every electron's own-spin orbitals: a CTA per electron, thread per orbital.
+// Envelope values of every electron's own-spin orbitals, orbital-major [K N][R]: the rows of an
+// orbital are adjacent, so that a kernel with one electron row per lane reads whole lines.  A CTA
+// takes one 128-row tile (thread = row) and 16 orbitals, whose parameters every thread of a spin
+// reads at the same time.
+constexpr int kEnvOrbs = 16;
 template <typename T>
-__global__ void k_envelope(Shape sh, OrbArgs a) {
-  __shared__ T ds[3 * kMaxNuclei];
-  const int w = blockIdx.x / sh.N, j = blockIdx.x % sh.N, spin = j < sh.n_up ? 0 : 1;
+__global__ void __launch_bounds__(kTileRows) k_envelope(Shape sh, OrbArgs a) {
+  __shared__ T ds[3 * kMaxNuclei][kTileRows];
+  const int tile = blockIdx.x, rl = threadIdx.x, wl = rl / sh.N, j = rl - wl * sh.N, w = tile * sh.wpt + wl;
+  if (wl >= sh.wpt || w >= sh.B) return;                        // no barrier below: each thread reads its own column
   const T* rj = (const T*)a.walkers + ((int64_t)w * sh.N + j) * 3;
-  if ((int)threadIdx.x < 3 * sh.M) ds[threadIdx.x] = (T)((double)rj[threadIdx.x % 3] - a.nuclei[threadIdx.x]);
-  __syncthreads();
-  const int n_ko = a.K * (spin ? sh.n_dn : sh.n_up), nc = a.aniso ? 9 : 1;
-  T* out = (T*)a.envv + tile_row(w, j, sh.N, sh.wpt) * a.K * sh.N + (spin ? a.K * sh.n_up : 0);
-  for (int ko = threadIdx.x; ko < n_ko; ko += blockDim.x)
-    out[ko] = env_value<T>((const T*)a.pi[spin] + (int64_t)ko * sh.M, (const T*)a.sig[spin] + (int64_t)ko * sh.M * nc,
-                           a.aniso, sh.M, ds);
+  for (int q = 0; q < 3 * sh.M; ++q) ds[q][rl] = (T)((double)rj[q % 3] - a.nuclei[q]);
+  const int spin = j < sh.n_up ? 0 : 1, n_ko = a.K * (spin ? sh.n_dn : sh.n_up), nc = a.aniso ? 9 : 1;
+  T* out = (T*)a.envv + (int64_t)(spin ? a.K * sh.n_up : 0) * sh.R + (int64_t)tile * kTileRows + rl;
+  for (int ko = blockIdx.y * kEnvOrbs; ko < min(n_ko, (int)(blockIdx.y + 1) * kEnvOrbs); ++ko)
+    out[(int64_t)ko * sh.R] = env_value<T>((const T*)a.pi[spin] + (int64_t)ko * sh.M,
+                                           (const T*)a.sig[spin] + (int64_t)ko * sh.M * nc, a.aniso, sh.M, &ds[0][rl],
+                                           kTileRows);
 }
 
 template <typename T, int TM, int TN, int WM, bool FULL, bool VEC>
@@ -263,13 +270,13 @@ __global__ void __launch_bounds__(32 * WM) k_orbitals(Shape sh, OrbArgs a, int s
           if (t == 0) p += ((const T*)a.g[spin])[ko + e];
           T env;
           if constexpr (FULL) {
-            env = ((const T*)a.envv)[row * ldp + poff + ko + e];
+            env = ((const T*)a.envv)[(int64_t)(poff + ko + e) * sh.R + row];
             if (slot >= 0 && t < sh.T - 1) ((T*)a.orbP)[(row * 4 + slot) * ldp + poff + ko + e] = p;
           } else {
             const int nc = a.aniso ? 9 : 1;
             env = env_value<T>((const T*)a.pi[spin] + (int64_t)(ko + e) * sh.M,
                                (const T*)a.sig[spin] + (int64_t)(ko + e) * sh.M * nc, a.aniso, sh.M,
-                               ds + rl * 3 * sh.M);
+                               ds + rl * 3 * sh.M, 1);
           }
           ys[rl * LDY + cl + e] = p * env;
         }
@@ -303,12 +310,14 @@ static void orbitals_cfg(const Shape& sh, const OrbArgs& a, int spin, cudaStream
 }
 
 template <typename T>
+void launch_envelope(const Shape& sh, const OrbArgs& a, cudaStream_t st) {
+  const int n_ko = a.K * std::max(sh.n_up, sh.n_dn);
+  k_envelope<T><<<dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st>>>(sh, a);
+}
+
+template <typename T>
 void launch_orbitals(const Shape& sh, const OrbArgs& a, int sm_count, cudaStream_t st) {
-  if (sh.T > 1) {
-    const int n_ko = a.K * std::max(sh.n_up, sh.n_dn);
-    k_envelope<T><<<(unsigned)((int64_t)sh.B * sh.N), (unsigned)std::max<int64_t>(64, std::min<int64_t>(256, round_up(n_ko, 32))), 0,
-                    st>>>(sh, a);
-  }
+  if (sh.T > 1) launch_envelope<T>(sh, a, st);
   for (int spin = 0; spin < 2; ++spin) {
     const int n_s = spin ? sh.n_dn : sh.n_up;
     if (!n_s) continue;
@@ -435,6 +444,7 @@ void launch_gemm(GemmArgs<T> g, bool at, bool bt, int max_split, int sm_count, c
 
 template void launch_layer<float>(const Shape&, const LayerArgs&, int, cudaStream_t);
 template void launch_layer<double>(const Shape&, const LayerArgs&, int, cudaStream_t);
+template void launch_envelope<float>(const Shape&, const OrbArgs&, cudaStream_t);
 template void launch_orbitals<float>(const Shape&, const OrbArgs&, int, cudaStream_t);
 template void launch_orbitals<double>(const Shape&, const OrbArgs&, int, cudaStream_t);
 template void launch_gemm<float>(GemmArgs<float>, bool, bool, int, int, cudaStream_t);

@@ -24,7 +24,7 @@ struct OrbArgs {
   int h1, K, aniso;
   const void* walkers;          // [B][N][3]
   const double* nuclei;
-  void* envv;                   // full pass: [R][K N] envelope values
+  void* envv;                   // full pass: [K N][R] envelope values
   void* orbP;                   // full pass: [R][4][K N] value and own-coordinate projections
 };
 
@@ -41,6 +41,8 @@ struct GemmArgs {
 
 // One stream layer over all slabs of sh; the tile shape is chosen from the number of CTAs.
 template <typename T> void launch_layer(const Shape& sh, const LayerArgs& a, int sm_count, cudaStream_t st);
+// Envelope values of every electron's own-spin orbitals into a.envv.
+template <typename T> void launch_envelope(const Shape& sh, const OrbArgs& a, cudaStream_t st);
 // Orbital matrices of every slab; in the full pass without the envelope-derivative terms
 // (which k_orbital_fixup adds from orbP).
 template <typename T> void launch_orbitals(const Shape& sh, const OrbArgs& a, int sm_count, cudaStream_t st);
