@@ -14,13 +14,14 @@
 //                  BF16 MMAs over all pairs of a walker)
 // In BF16 mode the large GEMMs run on the tensor cores (fn_layer_tc.cu): row-major
 // products directly, weight gradients as split-K products over the electron rows on
-// transposed BF16 copies.  Parameter gradients accumulate in the internal layout and
+// transposed BF16 copies; FP32 and FP64 take the register-tiled GEMM (fn_simt.cu).  Parameter gradients accumulate in the internal layout and
 // are scattered back to the blob order at the end.
 #include <algorithm>
 
 #include "fn_device.cuh"
 #include "fn_gemm.cuh"
 #include "fn_internal.cuh"
+#include "fn_simt_launch.cuh"
 
 namespace fn {
 
@@ -541,7 +542,7 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
   const Wlk* r = (const Wlk*)walkers;
   const int64_t R = sh.R;
   const int ldp = K * N;
-  const int split = (int)std::max<int64_t>(1, std::min<int64_t>(64, R / 1024));
+  constexpr int kAnySplit = 1 << 20;             // weight gradients: as many K splits as fill the chip
   cudaMemsetAsync(gradc, 0, sizeof(Cmp) * pl.total, st);
   cudaMemsetAsync(ws.dH, 0, sizeof(Cmp) * R * h1, st);
   // orbitals + envelopes: P = h_L w (both spins, every row), then the envelope kernel turns
@@ -557,8 +558,9 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       for (int q = 0; q < 2; ++q) {
         const int n_q = q ? s->n_dn : s->n_up;
         if (!n_q) continue;
-        gemm<Act, Cmp, Cmp, Cmp>(st, (int)R, K * n_q, h1, (const Act*)ws.HL, h1, 1, prep + pl.wT[q], K * n_q, 1,
-                                 (Cmp*)ws.dP + (q ? K * s->n_up : 0), ldp, 1, (const Cmp*)nullptr, 0, 1, false);
+        simt::launch_gemm<Cmp>({R, K * n_q, h1, (const Cmp*)ws.HL, h1, prep + pl.wT[q], K * n_q,
+                                (Cmp*)ws.dP + (q ? K * s->n_up : 0), ldp, nullptr, 0, 0},
+                               false, false, 1, s->sm_count, st);
       }
     }
   }
@@ -623,15 +625,15 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
     // dW_orb^T [h1][K n]: sum over rows of h_L[row][c] dP[row][ko]
     {
       ProfScope ps(s->prof, kProfBwdGemm, st);
-      gemm<Act, Cmp, Cmp, Cmp>(st, h1, n_ko, (int)R, (const Act*)ws.HL, 1, h1, dPq, ldp, 1, gradc + pl.wT[q], n_ko, 1,
-                               (const Cmp*)nullptr, 0, split, true);
+      simt::launch_gemm<Cmp>({h1, n_ko, (int)R, (const Cmp*)ws.HL, h1, dPq, ldp, gradc + pl.wT[q], n_ko, nullptr, 0, 1},
+                             true, false, kAnySplit, s->sm_count, st);
     }
     colsum<Cmp, Cmp>(s, st, dPq, R, ldp, n_ko, gradc + pl.g[q]);
     // dh_L[row][c] += sum_ko dP[row][ko] w[ko][c]
     {
       ProfScope ps(s->prof, kProfBwdGemm, st);
-      gemm<Cmp, Cmp, Cmp, Cmp>(st, (int)R, h1, n_ko, dPq, ldp, 1, prep + pl.wT[q], 1, n_ko, (Cmp*)ws.dH, h1, 1,
-                               (const Cmp*)nullptr, 0, 1, true);
+      simt::launch_gemm<Cmp>({R, h1, n_ko, dPq, ldp, prep + pl.wT[q], n_ko, (Cmp*)ws.dH, h1, nullptr, 0, 1}, false, true,
+                             1, s->sm_count, st);
     }
   }
   Cmp* dH = (Cmp*)ws.dH;
@@ -660,16 +662,20 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
         tc_or_flag(s, launch_gemm_tc(d.k_self, (int)R, t16a, (int)R, t16b, (int)R, 0, h1, (float*)(gradc + pl.VsT[l]),
                                      h1, nullptr, 0, ksplit_for(s, d.k_self, h1, R), true, ws.status, st));
       else
-        gemm<Act, Cmp, Cmp, Cmp>(st, d.k_self, h1, (int)R, X, 1, d.ldx, dZ, h1, 1, gradc + pl.VsT[l], h1, 1,
-                                 (const Cmp*)nullptr, 0, split, true);
+        simt::launch_gemm<Cmp>({d.k_self, h1, (int)R, (const Cmp*)ws.X[l], d.ldx, dZ, h1, gradc + pl.VsT[l], h1, nullptr, 0,
+                                1}, true, false, kAnySplit, s->sm_count, st);
     }
     colsum<Cmp, Cmp>(s, st, dZw, sh.B, h1, h1, gradc + pl.b[l]);
     // dU (internal [2 d_h][h1]) += Hbar^T dZw
     const int splitB = (int)std::max(1, std::min(32, sh.B / 256));
     {
       ProfScope ps(s->prof, kProfBwdGemm, st);
-      gemm<Act, Cmp, Cmp, Cmp>(st, 2 * d.d_h, h1, sh.B, (const Act*)ws.Hbar[l], 1, 2 * d.d_h, dZw, h1, 1,
-                               gradc + pl.UT[l], h1, 1, (const Cmp*)nullptr, 0, splitB, true);
+      if constexpr (kTc)
+        gemm<Act, Cmp, Cmp, Cmp>(st, 2 * d.d_h, h1, sh.B, (const Act*)ws.Hbar[l], 1, 2 * d.d_h, dZw, h1, 1,
+                                 gradc + pl.UT[l], h1, 1, (const Cmp*)nullptr, 0, splitB, true);
+      else
+        simt::launch_gemm<Cmp>({2 * d.d_h, h1, sh.B, (const Cmp*)ws.Hbar[l], 2 * d.d_h, dZw, h1, gradc + pl.UT[l], h1,
+                                nullptr, 0, 1}, true, false, kAnySplit, s->sm_count, st);
     }
     // dX = dZ V_self^T  ([R][k_self], row stride ldx)
     {
@@ -678,14 +684,14 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
         tc_or_flag(s, launch_gemm_tc((int)R, h1, g16, h1, prep16 + pl.VsT16[l], 2 * h1, h1, d.k_self, (float*)dX, d.ldx,
                                      nullptr, 0, 1, false, ws.status, st));
       else
-        gemm<Cmp, Cmp, Cmp, Cmp>(st, (int)R, d.k_self, h1, dZ, h1, 1, prep + pl.VsT[l], 1, h1, dX, d.ldx, 1,
-                                 (const Cmp*)nullptr, 0, 1, false);
+        simt::launch_gemm<Cmp>({R, d.k_self, h1, dZ, h1, prep + pl.VsT[l], h1, dX, d.ldx, nullptr, 0, 0}, false, true, 1,
+                               s->sm_count, st);
     }
     if (l >= 1) {
       {
         ProfScope ps(s->prof, kProfBwdGemm, st);
-        gemm<Cmp, Cmp, Cmp, Cmp>(st, sh.B, 2 * d.d_h, h1, dZw, h1, 1, prep + pl.UT[l], 1, h1, dHbar, 2 * d.d_h, 1,
-                                 (const Cmp*)nullptr, 0, 1, false);
+        simt::launch_gemm<Cmp>({sh.B, 2 * d.d_h, h1, dZw, h1, prep + pl.UT[l], h1, dHbar, 2 * d.d_h, nullptr, 0, 0}, false,
+                               true, 1, s->sm_count, st);
       }
       const int64_t n = (int64_t)sh.B * N * h1;
       ProfScope ps(s->prof, kProfBwdMisc, st);
