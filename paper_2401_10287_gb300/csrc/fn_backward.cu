@@ -19,7 +19,6 @@
 #include <algorithm>
 
 #include "fn_device.cuh"
-#include "fn_gemm.cuh"
 #include "fn_internal.cuh"
 #include "fn_simt_launch.cuh"
 
@@ -58,14 +57,25 @@ __global__ void k_colsum(const T* __restrict__ src, int64_t rows, int64_t lds, i
   const int64_t chunk = (rows + gridDim.y - 1) / gridDim.y;
   const int64_t r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
   Cmp acc = 0;
-  for (int64_t r = r0; r < r1; ++r) acc += (Cmp)ld(src + r * lds + c);
-  atomicAdd(dst + c, acc);
+  int64_t r = r0;
+  for (; r + 8 <= r1; r += 8) {                   // eight loads in flight
+    Cmp v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = (Cmp)ld(src + (r + u) * lds + c);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc += v[u];
+  }
+  for (; r < r1; ++r) acc += (Cmp)ld(src + r * lds + c);
+  if (r1 > r0) atomicAdd(dst + c, acc);
 }
 
 template <typename T, typename Cmp>
 static void colsum(const fn_system* s, cudaStream_t st, const T* src, int64_t rows, int64_t ld, int cols, Cmp* dst) {
   ProfScope ps(s->prof, kProfBwdMisc, st);
-  dim3 grid((cols + 127) / 128, (unsigned)std::min<int64_t>(64, std::max<int64_t>(1, rows / 256)));
+  // about four CTAs per SM, at least 16 rows each: 64 CTAs of 900 rows took 84 us for the
+  // 58368 x 112 orbital gradients (26 MB), bound by one load in flight per thread
+  const int64_t want = std::max<int64_t>(1, 4 * s->sm_count / ((cols + 127) / 128));
+  dim3 grid((cols + 127) / 128, (unsigned)std::min<int64_t>(want, std::max<int64_t>(1, rows / 16)));
   k_colsum<T, Cmp><<<grid, 128, 0, st>>>(src, rows, ld, cols, dst);
 }
 
@@ -96,6 +106,43 @@ __global__ void k_bf16_copy_T(Shape sh, const Tin* __restrict__ in, int64_t ld_i
     const int c = c0 + k;
     if (c < cols) outT[(int64_t)c * sh.R + r0 + tx] = __float2bfloat16_rn(tile[tx][k]);
   }
+}
+
+// The transposed copy alone of a BF16 matrix, in 64 x 64 tiles: 16-byte loads of 8 columns and
+// 16-byte stores of 8 rows (the 2-byte accesses of the kernel above take 51 us for the 58368 x 320
+// input of an N2 layer at 4096 walkers, 75 MB in all).
+__global__ void __launch_bounds__(256) k_bf16_T(Shape sh, const __nv_bfloat16* __restrict__ in, int64_t ld_in, int cols,
+                                                __nv_bfloat16* __restrict__ outT) {
+  __shared__ unsigned short tile[64][66];
+  const int c0 = blockIdx.x * 64, tid = threadIdx.x;
+  const int64_t r0 = (int64_t)blockIdx.y * 64;
+#pragma unroll
+  for (int e = tid; e < 512; e += 256) {
+    const int k = e >> 3, c = c0 + 8 * (e & 7);
+    const int64_t r = r0 + k;
+    const int rr = (int)(r % kTileRows), q = (int)(r / kTileRows), wl = rr / sh.N;
+    const bool valid = wl < sh.wpt && q * sh.wpt + wl < sh.B && c < cols;
+    const uint4 v = valid ? __ldg((const uint4*)(in + r * ld_in + c)) : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) *(uint32_t*)&tile[k][8 * (e & 7) + 2 * m] = u[m];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = tid; e < 512; e += 256) {
+    const int c = e & 63, k = 8 * (e >> 6);
+    if (c0 + c >= cols) continue;
+    uint32_t u[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) u[m] = (uint32_t)tile[k + 2 * m][c] | ((uint32_t)tile[k + 2 * m + 1][c] << 16);
+    *(uint4*)(outT + (int64_t)(c0 + c) * sh.R + r0 + k) = make_uint4(u[0], u[1], u[2], u[3]);
+  }
+}
+
+static void bf16_T(const fn_system* s, cudaStream_t st, const Shape& sh, const void* in, int64_t ld_in, int cols,
+                   __nv_bfloat16* outT) {
+  ProfScope ps(s->prof, kProfBwdMisc, st);
+  k_bf16_T<<<dim3((cols + 63) / 64, (unsigned)(sh.R / 64)), 256, 0, st>>>(sh, (const __nv_bfloat16*)in, ld_in, cols, outT);
 }
 
 template <typename Tin>
@@ -160,22 +207,46 @@ __global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ 
   const int ldp = a.K * sh.N, poff = spin ? a.K * sh.n_up : 0, poff_o = spin ? 0 : a.K * sh.n_up;
   const int w0 = blockIdx.x * a.chunk, w1 = min(sh.B, w0 + a.chunk);
   Cmp* dP = (Cmp*)a.dP;
+  const Cmp gk = active ? ((const Cmp*)a.g[spin])[ko] : (Cmp)0;
+  // The electron-nucleus distances of a walker are formed once per CTA in shared memory: as FP64
+  // differences in every thread they took most of the kernel's 327 us (FP64 operations and
+  // conversions run at 1/64 of the FP32 rate).  Four electrons' projections and determinant
+  // gradients are loaded together.
+  __shared__ Cmp dist[kMaxSpin * 3 * MM];
   for (int w = w0; w < w1; ++w) {
     const Cmp cw = (Cmp)a.cw[w];
-    for (int jj = 0; jj < n; ++jj) {
-      const int j = jj + (spin ? sh.n_up : 0);
-      const int64_t row = tile_row(w, j, sh.N, sh.wpt);
+    const int j0 = spin ? sh.n_up : 0;
+    const int64_t row0 = tile_row(w, j0, sh.N, sh.wpt);         // a walker's rows are consecutive
+    __syncthreads();
+    for (int e = threadIdx.x; e < n * 3 * sh.M; e += blockDim.x) {
+      const int jj = e / (3 * sh.M), q = e - jj * 3 * sh.M;
+      dist[jj * 3 * MM + q] = (Cmp)((double)r[((int64_t)w * sh.N + j0 + jj) * 3 + q % 3] - nuc[q]);
+    }
+    __syncthreads();
+    const Det* seed = (const Det*)a.dPhi + (int64_t)w * PW1 + inv_off + (int64_t)k * n * n + i * n;
+    for (int jq = 0; jq < n; jq += 4) {
+    Cmp Pv[4], sd[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool in = active && jq + u < n;
+      Pv[u] = in ? dP[(row0 + jq + u) * ldp + poff + ko] : (Cmp)0;
+      sd[u] = in ? (Cmp)seed[jq + u] : (Cmp)0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int jj = jq + u;
+      if (jj >= n) break;
+      const int64_t row = row0 + jj;
       if (ko < a.K * n_o) dP[row * ldp + poff_o + ko] = (Cmp)0;
       if (!active) continue;
-      const Cmp P = dP[row * ldp + poff + ko] + ((const Cmp*)a.g[spin])[ko];
-      const Wlk* rj = r + ((int64_t)w * sh.N + j) * 3;
+      const Cmp P = Pv[u] + gk;
       Cmp dv[MM][3], sv[MM], em[MM];
       Cmp env = 0;
 #pragma unroll
       for (int m = 0; m < MM; ++m) {
         if (m >= sh.M) break;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) dv[m][c] = (Cmp)((double)rj[c] - nuc[3 * m + c]);
+        for (int c = 0; c < 3; ++c) dv[m][c] = dist[jj * 3 * MM + 3 * m + c];
         if (!a.aniso) {
           sv[m] = S[m][0] * f_sqrt(dv[m][0] * dv[m][0] + dv[m][1] * dv[m][1] + dv[m][2] * dv[m][2]);
         } else {
@@ -190,7 +261,7 @@ __global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ 
         em[m] = f_exp(-sv[m]);
         env += pim[m] * em[m];
       }
-      const Cmp dphi = cw * (Cmp)((const Det*)a.dPhi)[(int64_t)w * PW1 + inv_off + (int64_t)k * n * n + i * n + jj];
+      const Cmp dphi = cw * sd[u];
       const Cmp denv = dphi * P;
       dP[row * ldp + poff + ko] = dphi * env;
 #pragma unroll
@@ -210,6 +281,7 @@ __global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ 
           }
         }
       }
+    }
     }
   }
   if (active) {
@@ -243,18 +315,75 @@ __global__ void k_bwd_tanh(Shape sh, int h1, const Cmp* __restrict__ dH, const C
   dZw[(int64_t)w * h1 + c] = sum;
 }
 
-template <typename Cmp>
+// BF16 mode: dz leaves only as the operands of the tensor-core products, row-major and transposed
+// BF16 (rows without an electron are zero), and as the walker sums.  One 128-row tile (whole
+// walkers) x 32 columns per CTA; separate tanh, copy and clear passes moved dz four times.
+__global__ void __launch_bounds__(256) k_bwd_tanh_bf16(Shape sh, int h1, const float* __restrict__ dH,
+                                                       const float* __restrict__ act, __nv_bfloat16* __restrict__ out,
+                                                       __nv_bfloat16* __restrict__ outT, float* __restrict__ dZw) {
+  __shared__ float tile[kTileRows][33];
+  const int c0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int q = blockIdx.y;
+  const int64_t r0 = (int64_t)q * kTileRows;
+  const int rows = min(sh.wpt, sh.B - q * sh.wpt) * sh.N;
+#pragma unroll 4
+  for (int k = ty; k < kTileRows; k += 8) {
+    float dz = 0.f;
+    if (k < rows) {
+      const float a = act[(r0 + k) * h1 + c0 + tx];
+      dz = dH[(r0 + k) * h1 + c0 + tx] * (1.f - a * a);
+    }
+    tile[k][tx] = dz;
+  }
+  __syncthreads();
+  // row-major: 4 lanes x 8 columns a row; transposed: 16 lanes x 8 rows a column
+#pragma unroll
+  for (int e = threadIdx.x; e < kTileRows * 4; e += 256) {
+    const int k = e >> 2, c = 8 * (e & 3);
+    __nv_bfloat162 v[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = __floats2bfloat162_rn(tile[k][c + 2 * m], tile[k][c + 2 * m + 1]);
+    *(uint4*)(out + (r0 + k) * h1 + c0 + c) = *(const uint4*)v;
+  }
+#pragma unroll
+  for (int e = threadIdx.x; e < 32 * 16; e += 256) {
+    const int c = e >> 4, k = 8 * (e & 15);
+    __nv_bfloat162 v[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = __floats2bfloat162_rn(tile[k + 2 * m][c], tile[k + 2 * m + 1][c]);
+    *(uint4*)(outT + (int64_t)(c0 + c) * sh.R + r0 + k) = *(const uint4*)v;
+  }
+  for (int wl = ty; wl * sh.N < rows; wl += 8) {
+    float sum = 0.f;
+    for (int i = 0; i < sh.N; ++i) sum += tile[wl * sh.N + i][tx];
+    dZw[(int64_t)(q * sh.wpt + wl) * h1 + c0 + tx] = sum;
+  }
+}
+
+// Four columns per thread where the width allows (the divisions and index arithmetic of one
+// element per thread took 77 us for 176 MB).
+template <typename Cmp, int V>
 __global__ void k_bwd_dh(Shape sh, int h1, int ldx, int d_h, const Cmp* __restrict__ dX,
                          const Cmp* __restrict__ dHbar, Cmp* __restrict__ dH) {
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)sh.B * sh.N * h1) return;
-  const int c = (int)(gid % h1);
-  const int64_t wi = gid / h1;
-  const int w = (int)(wi / sh.N), i = (int)(wi % sh.N);
+  const int hv = h1 / V;
+  const int64_t wi = gid / hv;
+  if (wi >= (int64_t)sh.B * sh.N) return;
+  const int c = (int)(gid - wi * hv) * V;
+  const int w = (int)(wi / sh.N), i = (int)(wi - (int64_t)w * sh.N);
   const int s = i < sh.n_up ? 0 : 1;
-  const int ns = s ? sh.n_dn : sh.n_up;
+  const Cmp ns = (Cmp)(s ? sh.n_dn : sh.n_up);
   const int64_t row = tile_row(w, i, sh.N, sh.wpt);
-  dH[row * h1 + c] = dX[row * ldx + c] + dH[row * h1 + c] + dHbar[(int64_t)w * 2 * d_h + s * d_h + c] / (Cmp)ns;
+  const Cmp* x = dX + row * ldx + c;
+  Cmp* h = dH + row * h1 + c;
+  const Cmp* b = dHbar + (int64_t)w * 2 * d_h + s * d_h + c;
+  if constexpr (V == 4) {
+    const float4 xv = *(const float4*)x, hv4 = *(const float4*)h, bv = *(const float4*)b;
+    *(float4*)h = make_float4(xv.x + hv4.x + bv.x / ns, xv.y + hv4.y + bv.y / ns, xv.z + hv4.z + bv.z / ns,
+                              xv.w + hv4.w + bv.w / ns);
+  } else {
+    *h = *x + *h + *b / ns;
+  }
 }
 
 // ---- two-electron stream, level l ----------------------------------------------------
@@ -366,7 +495,7 @@ __global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* __restrict__ r, Sha
 template <typename Wlk>
 __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r, Shape sh, PairBwdArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int w = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = lane >> 2, tig = lane & 3;
   const int N = sh.N, NP = N * N, NPp = (NP + 15) & ~15;
   const bool has_layer = a.l < a.L - 1;
@@ -374,7 +503,6 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
   __nv_bfloat16* wtl = wth + 32 * kBwdWLd;
   float* gin_s = (float*)(wtl + 32 * kBwdWLd);                   // [NPp][33] g^l, later dz W
   float* dz_s = gin_s + NPp * 33;                                // [NPp][33]
-  const float* dG = (const float*)a.dG + (int64_t)w * NP * a.h2;
   if (has_layer) {
     const float* W = (const float*)a.W;                          // [h2][d_g]
     for (int e = tid; e < 32 * 32; e += blockDim.x) {
@@ -384,7 +512,16 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
       wth[c * kBwdWLd + q] = h;
       wtl[c * kBwdWLd + q] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
+    // padding rows, and the columns beyond the widths, stay zero in dz_s; gin_s is written whole
     for (int e = tid; e < NPp * 33; e += blockDim.x) { gin_s[e] = 0.f; dz_s[e] = 0.f; }
+  }
+  // CTAs loop over walkers: the weights are staged once, and the weight gradients stay in
+  // registers until the end (one atomic per element and CTA instead of one per walker)
+  float c2[2][4] = {}, dc = 0.f;
+  const int q0 = (warp >> 1) * 16, nb0 = (warp & 1) * 2;
+  for (int w = blockIdx.x; w < sh.B; w += gridDim.x) {
+  const float* dG = (const float*)a.dG + (int64_t)w * NP * a.h2;
+  if (has_layer) {
     __syncthreads();
     const Wlk* rw = r + (int64_t)w * N * 3;
     const float* gin_g = a.g_in ? (const float*)a.g_in + (int64_t)w * NP * a.h2 : nullptr;
@@ -426,20 +563,10 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
       }
     }
     __syncthreads();
-    // dc = column sums of dz: four partial sums per column, one atomic per column
-    {
-      __shared__ float dcs[4][32];
-      const int q = tid & 31, k = tid >> 5;
-      float sum = 0.f;
-      for (int p = k; p < NP; p += 4) sum += dz_s[p * 33 + q];
-      dcs[k][q] = sum;
-      __syncthreads();
-      if (tid < a.h2) atomicAdd((float*)a.gc + tid, dcs[0][tid] + dcs[1][tid] + dcs[2][tid] + dcs[3][tid]);
-    }
+    // dc = column sums of dz: warp k sums every fourth pair of its lane's column
+    for (int p = warp; p < NP; p += 4) dc += dz_s[p * 33 + lane];
     // dW[q][c] = sum_p dz[p][q] g[p][c]: warp -> rows q0 .. q0 + 15, column blocks nb0, nb0 + 1
     {
-      const int q0 = (warp >> 1) * 16, nb0 = (warp & 1) * 2;
-      float c2[2][4] = {};
       for (int p0 = 0; p0 < NPp; p0 += 16) {
         uint32_t ah[4], al[4];
         const float* zc0 = dz_s + (p0 + 2 * tig) * 33 + q0 + grp;      // A[m = q][k = p] = dz[p][q]
@@ -459,13 +586,6 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
           mma_16816(c2[u], al, bh0, bh1);
         }
       }
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-          const int qq = q0 + grp + (q4 >= 2 ? 8 : 0), cc = 8 * (nb0 + u) + 2 * tig + (q4 & 1);
-          if (qq < a.h2 && cc < a.d_g) atomicAdd((float*)a.gW + qq * a.d_g + cc, c2[u][q4]);
-        }
     }
     __syncthreads();                                               // gin_s is overwritten below
     // dz W -> gin_s (rows = pairs)
@@ -500,7 +620,7 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
     }
     __syncthreads();
   }
-  if (a.l < 1) return;                                             // no gradient below the input features
+  if (a.l < 1) continue;                                           // no gradient below the input features
   // dG^l = (dz W) + dG^{l+1} (residual) + the spin-mean gradient of the layer input
   float* dGo = (float*)a.dG + (int64_t)w * NP * a.h2;
   for (int e = tid; e < NP * a.h2; e += blockDim.x) {
@@ -514,6 +634,26 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
       v += ((const float*)a.dX)[tile_row(w, i, N, sh.wpt) * a.ldx + a.col0 + sj * a.d_g + c] / (float)nsj;
     }
     dGo[e] = v;
+  }
+  }
+  if (!has_layer) return;
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int q4 = 0; q4 < 4; ++q4) {
+      const int qq = q0 + grp + (q4 >= 2 ? 8 : 0), cc = 8 * (nb0 + u) + 2 * tig + (q4 & 1);
+      if (qq < a.h2 && cc < a.d_g) atomicAdd((float*)a.gW + qq * a.d_g + cc, c2[u][q4]);
+    }
+  if (lane < a.h2) atomicAdd((float*)a.gc + lane, dc);
+}
+
+__global__ void k_widen_bf16(int64_t n8, const uint4* __restrict__ in, float4* __restrict__ out) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint4 v = __ldg(in + i);
+    out[2 * i] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                             __uint_as_float(v.y & 0xffff0000u));
+    out[2 * i + 1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
+                                 __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
   }
 }
 
@@ -600,7 +740,7 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
   if (kTc) {
     // dP as a bf16 row-major copy and transposed; h_L transposed
     bf16_copy_T<Cmp>(s, st, sh, (const Cmp*)ws.dP, ldp, ldp, g16, pl.ldWT, t16b);
-    bf16_copy_T<Act>(s, st, sh, (const Act*)ws.HL, h1, h1, nullptr, 0, t16a);
+    bf16_T(s, st, sh, ws.HL, h1, h1, t16a);
     for (int q = 0; q < 2; ++q) {
       if (!ns[q]) continue;
       const int n_ko = K * ns[q];
@@ -643,17 +783,18 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
   Cmp* dHbar = (Cmp*)ws.dHbar;
   for (int l = L - 1; l >= 0; --l) {
     const LayerDims& d = s->layer[l];
-    cudaMemsetAsync(dZ, 0, sizeof(Cmp) * R * h1, st);
-    {
+    if constexpr (kTc) {
+      // operands of the tensor-core products: dZ row-major and transposed, X_l transposed
+      {
+        ProfScope ps(s->prof, kProfBwdMisc, st);
+        k_bwd_tanh_bf16<<<dim3(h1 / 32, sh.tiles), 256, 0, st>>>(sh, h1, dH, (const float*)ws.act[l], g16, t16b, dZw);
+      }
+      bf16_T(s, st, sh, ws.X[l], d.ldx, d.k_self, t16a);
+    } else {
+      cudaMemsetAsync(dZ, 0, sizeof(Cmp) * R * h1, st);
       const int64_t n = (int64_t)sh.B * h1;
       ProfScope ps(s->prof, kProfBwdMisc, st);
       k_bwd_tanh<Cmp><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(sh, h1, dH, (const Cmp*)ws.act[l], dZ, dZw);
-    }
-    const Act* X = (const Act*)ws.X[l];
-    if (kTc) {
-      // bf16 operands: dZ row-major and transposed, X_l transposed
-      bf16_copy_T<Cmp>(s, st, sh, dZ, h1, h1, g16, h1, t16b);
-      bf16_copy_T<Act>(s, st, sh, X, d.ldx, d.k_self, nullptr, 0, t16a);
     }
     // dV_self (internal [k_self][h1]) += X^T dZ
     {
@@ -667,15 +808,18 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
     }
     colsum<Cmp, Cmp>(s, st, dZw, sh.B, h1, h1, gradc + pl.b[l]);
     // dU (internal [2 d_h][h1]) += Hbar^T dZw
-    const int splitB = (int)std::max(1, std::min(32, sh.B / 256));
     {
       ProfScope ps(s->prof, kProfBwdGemm, st);
-      if constexpr (kTc)
-        gemm<Act, Cmp, Cmp, Cmp>(st, 2 * d.d_h, h1, sh.B, (const Act*)ws.Hbar[l], 1, 2 * d.d_h, dZw, h1, 1,
-                                 gradc + pl.UT[l], h1, 1, (const Cmp*)nullptr, 0, splitB, true);
-      else
-        simt::launch_gemm<Cmp>({2 * d.d_h, h1, sh.B, (const Cmp*)ws.Hbar[l], 2 * d.d_h, dZw, h1, gradc + pl.UT[l], h1,
-                                nullptr, 0, 1}, true, false, kAnySplit, s->sm_count, st);
+      const Cmp* Hb = (const Cmp*)ws.Hbar[l];
+      if constexpr (kTc) {
+        // the means in FP32 (2 d_h is a multiple of 8), in the buffer their gradient fills below
+        const int64_t n8 = (int64_t)sh.B * 2 * d.d_h / 8;
+        k_widen_bf16<<<(unsigned)std::min<int64_t>((n8 + 255) / 256, 8 * s->sm_count), 256, 0, st>>>(
+            n8, (const uint4*)ws.Hbar[l], (float4*)dHbar);
+        Hb = dHbar;
+      }
+      simt::launch_gemm<Cmp>({2 * d.d_h, h1, sh.B, Hb, 2 * d.d_h, dZw, h1, gradc + pl.UT[l], h1, nullptr, 0, 1}, true, false,
+                             kAnySplit, s->sm_count, st);
     }
     // dX = dZ V_self^T  ([R][k_self], row stride ldx)
     {
@@ -693,9 +837,13 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
         simt::launch_gemm<Cmp>({sh.B, 2 * d.d_h, h1, dZw, h1, prep + pl.UT[l], h1, dHbar, 2 * d.d_h, nullptr, 0, 0}, false,
                                true, 1, s->sm_count, st);
       }
-      const int64_t n = (int64_t)sh.B * N * h1;
+      const int V = sizeof(Cmp) == 4 && h1 % 4 == 0 ? 4 : 1;
+      const int64_t n = (int64_t)sh.B * N * (h1 / V);
+      const unsigned blocks = (unsigned)((n + 255) / 256);
       ProfScope ps(s->prof, kProfBwdMisc, st);
-      k_bwd_dh<Cmp><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
+      if constexpr (sizeof(Cmp) == 4)
+        if (V == 4) k_bwd_dh<Cmp, 4><<<blocks, 256, 0, st>>>(sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
+      if (V == 1) k_bwd_dh<Cmp, 1><<<blocks, 256, 0, st>>>(sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
     }
     // two-electron stream level l
     if (L > 1) {
@@ -712,7 +860,7 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       if (Mode::kMode == FN_BF16_MIXED) {
         const size_t smem = smem_pair_bwd_mma(N);
         cudaFuncSetAttribute(k_pair_bwd_mma<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pair_bwd_mma<Wlk><<<sh.B, 128, smem, st>>>(r, sh, a);
+        k_pair_bwd_mma<Wlk><<<(unsigned)std::min(sh.B, 6 * s->sm_count), 128, smem, st>>>(r, sh, a);
       } else {
         k_pair_bwd<Cmp, Wlk><<<sh.B, 128, 0, st>>>(r, sh, a);
       }

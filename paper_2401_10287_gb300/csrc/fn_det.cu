@@ -1034,6 +1034,157 @@ __global__ void __launch_bounds__(128, 3) k_det_value_small(Shape sh, DetArgs a)
   }
 }
 
+// Gradient's value pass, FP64 blocks of at most 8 x 8: log|psi| as in k_det_value_small, and the
+// backward seed rho_k A^{-T}.  One thread inverts one block in registers (Gauss-Jordan in place,
+// partial pivoting by predicated row swaps; the column permutation of the inverse goes into
+// the store addresses), 128 / (2K) walkers per CTA.  The factors in shared memory with two
+// substitutions per column took 488 us for the 131072 7 x 7 blocks of 4096 N2 walkers, bound by the
+// latency of 8 warps per SM; n^3 multiply-adds per block are @SEED@ us of the FP64 pipe.
+template <int NN, int C>
+struct GjStep {
+  static __device__ __forceinline__ void run(double (&a)[NN][NN], int (&piv)[NN], double& mant, int& expo,
+                                             bool& singular) {
+    auto best = abs_key(a[C][C]);
+    int pr = C;
+#pragma unroll
+    for (int r = C + 1; r < NN; ++r) {
+      const auto v = abs_key(a[r][C]);
+      if (v > best) { best = v; pr = r; }
+    }
+    if (best == 0) singular = true;
+    piv[C] = pr;
+#pragma unroll
+    for (int r = C + 1; r < NN; ++r) {
+      const bool sw = r == pr;
+#pragma unroll
+      for (int j = 0; j < NN; ++j) {
+        const double t = a[C][j];
+        a[C][j] = sw ? a[r][j] : t;
+        a[r][j] = sw ? t : a[r][j];
+      }
+    }
+    const double p = a[C][C], rp = 1.0 / p;
+    int e, e2;
+    mant *= frexp(pr != C ? -p : p, &e);
+    mant = frexp(mant, &e2);
+    expo += e + e2;
+    a[C][C] = 1.0;
+#pragma unroll
+    for (int j = 0; j < NN; ++j) a[C][j] *= rp;
+#pragma unroll
+    for (int r = 0; r < NN; ++r) {
+      if (r == C) continue;
+      const double f = a[r][C];
+      a[r][C] = 0.0;
+#pragma unroll
+      for (int j = 0; j < NN; ++j) a[r][j] -= f * a[C][j];
+    }
+    GjStep<NN, C + 1>::run(a, piv, mant, expo, singular);
+  }
+};
+template <int NN>
+struct GjStep<NN, NN> {
+  static __device__ __forceinline__ void run(double (&)[NN][NN], int (&)[NN], double&, int&, bool&) {}
+};
+
+// out[i n + j] = (A^{-1})[j][i]; det A = mant 2^expo (mant = 0 and a zero inverse if singular)
+template <int NN, typename PhiT>
+__device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, double* __restrict__ out, double* mant_out,
+                                            int* expo_out) {
+  double a[NN][NN], mant = 1.0;
+  int piv[NN], expo = 0;
+  bool singular = false;
+#pragma unroll
+  for (int i = 0; i < NN; ++i)
+#pragma unroll
+    for (int j = 0; j < NN; ++j) a[i][j] = widen<double, PhiT>(Ag[i * NN + j]);
+  GjStep<NN, 0>::run(a, piv, mant, expo, singular);
+  // the row swaps of A are column swaps of its inverse, undone last to first: column c of `a` is
+  // column col[c] of A^{-1}
+  int col[NN];
+#pragma unroll
+  for (int c = 0; c < NN; ++c) col[c] = c;
+#pragma unroll
+  for (int c = 0; c < NN; ++c) {
+#pragma unroll
+    for (int r = c + 1; r < NN; ++r) {
+      const bool sw = piv[c] == r;
+      const int t = col[c];
+      col[c] = sw ? col[r] : t;
+      col[r] = sw ? t : col[r];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NN; ++c)
+#pragma unroll
+    for (int j = 0; j < NN; ++j) out[col[c] * NN + j] = singular ? 0.0 : a[j][c];
+  *mant_out = singular ? 0.0 : mant;
+  *expo_out = singular ? 0 : expo;
+}
+
+template <typename PhiT>
+__global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) {
+  __shared__ double mt2[128], rho[64];
+  __shared__ int ex2[128];
+  const int K = a.K, NM = 2 * K, per_cta = 128 / NM;
+  const int wl = threadIdx.x / NM, p = threadIdx.x % NM, w0 = blockIdx.x * per_cta, w = w0 + wl;
+  const int ns[2] = {sh.n_up, sh.n_dn};
+  const int64_t dn_off = (int64_t)K * ns[0] * ns[0], per = dn_off + (int64_t)K * ns[1] * ns[1];
+  double* io = (double*)a.inv_out;
+  if (wl < per_cta && w < sh.B) {
+    const int k = p >> 1, sp = p & 1, n = ns[sp];
+    const int64_t off = (sp ? dn_off : 0) + (int64_t)k * n * n;
+    const PhiT* A = (const PhiT*)a.Phi + (int64_t)w * a.PW + off;
+    double* out = io + (int64_t)w * per + off;
+    double* m = mt2 + threadIdx.x;
+    int* e = ex2 + threadIdx.x;
+    switch (n) {
+      case 0: *m = 1.0; *e = 0; break;
+      case 1: invert_regs<1, PhiT>(A, out, m, e); break;
+      case 2: invert_regs<2, PhiT>(A, out, m, e); break;
+      case 3: invert_regs<3, PhiT>(A, out, m, e); break;
+      case 4: invert_regs<4, PhiT>(A, out, m, e); break;
+      case 5: invert_regs<5, PhiT>(A, out, m, e); break;
+      case 6: invert_regs<6, PhiT>(A, out, m, e); break;
+      case 7: invert_regs<7, PhiT>(A, out, m, e); break;
+      default: invert_regs<8, PhiT>(A, out, m, e); break;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < per_cta && w0 + (int)threadIdx.x < sh.B) {
+    const int w2 = w0 + threadIdx.x;
+    const double* mt = mt2 + threadIdx.x * NM;
+    const int* ex = ex2 + threadIdx.x * NM;
+    int emax = INT_MIN;
+    for (int k = 0; k < K; ++k)
+      if (mt[2 * k] * mt[2 * k + 1] != 0 && ex[2 * k] + ex[2 * k + 1] > emax) emax = ex[2 * k] + ex[2 * k + 1];
+    double S = 0;
+    for (int k = 0; k < K; ++k) {
+      const double mk = mt[2 * k] * mt[2 * k + 1];
+      const double t = mk != 0 ? ldexp(mk, ex[2 * k] + ex[2 * k + 1] - emax) : 0.0;
+      rho[threadIdx.x * K + k] = t;
+      S += t;
+    }
+    for (int k = 0; k < K; ++k) rho[threadIdx.x * K + k] = S != 0 ? rho[threadIdx.x * K + k] / S : 0.0;
+    const int sgn = S > 0 ? 1 : (S < 0 ? -1 : 0);
+    const double lpsi = sgn == 0 ? log(fabs(S)) : log(fabs(S)) + (double)emax * 0.6931471805599453;
+    if (a.log_psi) a.log_psi[w2] = lpsi;
+    if (a.sign) a.sign[w2] = (int8_t)sgn;
+    if (sgn == 0) atomicOr(a.status, kStatusSingular);
+    else if (!isfinite(lpsi)) atomicOr(a.status, kStatusNonFinite);
+  }
+  __syncthreads();
+  // scale by rho_k, consecutive elements per lane (the inverses of this CTA are in L2)
+  const int nw = min(per_cta, sh.B - w0);
+  for (int v = 0; v < nw; ++v) {
+    double* o = io + (int64_t)(w0 + v) * per;
+    for (int e = threadIdx.x; e < (int)per; e += blockDim.x) {
+      const int k = e < dn_off ? e / (ns[0] * ns[0]) : (e - (int)dn_off) / (ns[1] * ns[1]);
+      o[e] *= rho[v * K + k];
+    }
+  }
+}
+
 // ---- local-energy pass for small blocks --------------------------------------------------
 // Blocks of at most 4 x 4 and at most 8 electrons (hydrogen, lithium hydride and its ions,
 // atoms up to oxygen): one thread per (walker, determinant, spin) block does the
@@ -1269,6 +1420,9 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
   } else if (!keep_inverse && nmax <= 8) {
     const int per_cta = 128 / (2 * K);
     k_det_value_small<Det, PhiT><<<(unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st>>>(sh, a);
+  } else if (std::is_same<Det, double>::value && nmax <= 8) {
+    const int per_cta = 128 / (2 * K);
+    k_det_seed_small<PhiT><<<(unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st>>>(sh, a);
   } else {
     const int threads = (int)round_up(2 * K, 32);
     const size_t vsmem = smem_det_value(sizeof(Det), nmax, K, keep_inverse);
