@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "fn_internal.cuh"
+#include "fn_small.cuh"
 
 namespace fn {
 
@@ -328,6 +329,23 @@ static const char* shared_memory_overflow(const fn_system* s, size_t limit, size
   return nullptr;
 }
 
+// Metropolis steps from log|psi| of the walkers (parameters prepared): the single-kernel chain of a
+// small network, or propose, value pass and accept per step.
+template <class Mode>
+static void launch_mcmc(const fn_system* s, void* walkers, double* lp, int B, int n_steps, double step_size,
+                        uint64_t seed, uint64_t step_offset, int64_t* accept, cudaStream_t st) {
+  if (small_covers(s)) {
+    launch_small_mcmc(s, walkers, lp, B, n_steps, step_size, seed, step_offset, accept, st);
+    return;
+  }
+  for (int k = 0; k < n_steps; ++k) {
+    const uint32_t step = (uint32_t)(step_offset + (uint64_t)k);
+    launch_propose<Mode>(s, B, walkers, s->ws.walk2, step_size, seed, step, st);
+    launch_log_psi<Mode>(s, s->ws.walk2, B, s->ws.lp2, nullptr, st);
+    launch_accept<Mode>(s, B, walkers, s->ws.walk2, lp, s->ws.lp2, seed, step, accept, st);
+  }
+}
+
 static fn_status check_launch(fn_system* s, const char* what) {
   if (s->host_error != FN_OK) {
     const fn_status e = s->host_error;
@@ -509,10 +527,8 @@ fn_status fn_log_psi(fn_system_t s, const void* d_params, const void* d_walkers,
   cudaStream_t cs = (cudaStream_t)stream;
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
-    const Shape sh = make_shape(s, B, 1);
     launch_prep_params<Mode>(s, d_params, false, cs);
-    launch_forward<Mode>(s, d_walkers, sh, false, cs);
-    launch_det_energy<Mode>(s, d_walkers, sh, nullptr, d_log_psi, d_sign, false, cs);
+    launch_log_psi<Mode>(s, d_walkers, B, d_log_psi, d_sign, cs);
     return 0;
   });
   return check_launch(s, "log_psi");
@@ -547,15 +563,8 @@ fn_status fn_mcmc_steps(fn_system_t s, const void* d_params, void* d_walkers, do
   cudaStream_t cs = (cudaStream_t)stream;
   dispatch(s, [&](auto m) {
     using Mode = decltype(m);
-    const Shape sh = make_shape(s, B, 1);
     launch_prep_params<Mode>(s, d_params, false, cs);
-    for (int k = 0; k < n_steps; ++k) {
-      const uint32_t step = (uint32_t)(step_offset + (uint64_t)k);
-      launch_propose<Mode>(s, B, d_walkers, s->ws.walk2, step_size, seed, step, cs);
-      launch_forward<Mode>(s, s->ws.walk2, sh, false, cs);
-      launch_det_energy<Mode>(s, s->ws.walk2, sh, nullptr, s->ws.lp2, nullptr, false, cs);
-      launch_accept<Mode>(s, B, d_walkers, s->ws.walk2, d_log_psi, s->ws.lp2, seed, step, d_accept, cs);
-    }
+    launch_mcmc<Mode>(s, d_walkers, d_log_psi, B, n_steps, step_size, seed, step_offset, d_accept, cs);
     return 0;
   });
   return check_launch(s, "mcmc_steps");
@@ -664,16 +673,10 @@ fn_status fn_vmc_iteration(fn_system_t s, const fn_train_config* c, void* d_para
     const Shape full = make_shape(s, B, 3 * s->N + 2);
     launch_prep_params<Mode>(s, d_params, true, cs);
     // log|psi| of the persistent walkers under the current parameters
-    launch_forward<Mode>(s, d_walkers, value, false, cs);
-    launch_det_energy<Mode>(s, d_walkers, value, nullptr, d_log_psi, nullptr, false, cs);
+    launch_log_psi<Mode>(s, d_walkers, B, d_log_psi, nullptr, cs);
     // Metropolis, step indices iteration * n + k
-    for (int k = 0; k < c->n_mcmc_steps; ++k) {
-      const uint32_t step = (uint32_t)((uint64_t)iteration * (uint64_t)c->n_mcmc_steps + (uint64_t)k);
-      launch_propose<Mode>(s, B, d_walkers, s->ws.walk2, c->step_size, c->seed, step, cs);
-      launch_forward<Mode>(s, s->ws.walk2, value, false, cs);
-      launch_det_energy<Mode>(s, s->ws.walk2, value, nullptr, s->ws.lp2, nullptr, false, cs);
-      launch_accept<Mode>(s, B, d_walkers, s->ws.walk2, d_log_psi, s->ws.lp2, c->seed, step, d_accept, cs);
-    }
+    launch_mcmc<Mode>(s, d_walkers, d_log_psi, B, c->n_mcmc_steps, c->step_size, c->seed,
+                      (uint64_t)iteration * (uint64_t)c->n_mcmc_steps, d_accept, cs);
     // local energies (Eqs. 2-3)
     launch_forward<Mode>(s, d_walkers, full, false, cs);
     launch_det_energy<Mode>(s, d_walkers, full, d_e_local, nullptr, nullptr, false, cs);

@@ -279,6 +279,9 @@ template <class Mode> void launch_forward(const fn_system* s, const void* walker
 template <class Mode> void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
                                              double* e_local, double* log_psi, int8_t* sign,
                                              bool keep_inverse, cudaStream_t st);
+// log|psi| and sign (parameters prepared): one kernel for a small network, else forward and determinants.
+template <class Mode> void launch_log_psi(const fn_system* s, const void* walkers, int B, double* log_psi,
+                                          int8_t* sign, cudaStream_t st);
 template <class Mode> void launch_init_walkers(const fn_system* s, int B, uint64_t seed, double std_,
                                                void* walkers, cudaStream_t st);
 template <class Mode> void launch_init_params(const fn_system* s, uint64_t seed, void* params,

@@ -120,10 +120,8 @@ static fn_status log_psi_noalloc(fn_system* s, const void* params, const void* w
   Profiler* saved_prof = s->prof;
   s->ws = arena;
   s->prof = nullptr;
-  const Shape sh = make_shape(s, B, 1);
   launch_prep_params<Mode>(s, params, false, st);
-  launch_forward<Mode>(s, walkers, sh, false, st);
-  launch_det_energy<Mode>(s, walkers, sh, nullptr, log_psi, sign, false, st);
+  launch_log_psi<Mode>(s, walkers, B, log_psi, sign, st);
   s->ws = saved;
   s->prof = saved_prof;
   if (s->host_error != FN_OK) {

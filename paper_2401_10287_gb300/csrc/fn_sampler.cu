@@ -26,15 +26,22 @@ __global__ void k_init_walkers(int B, int N, const int* __restrict__ atom, const
   out[gid] = (Wlk)__dadd_rn(nuc[3 * atom[e] + c], __dmul_rn(z, init_std));
 }
 
+// One thread per Box-Muller pair, i.e. per two coordinates of a walker: the FP64 logarithm, root,
+// sine and cosine are most of the kernel.
 template <typename Wlk>
 __global__ void k_propose(int B, int N, const Wlk* __restrict__ r, Wlk* __restrict__ out, double step,
                           uint64_t seed, uint32_t step_idx, uint64_t walker_offset) {
+  const int n3 = 3 * N, pairs = (n3 + 1) / 2;
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)B * N * 3) return;
-  const int64_t w = gid / (3 * N);
-  const int j = (int)(gid % (3 * N));
-  const double z = normal_at((uint64_t)j, (uint32_t)(walker_offset + w), step_idx, kStreamProposal, seed);
-  out[gid] = (Wlk)__dadd_rn((double)r[gid], __dmul_rn(z, step));
+  if (gid >= (int64_t)B * pairs) return;
+  const int64_t w = gid / pairs;
+  const int j = 2 * (int)(gid - w * pairs);
+  double z0, z1;
+  normal_pair((uint32_t)(j >> 1), (uint32_t)(walker_offset + w), step_idx, kStreamProposal, seed, &z0, &z1);
+  const Wlk* rw = r + w * n3 + j;
+  Wlk* ow = out + w * n3 + j;
+  ow[0] = (Wlk)__dadd_rn((double)rw[0], __dmul_rn(z0, step));
+  if (j + 1 < n3) ow[1] = (Wlk)__dadd_rn((double)rw[1], __dmul_rn(z1, step));
 }
 
 template <typename Wlk>
@@ -99,9 +106,9 @@ template <class Mode>
 void launch_propose(const fn_system* s, int B, const void* walkers, void* out, double step, uint64_t seed,
                     uint32_t step_idx, cudaStream_t st) {
   using Wlk = typename Mode::Wlk;
-  const int64_t n = (int64_t)B * s->N * 3;
+  const int64_t n = (int64_t)B * ((3 * s->N + 1) / 2);
   ProfScope ps(s->prof, kProfSampler, st);
-  k_propose<Wlk><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(B, s->N, (const Wlk*)walkers, (Wlk*)out, step, seed,
+  k_propose<Wlk><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(B, s->N, (const Wlk*)walkers, (Wlk*)out, step, seed,
                                                                 step_idx, s->walker_offset);
 }
 
