@@ -28,6 +28,8 @@ namespace fn {
 // e and c may be the same buffer: each thread reads e[w] before writing c[w], and only
 // after the barrier that ends the sum.
 __global__ void k_energy_weights(int B, const double* e, double* c, double* __restrict__ mean_out) {
+  pdl_wait();
+  pdl_launch();
   __shared__ double red[1024];
   double s = 0.0;
   for (int w = threadIdx.x; w < B; w += blockDim.x) s += e[w];
@@ -46,12 +48,14 @@ template <class Mode>
 void launch_energy_weights(const fn_system* s, int B, const double* e_local, double* weights, double* e_mean,
                            cudaStream_t st) {
   ProfScope ps(s->prof, kProfBwdMisc, st);
-  k_energy_weights<<<1, 1024, 0, st>>>(B, e_local, weights, e_mean);
+  launch_k(true, k_energy_weights, 1, 1024, 0, st, B, e_local, weights, e_mean);
 }
 
 // ---- column sums (atomic) -------------------------------------------------------------
 template <typename T, typename Cmp>
 __global__ void k_colsum(const T* __restrict__ src, int64_t rows, int64_t lds, int cols, Cmp* __restrict__ dst) {
+  pdl_wait();
+  pdl_launch();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= cols) return;
   const int64_t chunk = (rows + gridDim.y - 1) / gridDim.y;
@@ -76,7 +80,7 @@ static void colsum(const fn_system* s, cudaStream_t st, const T* src, int64_t ro
   // 58368 x 112 orbital gradients (26 MB), bound by one load in flight per thread
   const int64_t want = std::max<int64_t>(1, 4 * s->sm_count / ((cols + 127) / 128));
   dim3 grid((cols + 127) / 128, (unsigned)std::min<int64_t>(want, std::max<int64_t>(1, rows / 16)));
-  k_colsum<T, Cmp><<<grid, 128, 0, st>>>(src, rows, ld, cols, dst);
+  launch_k(true, k_colsum<T, Cmp>, grid, 128, 0, st, src, rows, ld, cols, dst);
 }
 
 // ---- BF16 operands of the tensor-core backward GEMMs (BF16 mode) ---------------------
@@ -87,6 +91,8 @@ static void colsum(const fn_system* s, cudaStream_t st, const T* src, int64_t ro
 template <typename Tin>
 __global__ void k_bf16_copy_T(Shape sh, const Tin* __restrict__ in, int64_t ld_in, int cols,
                               __nv_bfloat16* __restrict__ out, int64_t ld_out, __nv_bfloat16* __restrict__ outT) {
+  pdl_wait();
+  pdl_launch();
   __shared__ float tile[32][33];
   const int c0 = blockIdx.x * 32;
   const int64_t r0 = (int64_t)blockIdx.y * 32;
@@ -113,6 +119,8 @@ __global__ void k_bf16_copy_T(Shape sh, const Tin* __restrict__ in, int64_t ld_i
 // input of an N2 layer at 4096 walkers, 75 MB in all).
 __global__ void __launch_bounds__(256) k_bf16_T(Shape sh, const __nv_bfloat16* __restrict__ in, int64_t ld_in, int cols,
                                                 __nv_bfloat16* __restrict__ outT) {
+  pdl_wait();
+  pdl_launch();
   __shared__ unsigned short tile[64][66];
   const int c0 = blockIdx.x * 64, tid = threadIdx.x;
   const int64_t r0 = (int64_t)blockIdx.y * 64;
@@ -142,7 +150,9 @@ __global__ void __launch_bounds__(256) k_bf16_T(Shape sh, const __nv_bfloat16* _
 static void bf16_T(const fn_system* s, cudaStream_t st, const Shape& sh, const void* in, int64_t ld_in, int cols,
                    __nv_bfloat16* outT) {
   ProfScope ps(s->prof, kProfBwdMisc, st);
-  k_bf16_T<<<dim3((cols + 63) / 64, (unsigned)(sh.R / 64)), 256, 0, st>>>(sh, (const __nv_bfloat16*)in, ld_in, cols, outT);
+  launch_k(overlap_launches(sh), k_bf16_T, dim3((cols + 63) / 64, (unsigned)(sh.R / 64)), 256, 0, st, sh,
+      (const __nv_bfloat16*)in,
+             ld_in, cols, outT);
 }
 
 template <typename Tin>
@@ -150,7 +160,8 @@ static void bf16_copy_T(const fn_system* s, cudaStream_t st, const Shape& sh, co
                         __nv_bfloat16* out, int64_t ld_out, __nv_bfloat16* outT) {
   ProfScope ps(s->prof, kProfBwdMisc, st);
   dim3 grid((cols + 31) / 32, (unsigned)(sh.R / 32));
-  k_bf16_copy_T<Tin><<<grid, dim3(32, 8), 0, st>>>(sh, in, ld_in, cols, out, ld_out, outT);
+  launch_k(overlap_launches(sh), k_bf16_copy_T<Tin>, grid, dim3(32, 8), 0, st, sh, in, ld_in, cols, out, ld_out,
+      outT);
 }
 
 // K splits of a weight-gradient GEMM (K = all rows): about two CTAs per SM, >= 4 k-blocks each.
@@ -183,6 +194,8 @@ struct OrbBwdArgs {
 // registers (MM >= the number of nuclei bounds the unrolled per-nucleus arrays).
 template <typename Cmp, typename Det, typename Wlk, int MM>
 __global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbBwdArgs a) {
+  pdl_wait();
+  pdl_launch();
   const int spin = blockIdx.y;
   const int n = spin ? sh.n_dn : sh.n_up, n_o = spin ? sh.n_up : sh.n_dn;
   if (n == 0) return;
@@ -301,6 +314,8 @@ __global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ 
 template <typename Cmp>
 __global__ void k_bwd_tanh(Shape sh, int h1, const Cmp* __restrict__ dH, const Cmp* __restrict__ act,
                            Cmp* __restrict__ dZ, Cmp* __restrict__ dZw) {
+  pdl_wait();
+  pdl_launch();
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gid >= (int64_t)sh.B * h1) return;
   const int w = (int)(gid / h1), c = (int)(gid % h1);
@@ -321,6 +336,8 @@ __global__ void k_bwd_tanh(Shape sh, int h1, const Cmp* __restrict__ dH, const C
 __global__ void __launch_bounds__(256) k_bwd_tanh_bf16(Shape sh, int h1, const float* __restrict__ dH,
                                                        const float* __restrict__ act, __nv_bfloat16* __restrict__ out,
                                                        __nv_bfloat16* __restrict__ outT, float* __restrict__ dZw) {
+  pdl_wait();
+  pdl_launch();
   __shared__ float tile[kTileRows][33];
   const int c0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int q = blockIdx.y;
@@ -365,6 +382,8 @@ __global__ void __launch_bounds__(256) k_bwd_tanh_bf16(Shape sh, int h1, const f
 template <typename Cmp, int V>
 __global__ void k_bwd_dh(Shape sh, int h1, int ldx, int d_h, const Cmp* __restrict__ dX,
                          const Cmp* __restrict__ dHbar, Cmp* __restrict__ dH) {
+  pdl_wait();
+  pdl_launch();
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int hv = h1 / V;
   const int64_t wi = gid / hv;
@@ -399,6 +418,8 @@ struct PairBwdArgs {
 
 template <typename Cmp, typename Wlk>
 __global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* __restrict__ r, Shape sh, PairBwdArgs a) {
+  pdl_wait();
+  pdl_launch();
   __shared__ Cmp red[4][32][33];
   __shared__ Cmp sW[32][33];                                   // W_l[q][c], zero outside [h2][d_g]
   const int w = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -494,6 +515,8 @@ __global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* __restrict__ r, Sha
 
 template <typename Wlk>
 __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r, Shape sh, PairBwdArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = lane >> 2, tig = lane & 3;
@@ -648,6 +671,8 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
 }
 
 __global__ void k_widen_bf16(int64_t n8, const uint4* __restrict__ in, float4* __restrict__ out) {
+  pdl_wait();
+  pdl_launch();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
     const uint4 v = __ldg(in + i);
     out[2 * i] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
@@ -660,6 +685,8 @@ __global__ void k_widen_bf16(int64_t n8, const uint4* __restrict__ in, float4* _
 // ---- internal layout -> blob order ---------------------------------------------------
 template <typename Par, typename Cmp>
 __global__ void k_unprep(Par* __restrict__ blob, const CopyDesc* __restrict__ descs, const Cmp* __restrict__ gradc) {
+  pdl_wait();
+  pdl_launch();
   const CopyDesc d = descs[blockIdx.y];
   if (d.to16) return;
   const int64_t n = (int64_t)d.rows * d.cols;
@@ -728,10 +755,14 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
     const int threads = (int)std::min<int64_t>(1024, round_up((int64_t)K * std::max(s->n_up, s->n_dn), 32));
     dim3 grid((sh.B + a.chunk - 1) / a.chunk, 2);
     ProfScope ps(s->prof, kProfBwdOrb, st);
-    if (s->M <= 2) k_orb_bwd<Cmp, Det, Wlk, 2><<<grid, threads, 0, st>>>(r, s->d_nuclei, sh, a);
-    else if (s->M <= 4) k_orb_bwd<Cmp, Det, Wlk, 4><<<grid, threads, 0, st>>>(r, s->d_nuclei, sh, a);
-    else if (s->M <= 8) k_orb_bwd<Cmp, Det, Wlk, 8><<<grid, threads, 0, st>>>(r, s->d_nuclei, sh, a);
-    else k_orb_bwd<Cmp, Det, Wlk, kMaxNuclei><<<grid, threads, 0, st>>>(r, s->d_nuclei, sh, a);
+    if (s->M <= 2) launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, 2>, grid, threads, 0, st, r, s->d_nuclei,
+        sh, a);
+    else if (s->M <= 4) launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, 4>, grid, threads, 0, st, r,
+        s->d_nuclei, sh, a);
+    else if (s->M <= 8) launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, 8>, grid, threads, 0, st, r,
+        s->d_nuclei, sh, a);
+    else launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, kMaxNuclei>, grid, threads, 0, st, r, s->d_nuclei,
+        sh, a);
   }
   const int ns[2] = {s->n_up, s->n_dn};
   __nv_bfloat16* g16 = (__nv_bfloat16*)ws.g16;
@@ -787,14 +818,18 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       // operands of the tensor-core products: dZ row-major and transposed, X_l transposed
       {
         ProfScope ps(s->prof, kProfBwdMisc, st);
-        k_bwd_tanh_bf16<<<dim3(h1 / 32, sh.tiles), 256, 0, st>>>(sh, h1, dH, (const float*)ws.act[l], g16, t16b, dZw);
+        launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_tanh_bf16, dim3(h1 / 32, sh.tiles), 256, 0, st, sh, h1, dH,
+            (const float*)ws.act[l], g16,
+                   t16b, dZw);
       }
       bf16_T(s, st, sh, ws.X[l], d.ldx, d.k_self, t16a);
     } else {
       cudaMemsetAsync(dZ, 0, sizeof(Cmp) * R * h1, st);
       const int64_t n = (int64_t)sh.B * h1;
       ProfScope ps(s->prof, kProfBwdMisc, st);
-      k_bwd_tanh<Cmp><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(sh, h1, dH, (const Cmp*)ws.act[l], dZ, dZw);
+      launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_tanh<Cmp>, (unsigned)((n + 255) / 256), 256, 0, st, sh, h1, dH,
+          (const Cmp*)ws.act[l], dZ,
+                 dZw);
     }
     // dV_self (internal [k_self][h1]) += X^T dZ
     {
@@ -814,8 +849,9 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       if constexpr (kTc) {
         // the means in FP32 (2 d_h is a multiple of 8), in the buffer their gradient fills below
         const int64_t n8 = (int64_t)sh.B * 2 * d.d_h / 8;
-        k_widen_bf16<<<(unsigned)std::min<int64_t>((n8 + 255) / 256, 8 * s->sm_count), 256, 0, st>>>(
-            n8, (const uint4*)ws.Hbar[l], (float4*)dHbar);
+        launch_k(overlap_launches(sh, sizeof(Cmp)), k_widen_bf16, (unsigned)std::min<int64_t>((n8 + 255) / 256, 8 * s->sm_count),
+            256, 0, st, n8,
+                   (const uint4*)ws.Hbar[l], (float4*)dHbar);
         Hb = dHbar;
       }
       simt::launch_gemm<Cmp>({2 * d.d_h, h1, sh.B, Hb, 2 * d.d_h, dZw, h1, gradc + pl.UT[l], h1, nullptr, 0, 1}, true, false,
@@ -842,8 +878,10 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       const unsigned blocks = (unsigned)((n + 255) / 256);
       ProfScope ps(s->prof, kProfBwdMisc, st);
       if constexpr (sizeof(Cmp) == 4)
-        if (V == 4) k_bwd_dh<Cmp, 4><<<blocks, 256, 0, st>>>(sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
-      if (V == 1) k_bwd_dh<Cmp, 1><<<blocks, 256, 0, st>>>(sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
+        if (V == 4) launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_dh<Cmp, 4>, blocks, 256, 0, st, sh, h1, d.ldx, d.d_h, dX,
+            dHbar, dH);
+      if (V == 1) launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_dh<Cmp, 1>, blocks, 256, 0, st, sh, h1, d.ldx, d.d_h, dX,
+          dHbar, dH);
     }
     // two-electron stream level l
     if (L > 1) {
@@ -860,15 +898,17 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       if (Mode::kMode == FN_BF16_MIXED) {
         const size_t smem = smem_pair_bwd_mma(N);
         cudaFuncSetAttribute(k_pair_bwd_mma<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pair_bwd_mma<Wlk><<<(unsigned)std::min(sh.B, 6 * s->sm_count), 128, smem, st>>>(r, sh, a);
+        launch_k(overlap_launches(sh, sizeof(Cmp)), k_pair_bwd_mma<Wlk>, (unsigned)std::min(sh.B, 6 * s->sm_count), 128, smem,
+            st, r, sh, a);
       } else {
-        k_pair_bwd<Cmp, Wlk><<<sh.B, 128, 0, st>>>(r, sh, a);
+        launch_k(overlap_launches(sh, sizeof(Cmp)), k_pair_bwd<Cmp, Wlk>, sh.B, 128, 0, st, r, sh, a);
       }
     }
   }
   dim3 grid(32, s->n_descs);
   ProfScope ps(s->prof, kProfBwdMisc, st);
-  k_unprep<Par, Cmp><<<grid, 256, 0, st>>>((Par*)grad, (const CopyDesc*)s->d_descs, gradc);
+  launch_k(overlap_launches(sh, sizeof(Cmp)), k_unprep<Par, Cmp>, grid, 256, 0, st, (Par*)grad, (const CopyDesc*)s->d_descs,
+      gradc);
 }
 
 #define FN_INST(M)                                                                                           \

@@ -278,6 +278,8 @@ __device__ __forceinline__ bool tangent_item_split(const float* Ch, const float*
 template <typename Det, typename Wlk, typename PhiT>
 __global__ void __launch_bounds__(128) k_det_energy(const Wlk* __restrict__ r, const double* __restrict__ nuc,
                                                     Shape sh, DetArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int w = blockIdx.x, tid = threadIdx.x;
   const int N = sh.N, T = sh.T, K = a.K, NC = 3 * N, NM = 2 * K;
@@ -514,6 +516,8 @@ __device__ __forceinline__ void ff_row2(const float* __restrict__ chr, const flo
 template <typename Wlk>
 __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict__ r, const double* __restrict__ nuc,
                                                            Shape sh, DetArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int w = blockIdx.x, tid = threadIdx.x;
   const int N = sh.N, T = sh.T, K = a.K, NC = 3 * N, NM = 2 * K;
@@ -812,6 +816,8 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
 // walker, one thread per (determinant, spin) block.
 template <typename Det, typename PhiT>
 __global__ void k_det_value(Shape sh, DetArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int w = blockIdx.x, tid = threadIdx.x;
   const int K = a.K, NM = 2 * K, ST = blockDim.x;
@@ -894,6 +900,8 @@ __global__ void k_det_value(Shape sh, DetArgs a) {
 // (the same signed log-sum-exp, without forming log|D_k|).
 template <typename Det, typename PhiT>
 __global__ void __launch_bounds__(128, 3) k_det_value_small(Shape sh, DetArgs a) {
+  pdl_wait();
+  pdl_launch();
   __shared__ Det mt2[128];
   __shared__ int ex2[128];
   const int K = a.K, NM = 2 * K;
@@ -1027,6 +1035,8 @@ __device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, double*
 
 template <typename PhiT>
 __global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) {
+  pdl_wait();
+  pdl_launch();
   __shared__ double mt2[128], rho[64];
   __shared__ int ex2[128];
   const int K = a.K, NM = 2 * K, per_cta = 128 / NM;
@@ -1099,6 +1109,8 @@ __global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) 
 template <int NMAX, typename Det, typename Wlk, typename PhiT>
 __global__ void __launch_bounds__(128) k_det_energy_small(const Wlk* __restrict__ r, const double* __restrict__ nuc,
                                                           Shape sh, DetArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int K = a.K, NM = 2 * K, NC = 3 * sh.N, T = sh.T;
   const int per_cta = 128 / NM;
@@ -1302,35 +1314,41 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
   a.v_nn = s->v_nn;
   a.status = s->ws.status;
   const bool full = sh.T > 1 && e_local != nullptr;
+  const bool ov = overlap_launches(sh, Mode::kMode == FN_FP64 ? 8 : 4);
   const int nmax = std::max(s->n_up, s->n_dn), K = s->cfg.n_dets;
   ProfScope ps(s->prof, full ? kProfDetFull : kProfDetValue, st);
   if (full && nmax <= 4 && s->N <= 8) {
     const int per_cta = 128 / (2 * K);
     const size_t smem = smem_det_energy_small(sizeof(Det), s->N, K);
     cudaFuncSetAttribute(k_det_energy_small<4, Det, Wlk, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_det_energy_small<4, Det, Wlk, PhiT><<<(unsigned)((sh.B + per_cta - 1) / per_cta), 128, smem, st>>>(
-        (const Wlk*)walkers, s->d_nuclei, sh, a);
+    launch_k(ov, k_det_energy_small<4, Det, Wlk, PhiT>,
+        (unsigned)((sh.B + per_cta - 1) / per_cta), 128, smem, st,
+               (const Wlk*)walkers, s->d_nuclei, sh, a);
   } else if (full && std::is_same<Det, double>::value && std::is_same<PhiT, float>::value && nmax <= kGrpN &&
              det_grp_enabled()) {
     const size_t smem = smem_det_energy_grp(s->N, K);
     cudaFuncSetAttribute(k_det_energy_grp<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_det_energy_grp<Wlk><<<sh.B, 128, smem, st>>>((const Wlk*)walkers, s->d_nuclei, sh, a);
+    launch_k(ov, k_det_energy_grp<Wlk>, sh.B, 128, smem, st, (const Wlk*)walkers, s->d_nuclei, sh,
+        a);
   } else if (full) {
     const size_t smem = smem_det_energy(sizeof(Det), nmax, s->N, K,
                                         std::is_same<Det, double>::value && std::is_same<PhiT, float>::value);
     cudaFuncSetAttribute(k_det_energy<Det, Wlk, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_det_energy<Det, Wlk, PhiT><<<sh.B, 128, smem, st>>>((const Wlk*)walkers, s->d_nuclei, sh, a);
+    launch_k(ov, k_det_energy<Det, Wlk, PhiT>, sh.B, 128, smem, st, (const Wlk*)walkers,
+        s->d_nuclei, sh, a);
   } else if (!keep_inverse && nmax <= 8) {
     const int per_cta = 128 / (2 * K);
-    k_det_value_small<Det, PhiT><<<(unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st>>>(sh, a);
+    launch_k(ov, k_det_value_small<Det, PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0,
+        st, sh, a);
   } else if (std::is_same<Det, double>::value && nmax <= 8) {
     const int per_cta = 128 / (2 * K);
-    k_det_seed_small<PhiT><<<(unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st>>>(sh, a);
+    launch_k(ov, k_det_seed_small<PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st,
+        sh, a);
   } else {
     const int threads = (int)round_up(2 * K, 32);
     const size_t vsmem = smem_det_value(sizeof(Det), nmax, K, keep_inverse);
     cudaFuncSetAttribute(k_det_value<Det, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsmem);
-    k_det_value<Det, PhiT><<<sh.B, threads, vsmem, st>>>(sh, a);
+    launch_k(ov, k_det_value<Det, PhiT>, sh.B, threads, vsmem, st, sh, a);
   }
 }
 

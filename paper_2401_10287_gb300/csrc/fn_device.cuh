@@ -6,6 +6,13 @@
 
 namespace fn {
 
+// Programmatic dependent launch.  Every kernel launched with launch_k waits here before it
+// touches memory, and lets the next kernel of the stream begin only after that: when a kernel
+// runs, everything before its predecessor is complete, so its prologue (barriers, tensor
+// memory, weights prepared at least two kernels earlier) may overlap the predecessor's tail.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ double ld(const double* p) { return *p; }
 __device__ __forceinline__ float ld(const float* p) { return *p; }
 __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }

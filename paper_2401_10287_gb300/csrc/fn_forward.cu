@@ -29,6 +29,8 @@ namespace fn {
 template <typename Par, typename Cmp>
 __global__ void k_prep(const Par* __restrict__ blob, const CopyDesc* __restrict__ descs, int n_desc,
                        Cmp* __restrict__ prep, __nv_bfloat16* __restrict__ prep16) {
+  pdl_wait();
+  pdl_launch();
   const CopyDesc d = descs[blockIdx.y];
   const int64_t n = (int64_t)d.rows * d.cols;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
@@ -140,7 +142,7 @@ void launch_prep_params(const fn_system* s, const void* params, bool full, cudaS
   using Par = typename Mode::Par; using Cmp = typename Mode::Cmp;
   dim3 grid(32, s->n_descs);
   ProfScope ps(s->prof, kProfPrep, st);
-  k_prep<Par, Cmp><<<grid, 256, 0, st>>>((const Par*)params, (const CopyDesc*)s->d_descs, s->n_descs,
+  launch_k(true, k_prep<Par, Cmp>, grid, 256, 0, st, (const Par*)params, (const CopyDesc*)s->d_descs, s->n_descs,
                                          (Cmp*)s->ws.prep,
                                          (__nv_bfloat16*)s->ws.prep16);
   if (!use_x3<Mode>(s, full)) return;
@@ -163,6 +165,8 @@ void launch_prep_params(const fn_system* s, const void* params, bool full, cudaS
 template <typename Act, typename Wlk>
 __global__ void k_features_en(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh,
                               Act* __restrict__ X0, int ldx) {
+  pdl_wait();
+  pdl_launch();
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gid >= (int64_t)sh.B * sh.N) return;
   const int w = (int)(gid / sh.N), i = (int)(gid % sh.N);
@@ -200,6 +204,8 @@ __global__ void k_features_en(const Wlk* __restrict__ r, const double* __restric
 template <typename Act, typename Wlk>
 __global__ void k_features_mean(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh,
                                 Act* __restrict__ Hbar) {
+  pdl_wait();
+  pdl_launch();
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gid >= (int64_t)sh.B * 2 * sh.M) return;
   const int w = (int)(gid / (2 * sh.M)), spin = (int)((gid / sh.M) % 2), m = (int)(gid % sh.M);
@@ -339,6 +345,8 @@ __device__ __forceinline__ void pair_matvec(const Cmp* __restrict__ sWl, const C
 
 template <typename Act, typename Cmp, typename Wlk>
 __global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Shape sh, PairArgs a, int ib) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cmp* sW = (Cmp*)smem_raw;                                  // [L-1][32][32]
   Cmp* sc = sW + (a.L - 1) * kMaxH2 * kMaxH2;               // [L-1][32]
@@ -458,6 +466,8 @@ __global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Sh
 // (i, spin, channel), then every pair is advanced through the next pair layer.
 template <typename Act, typename Cmp, typename Wlk>
 __global__ void __launch_bounds__(512) k_pair_value(const Wlk* __restrict__ r, Shape sh, PairArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cmp* sW = (Cmp*)smem_raw;
   Cmp* sc = sW + (a.L - 1) * kMaxH2 * kMaxH2;
@@ -523,6 +533,8 @@ __global__ void __launch_bounds__(512) k_pair_value(const Wlk* __restrict__ r, S
 // columns); a warp reads 512 contiguous bytes of a row.
 __global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* __restrict__ Y, int ldy, int h1,
                                   __nv_bfloat16* __restrict__ Hbar) {
+  pdl_wait();
+  pdl_launch();
   const int g8 = h1 >> 3;
   const int64_t n = (int64_t)sh.T * sh.B * 2 * g8;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
@@ -577,6 +589,8 @@ __global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* __restrict__ Y,
 
 // The same in FP32 (after the FP32 tensor-core layer): one thread per (slab, walker, spin, 4 columns).
 __global__ void k_spin_means_f32(Shape sh, const float* __restrict__ Y, int ldy, int h1, float* __restrict__ Hbar) {
+  pdl_wait();
+  pdl_launch();
   const int g4 = h1 >> 2;
   const int64_t n = (int64_t)sh.T * sh.B * 2 * g4;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
@@ -611,6 +625,8 @@ __global__ void k_spin_means_f32(Shape sh, const float* __restrict__ Y, int ldy,
 
 template <typename Wlk>
 __global__ void __launch_bounds__(128) k_pair_value_mma(const Wlk* __restrict__ r, Shape sh, PairArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int L1 = a.L - 1;
   __nv_bfloat16* wh = (__nv_bfloat16*)smem_raw;                  // [L-1][32 n][kPairWLd]: bf16(W[n][k])
@@ -726,6 +742,8 @@ __global__ void __launch_bounds__(128) k_pair_value_mma(const Wlk* __restrict__ 
 // of the spin means and d/dr_j slabs to the next layer input, as in k_pair_full.
 template <typename Wlk>
 __global__ void __launch_bounds__(256) k_pair_full_mma(const Wlk* __restrict__ r, Shape sh, PairArgs a, int ib) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int L1 = a.L - 1;
   __nv_bfloat16* wh = (__nv_bfloat16*)smem_raw;                  // [L-1][32 n][kPairWLd]: bf16(W[n][k])
@@ -925,6 +943,8 @@ __device__ __forceinline__ void env_jet(const OrbArgs& a, int spin, int ko, cons
 template <typename Cmp, typename PhiT, typename Wlk>
 __global__ void k_orbital_fixup(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbArgs a,
                                 const Cmp* __restrict__ orbP) {
+  pdl_wait();
+  pdl_launch();
   const int w = blockIdx.x / sh.N, j = blockIdx.x % sh.N;
   const int spin = j < sh.n_up ? 0 : 1;
   const int n_s = spin ? sh.n_dn : sh.n_up;
@@ -953,6 +973,8 @@ __global__ void k_orbital_fixup(const Wlk* __restrict__ r, const double* __restr
 template <typename Wlk>
 __global__ void k_envelope_values(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbArgs a,
                                   float* __restrict__ envv) {
+  pdl_wait();
+  pdl_launch();
   // one thread per (walker, electron j, orbital of j's spin); K n_s orbitals per electron.
   // Nuclei as FP32 in shared memory: the envelope values are FP32 in this mode, and FP64
   // arithmetic (conversions included) runs at a small fraction of the FP32 rate on this part.
@@ -1002,6 +1024,8 @@ __global__ void k_envelope_values(const Wlk* __restrict__ r, const double* __res
 template <typename Wlk>
 __global__ void k_envelope_values_smem(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh,
                                        OrbArgs a, float* __restrict__ envv) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) float env_smem[];
   __shared__ float nucf[3 * kMaxNuclei];
   const int M = sh.M, nc = a.aniso ? 9 : 1;
@@ -1070,16 +1094,19 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
   const Workspace& ws = s->ws;
   const int L = s->cfg.n_layers, h1 = s->cfg.h1, h2 = s->cfg.h2;
   const Cmp* prep = (const Cmp*)ws.prep;
-  const bool full = sh.T > 1;
+  const bool full = sh.T > 1, ov = overlap_launches(sh, sizeof(Cmp));
   const Wlk* r = (const Wlk*)walkers;
   // inputs
   {
     const int64_t n = (int64_t)sh.B * sh.N;
     ProfScope ps(s->prof, kProfFeatures, st);
-    k_features_en<Act, Wlk><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(r, s->d_nuclei, sh, (Act*)ws.X[0],
+    launch_k(ov, k_features_en<Act, Wlk>, (unsigned)((n + 127) / 128), 128, 0, st, r, s->d_nuclei,
+        sh, (Act*)ws.X[0],
                                                                            s->layer[0].ldx);
     const int64_t m = (int64_t)sh.B * 2 * sh.M;
-    k_features_mean<Act, Wlk><<<(unsigned)((m + 127) / 128), 128, 0, st>>>(r, s->d_nuclei, sh, (Act*)ws.Hbar[0]);
+    launch_k(ov, k_features_mean<Act, Wlk>, (unsigned)((m + 127) / 128), 128, 0, st, r,
+        s->d_nuclei, sh,
+               (Act*)ws.Hbar[0]);
   }
   {
     PairArgs pa{};
@@ -1103,24 +1130,25 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         const int64_t blocks_m =
             std::min<int64_t>((int64_t)sh.B * ((sh.N + ibm - 1) / ibm), (int64_t)s->sm_count * 8);
         cudaFuncSetAttribute(k_pair_full_mma<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_m);
-        k_pair_full_mma<Wlk><<<(unsigned)blocks_m, 256, smem_m, st>>>(r, sh, pa, ibm);
+        launch_k(ov, k_pair_full_mma<Wlk>, (unsigned)blocks_m, 256, smem_m, st, r, sh, pa, ibm);
       } else {
       const size_t smem = smem_pair_full(sizeof(Cmp), sh.N, L, ib);
       const int64_t blocks = (int64_t)sh.B * ((sh.N + ib - 1) / ib);
       cudaFuncSetAttribute(k_pair_full<Act, Cmp, Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_pair_full<Act, Cmp, Wlk><<<(unsigned)blocks, 32 * warps, smem, st>>>(r, sh, pa, ib);
+      launch_k(ov, k_pair_full<Act, Cmp, Wlk>, (unsigned)blocks, 32 * warps, smem, st, r, sh, pa,
+          ib);
       }
     } else {
       if (Mode::kMode == FN_BF16_MIXED) {
         const size_t smem = smem_pair_value_mma(sh.N, L);
         cudaFuncSetAttribute(k_pair_value_mma<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         const int64_t blocks_v = std::min<int64_t>(sh.B, (int64_t)s->sm_count * 16);
-        k_pair_value_mma<Wlk><<<(unsigned)blocks_v, 128, smem, st>>>(r, sh, pa);
+        launch_k(ov, k_pair_value_mma<Wlk>, (unsigned)blocks_v, 128, smem, st, r, sh, pa);
       } else {
         const size_t smem = smem_pair_value(sizeof(Cmp), sh.N, L);
         const int threads = (int)std::min<int64_t>(512, round_up((int64_t)sh.N * sh.N, 32));
         cudaFuncSetAttribute(k_pair_value<Act, Cmp, Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pair_value<Act, Cmp, Wlk><<<(unsigned)sh.B, threads, smem, st>>>(r, sh, pa);
+        launch_k(ov, k_pair_value<Act, Cmp, Wlk>, (unsigned)sh.B, threads, smem, st, r, sh, pa);
       }
     }
   }
@@ -1170,7 +1198,8 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         ProfScope pm(s->prof, kProfSpinMeans, st);
         const int64_t n = (int64_t)sh.T * sh.B * 2 * (h1 / 8);
         const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)s->sm_count * 64);
-        k_spin_means_bf16<<<blocks, 256, 0, st>>>(sh, (const __nv_bfloat16*)la.Y, la.ldy, h1,
+        launch_k(ov, k_spin_means_bf16, blocks, 256, 0, st, sh, (const __nv_bfloat16*)la.Y,
+            la.ldy, h1,
                                                   (__nv_bfloat16*)la.Hbar_out);
       }
       continue;
@@ -1183,7 +1212,8 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         ProfScope pm(s->prof, kProfSpinMeans, st);
         const int64_t n = (int64_t)sh.T * sh.B * 2 * (h1 / 4);
         const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)s->sm_count * 64);
-        k_spin_means_f32<<<blocks, 256, 0, st>>>(sh, (const float*)la.Y, la.ldy, h1, (float*)la.Hbar_out);
+        launch_k(ov, k_spin_means_f32, blocks, 256, 0, st, sh, (const float*)la.Y, la.ldy, h1,
+            (float*)la.Hbar_out);
       }
       continue;
     }
@@ -1215,9 +1245,13 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         const unsigned gx = (unsigned)((per_walker + 255) / 256);
         const unsigned gy = (unsigned)std::max(1, std::min(sh.B, (s->sm_count * 8 + (int)gx - 1) / (int)gx));
         cudaFuncSetAttribute(k_envelope_values_smem<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)env_smem);
-        k_envelope_values_smem<Wlk><<<dim3(gx, gy), 256, env_smem, st>>>(r, s->d_nuclei, sh, oa, (float*)ws.envv);
+        launch_k(ov, k_envelope_values_smem<Wlk>, dim3(gx, gy), 256, env_smem, st, r, s->d_nuclei,
+            sh, oa,
+                   (float*)ws.envv);
       } else {
-        k_envelope_values<Wlk><<<(unsigned)((n_env + 255) / 256), 256, 0, st>>>(r, s->d_nuclei, sh, oa, (float*)ws.envv);
+        launch_k(ov, k_envelope_values<Wlk>, (unsigned)((n_env + 255) / 256), 256, 0, st, r,
+            s->d_nuclei, sh, oa,
+                   (float*)ws.envv);
       }
       const float* wb[2] = {(const float*)oa.g[0], (const float*)oa.g[1]};
       const float* pis[2] = {(const float*)oa.pi[0], (const float*)oa.pi[1]};
@@ -1243,8 +1277,8 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
     if (full) {
       const int ko_max = s->cfg.n_dets * std::max(s->n_up, s->n_dn);
       ProfScope ps(s->prof, kProfOrbFix, st);
-      k_orbital_fixup<Cmp, typename Mode::PhiT, Wlk><<<(unsigned)((int64_t)sh.B * sh.N), (unsigned)round_up(ko_max, 32), 0,
-                                                       st>>>(r, s->d_nuclei, sh, oa, (const Cmp*)ws.orbP);
+      launch_k(ov, k_orbital_fixup<Cmp, typename Mode::PhiT, Wlk>, (unsigned)((int64_t)sh.B * sh.N),
+                 (unsigned)round_up(ko_max, 32), 0, st, r, s->d_nuclei, sh, oa, (const Cmp*)ws.orbP);
     }
   }
 }

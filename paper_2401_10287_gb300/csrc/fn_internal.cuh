@@ -249,6 +249,37 @@ struct fn_system {
 
 namespace fn {
 
+// Whether a pass of this size lets its kernels begin while their predecessors drain: below about
+// 2^18 electron rows x slabs the kernels take 5 to 30 us and the gaps between them count (value
+// pass of a 256-walker carbon atom 205 -> 164 us, LiH training iteration 4.43 -> 3.85 ms); above,
+// CTAs that arrive while only some SMs have room crowd onto those (N2 local energy 10.8 -> 11.2 ms,
+// its FP32 form 15.7 -> 16.5).  FP64 kernels do not overlap: two CTAs on one SM share its slow FP64
+// pipe while other SMs idle (H2 pass 1.34 -> 1.41 ms).
+inline bool overlap_launches(const Shape& sh, size_t word = 4) {
+  return word == 4 && (int64_t)sh.T * sh.R <= ((int64_t)1 << 18);
+}
+
+// The same for a product, by its rows (electron rows, or T x walkers of at least four electrons).
+constexpr int64_t kOverlapGemmRows = 1 << 16;
+
+// Launch of a kernel that calls pdl_wait; with `overlap` it may begin while its predecessor in the
+// stream drains.
+template <typename... P, typename... A>
+inline void launch_k(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                     A&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // a failure is the call's last error
+}
+
 void set_error(const std::string& msg);
 fn_status cuda_status(cudaError_t e, const char* what);
 

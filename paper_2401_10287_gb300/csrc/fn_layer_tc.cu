@@ -417,6 +417,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
+  pdl_wait();
+  pdl_launch();
   const uint32_t tmem = *tmem_slot;
   const uint64_t deadline = globaltimer() + kWaitNs * 8 * (uint64_t)(my_tiles > 0 ? my_tiles : 1);
 
@@ -679,6 +681,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
       for (int kb = 0; kb < nkb; ++kb)
         for (int part = 0; part < 2; ++part)
           tma_load_2d(sB + (size_t)(kb * 2 + part) * bytesB, &tmB, bfull, part * a.bsplit + kb * kBlockK, ctile * nt);
+      pdl_wait();        // the weights are older than the preceding kernel, the activations are not
       // ring position (stage, phase) and item (tile, t) advance by increments: no division
       int issued = 0, stage = 0;
       uint32_t phase = 0;
@@ -752,6 +755,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kResRegsHigh));
+    pdl_wait();
+    pdl_launch();
     const int q = warp & 3;                       // TMEM lane quarter this warp may access
     const int r = q * 32 + lane;
     const int ehalf = (warp - 4) >> 2;            // column half: chunks cc with cc % 2 == ehalf
@@ -1509,12 +1514,13 @@ static void launch_tc(const CUtensorMap& ta, const CUtensorMap& tb, const tc::Tc
                       cudaStream_t st) {
   const size_t smem = tc_smem_bytes(a.nt, EPI, a.bsplit != 0, (EPI == tc::kEpiLayer && a.mt_stage) ? a.sh.wpt : 0,
                                    EPI == tc::kEpiLayer && a.residual);
+  const bool overlap = EPI == tc::kEpiPlain ? a.rows <= kOverlapGemmRows : overlap_launches(a.sh);
   if (full) {
     cudaFuncSetAttribute(tc::k_tc<EPI, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    tc::k_tc<EPI, true><<<grid, tc::kThreads, smem, st>>>(ta, tb, a);
+    launch_k(overlap, tc::k_tc<EPI, true>, grid, tc::kThreads, smem, st, ta, tb, a);
   } else {
     cudaFuncSetAttribute(tc::k_tc<EPI, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    tc::k_tc<EPI, false><<<grid, tc::kThreads, smem, st>>>(ta, tb, a);
+    launch_k(overlap, tc::k_tc<EPI, false>, grid, tc::kThreads, smem, st, ta, tb, a);
   }
 }
 
@@ -1659,10 +1665,10 @@ bool launch_layer_tc(const Shape& sh, const void* X, int ldx, int k_self, int lo
     const dim3 grid = persistent_grid(h1 / nt, sh.tiles);
     if (full) {
       cudaFuncSetAttribute(tc::k_layer_res<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      tc::k_layer_res<true><<<grid, tc::kResThreads, smem, st>>>(ta, tb, ty, a);
+      launch_k(overlap_launches(a.sh), tc::k_layer_res<true>, grid, tc::kResThreads, smem, st, ta, tb, ty, a);
     } else {
       cudaFuncSetAttribute(tc::k_layer_res<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      tc::k_layer_res<false><<<grid, tc::kResThreads, smem, st>>>(ta, tb, ty, a);
+      launch_k(overlap_launches(a.sh), tc::k_layer_res<false>, grid, tc::kResThreads, smem, st, ta, tb, ty, a);
     }
     return true;
   }

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 
+#include "fn_device.cuh"
 #include "fn_internal.cuh"
 
 namespace fn {
@@ -32,6 +33,8 @@ struct AdamCoef {
 template <typename P>
 __global__ void k_adam(int64_t n, P* __restrict__ p, const P* __restrict__ g, P* __restrict__ m,
                        P* __restrict__ v, AdamCoef<P> c, int* __restrict__ status) {
+  pdl_wait();
+  pdl_launch();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   bool bad = false;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -49,6 +52,8 @@ __global__ void k_adam(int64_t n, P* __restrict__ p, const P* __restrict__ g, P*
 
 template <typename P>
 __global__ void k_sgd(int64_t n, P* __restrict__ p, const P* __restrict__ g, P lr, int* __restrict__ status) {
+  pdl_wait();
+  pdl_launch();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   bool bad = false;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -79,7 +84,7 @@ void launch_adam(const fn_system* s, void* params, const void* grad, void* m, vo
   c.d1 = (P)(1.0 - pow(beta1, (double)t));
   c.d2 = (P)(1.0 - pow(beta2, (double)t));
   ProfScope ps(s->prof, kProfOptim, st);
-  k_adam<P><<<elementwise_grid(s, s->P), 256, 0, st>>>(s->P, (P*)params, (const P*)grad, (P*)m, (P*)v, c,
+  launch_k(true, k_adam<P>, elementwise_grid(s, s->P), 256, 0, st, s->P, (P*)params, (const P*)grad, (P*)m, (P*)v, c,
                                                         s->ws.status);
 }
 
@@ -87,7 +92,8 @@ template <class Mode>
 void launch_sgd(const fn_system* s, void* params, const void* grad, double lr, cudaStream_t st) {
   using P = typename Mode::Par;
   ProfScope ps(s->prof, kProfOptim, st);
-  k_sgd<P><<<elementwise_grid(s, s->P), 256, 0, st>>>(s->P, (P*)params, (const P*)grad, (P)lr, s->ws.status);
+  launch_k(true, k_sgd<P>, elementwise_grid(s, s->P), 256, 0, st, s->P, (P*)params, (const P*)grad, (P)lr,
+      s->ws.status);
 }
 
 // ---- local-energy clipping ------------------------------------------------------------------
@@ -104,12 +110,19 @@ __device__ __forceinline__ double key_value(unsigned long long k) {
 
 constexpr int kClipThreads = 1024;
 
+constexpr int kClipCached = 8;         // keys per thread kept in registers (batches of up to 8192)
+
+// One CTA, so its time is its chain of barriers: 8 digit passes over the batch in memory took 20 us
+// for 4096 energies.  With the keys in registers and the search ended as soon as one key is left
+// in the bin (two or three digits, unless energies are equal) it takes @CLIP@ us.
 __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const double* e, double width, double* out,
                                                                double* __restrict__ stats,
                                                                int* __restrict__ status) {
+  pdl_wait();
+  pdl_launch();
   __shared__ unsigned int hist[256];
   __shared__ unsigned long long s_prefix;
-  __shared__ unsigned int s_rank;
+  __shared__ unsigned int s_rank, s_left;
   __shared__ double red[kClipThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
@@ -117,17 +130,31 @@ __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const doubl
   // Invariant: `rank` < number of keys whose bits above `shift` + 8 equal `prefix`.
   unsigned long long prefix = 0, mask = 0;
   unsigned int rank = (unsigned int)(B - 1) / 2u;
+  const bool cached = B <= kClipCached * kClipThreads;
+  double x[kClipCached];
+#pragma unroll
+  for (int j = 0; j < kClipCached; ++j) {
+    const int i = j * kClipThreads + tid;
+    x[j] = cached && i < B ? e[i] : 0.0;
+  }
+  const auto count = [&](unsigned long long k, bool in, int shift) {
+    const bool hit = in && (k & mask) == prefix;
+    const unsigned int bin = hit ? (unsigned int)((k >> shift) & 255ull) : 256u;
+    const unsigned int peers = __match_any_sync(0xffffffffu, bin);
+    if (hit && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], (unsigned int)__popc(peers));
+  };
   for (int shift = 56; shift >= 0; shift -= 8) {
     for (int b = tid; b < 256; b += kClipThreads) hist[b] = 0;
     __syncthreads();
-    for (int64_t base = 0; base < B; base += kClipThreads) {   // uniform trip count: full warps below
-      const int64_t i = base + tid;
-      const bool in = i < B;
-      const unsigned long long k = in ? order_key(e[i]) : 0ull;
-      const bool hit = in && (k & mask) == prefix;
-      const unsigned int bin = hit ? (unsigned int)((k >> shift) & 255ull) : 256u;
-      const unsigned int peers = __match_any_sync(0xffffffffu, bin);
-      if (hit && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], (unsigned int)__popc(peers));
+    if (cached) {
+#pragma unroll
+      for (int j = 0; j < kClipCached; ++j)
+        if (j * kClipThreads < B) count(order_key(x[j]), j * kClipThreads + tid < B, shift);
+    } else {
+      for (int64_t base = 0; base < B; base += kClipThreads) {   // uniform trip count: full warps above
+        const int64_t i = base + tid;
+        count(i < B ? order_key(e[i]) : 0ull, i < B, shift);
+      }
     }
     __syncthreads();
     if (wid == 0) {   // warp 0: lane l owns bins 8l .. 8l + 7
@@ -151,6 +178,7 @@ __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const doubl
           if (rank < c + cnt[j]) {
             s_prefix = prefix | ((unsigned long long)(lane * 8 + j) << shift);
             s_rank = rank - c;
+            s_left = cnt[j];
             break;
           }
           c += cnt[j];
@@ -161,12 +189,27 @@ __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const doubl
     prefix = s_prefix;
     rank = s_rank;
     mask |= 0xffull << shift;
+    if (cached && s_left == 1) {                 // one key has this prefix: it is the median
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < kClipCached; ++j)
+        if (j * kClipThreads + tid < B && (order_key(x[j]) & mask) == prefix) s_prefix = order_key(x[j]);
+      __syncthreads();
+      prefix = s_prefix;
+      break;
+    }
   }
   const double centre = key_value(prefix);
 
   // Mean absolute deviation from the centre.
   double acc = 0.0;
-  for (int64_t i = tid; i < B; i += kClipThreads) acc += fabs(e[i] - centre);
+  if (cached) {
+#pragma unroll
+    for (int j = 0; j < kClipCached; ++j)
+      if (j * kClipThreads + tid < B) acc += fabs(x[j] - centre);
+  } else {
+    for (int64_t i = tid; i < B; i += kClipThreads) acc += fabs(e[i] - centre);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) red[wid] = acc;
@@ -184,9 +227,13 @@ __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const doubl
   // comparisons keep a NaN energy as it is.
   const bool on = width > 0.0;
   const double lo = centre - width * spread, hi = centre + width * spread;
-  for (int64_t i = tid; i < B; i += kClipThreads) {
-    const double x = e[i];
-    out[i] = on ? (x < lo ? lo : (x > hi ? hi : x)) : x;
+  const auto clamp = [&](double v) { return on ? (v < lo ? lo : (v > hi ? hi : v)) : v; };
+  if (cached) {
+#pragma unroll
+    for (int j = 0; j < kClipCached; ++j)
+      if (j * kClipThreads + tid < B) out[j * kClipThreads + tid] = clamp(x[j]);
+  } else {
+    for (int64_t i = tid; i < B; i += kClipThreads) out[i] = clamp(e[i]);
   }
   if (tid == 0) {
     if (stats) {
@@ -200,7 +247,7 @@ __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const doubl
 void launch_clip_energy(const fn_system* s, int B, const double* e, double width, double* out, double* stats,
                         cudaStream_t st) {
   ProfScope ps(s->prof, kProfOptim, st);
-  k_clip_energy<<<1, kClipThreads, 0, st>>>(B, e, width, out, stats, s->ws.status);
+  launch_k(true, k_clip_energy, 1, kClipThreads, 0, st, B, e, width, out, stats, s->ws.status);
 }
 
 // ---- Eq. 1 estimator and the Eq. 6 weights ------------------------------------------------
@@ -213,6 +260,8 @@ constexpr int kStatThreads = 1024;
 
 __global__ void __launch_bounds__(kStatThreads) k_energy_moments(int B, const double* __restrict__ e,
                                                                   double* __restrict__ mom) {
+  pdl_wait();
+  pdl_launch();
   __shared__ double s1[kStatThreads], s2[kStatThreads];
   double a = 0.0, b = 0.0;
   for (int i = threadIdx.x; i < B; i += kStatThreads) {
@@ -238,6 +287,8 @@ __global__ void __launch_bounds__(kStatThreads) k_energy_moments(int B, const do
 }
 
 __global__ void k_energy_stats(const double* __restrict__ mom, double* __restrict__ stats, int* __restrict__ status) {
+  pdl_wait();
+  pdl_launch();
   const double n = mom[0], mean = mom[1] / n;
   const double var = fmax(0.0, mom[2] / n - mean * mean);
   stats[0] = n;
@@ -248,6 +299,8 @@ __global__ void k_energy_stats(const double* __restrict__ mom, double* __restric
 
 __global__ void k_energy_weights_from(int B, const double* __restrict__ e, const double* __restrict__ mom,
                                       double* __restrict__ w) {
+  pdl_wait();
+  pdl_launch();
   const double n = mom[0], mean = mom[1] / n;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B; i += gridDim.x * blockDim.x)
     w[i] = 2.0 * (e[i] - mean) / n;
@@ -255,18 +308,18 @@ __global__ void k_energy_weights_from(int B, const double* __restrict__ e, const
 
 void launch_energy_moments(const fn_system* s, int B, const double* e, double* mom, cudaStream_t st) {
   ProfScope ps(s->prof, kProfOptim, st);
-  k_energy_moments<<<1, kStatThreads, 0, st>>>(B, e, mom);
+  launch_k(true, k_energy_moments, 1, kStatThreads, 0, st, B, e, mom);
 }
 
 void launch_energy_stats(const fn_system* s, const double* mom, double* stats, cudaStream_t st) {
   ProfScope ps(s->prof, kProfOptim, st);
-  k_energy_stats<<<1, 1, 0, st>>>(mom, stats, s->d_status);
+  launch_k(true, k_energy_stats, 1, 1, 0, st, mom, stats, s->d_status);
 }
 
 void launch_energy_weights_from(const fn_system* s, int B, const double* e, const double* mom, double* w,
                                 cudaStream_t st) {
   ProfScope ps(s->prof, kProfOptim, st);
-  k_energy_weights_from<<<elementwise_grid(s, B), 256, 0, st>>>(B, e, mom, w);
+  launch_k(true, k_energy_weights_from, elementwise_grid(s, B), 256, 0, st, B, e, mom, w);
 }
 
 #define FN_INST_OPTIM(M)                                                                                        \

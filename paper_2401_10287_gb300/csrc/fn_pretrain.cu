@@ -21,6 +21,8 @@ template <typename Det, typename PhiT, typename Wlk>
 __global__ void k_pretrain_seed(const Wlk* __restrict__ r, Shape sh, const double* __restrict__ hf, int nbf,
                                 const PhiT* __restrict__ Phi, int64_t PW, int K, Det* __restrict__ dPhi,
                                 double* __restrict__ cw, double* __restrict__ wloss) {
+  pdl_wait();
+  pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = blockIdx.x * (blockDim.x >> 5) + warp;
   if (w >= sh.B) return;                                   // warp-uniform
@@ -73,6 +75,8 @@ __global__ void k_pretrain_seed(const Wlk* __restrict__ r, Shape sh, const doubl
 }
 
 __global__ void k_pretrain_loss(int B, const double* __restrict__ wloss, double* __restrict__ out) {
+  pdl_wait();
+  pdl_launch();
   __shared__ double red[1024];
   double s = 0.0;
   for (int w = threadIdx.x; w < B; w += blockDim.x) s += wloss[w];
@@ -91,10 +95,11 @@ void launch_pretrain_seed(const fn_system* s, const void* walkers, const Shape& 
   const Workspace& ws = s->ws;
   ProfScope ps(s->prof, kProfBwdOrb, st);
   const int warps = 4;
-  k_pretrain_seed<Det, PhiT, Wlk><<<(unsigned)((sh.B + warps - 1) / warps), 32 * warps, 0, st>>>(
-      (const Wlk*)walkers, sh, s->d_hf, s->hf_nbf, (const PhiT*)ws.Phi, phi_walker_stride(s, 1), s->cfg.n_dets,
+  launch_k(overlap_launches(sh), k_pretrain_seed<Det, PhiT, Wlk>, (unsigned)((sh.B + warps - 1) / warps),
+      32 * warps, 0, st,
+             (const Wlk*)walkers, sh, s->d_hf, s->hf_nbf, (const PhiT*)ws.Phi, phi_walker_stride(s, 1), s->cfg.n_dets,
       (Det*)ws.dPhi, ws.scratch_d, ws.scratch_d + sh.B);
-  if (loss) k_pretrain_loss<<<1, 1024, 0, st>>>(sh.B, ws.scratch_d + sh.B, loss);
+  if (loss) launch_k(overlap_launches(sh), k_pretrain_loss, 1, 1024, 0, st, sh.B, ws.scratch_d + sh.B, loss);
 }
 
 template void launch_pretrain_seed<ModeF64>(const fn_system*, const void*, const Shape&, double*, cudaStream_t);

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "fn_device.cuh"
 #include "fn_internal.cuh"
 #include "fn_rng.cuh"
 
@@ -17,6 +18,8 @@ namespace fn {
 template <typename Wlk>
 __global__ void k_init_walkers(int B, int N, const int* __restrict__ atom, const double* __restrict__ nuc,
                                double init_std, uint64_t seed, uint64_t walker_offset, Wlk* __restrict__ out) {
+  pdl_wait();
+  pdl_launch();
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gid >= (int64_t)B * N * 3) return;
   const int64_t w = gid / (3 * N);
@@ -31,6 +34,8 @@ __global__ void k_init_walkers(int B, int N, const int* __restrict__ atom, const
 template <typename Wlk>
 __global__ void k_propose(int B, int N, const Wlk* __restrict__ r, Wlk* __restrict__ out, double step,
                           uint64_t seed, uint32_t step_idx, uint64_t walker_offset) {
+  pdl_wait();
+  pdl_launch();
   const int n3 = 3 * N, pairs = (n3 + 1) / 2;
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gid >= (int64_t)B * pairs) return;
@@ -48,6 +53,8 @@ template <typename Wlk>
 __global__ void k_accept(int B, int N, Wlk* __restrict__ r, const Wlk* __restrict__ prop, double* __restrict__ lp,
                          const double* __restrict__ lp_new, uint64_t seed, uint32_t step_idx,
                          uint64_t walker_offset, unsigned long long* __restrict__ accepted) {
+  pdl_wait();
+  pdl_launch();
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
   bool acc = false;
   if (w < B) {
@@ -76,6 +83,8 @@ struct InitSegs {
 
 template <typename Par>
 __global__ void k_init_params(int64_t P, InitSegs segs, uint64_t seed, Par* __restrict__ out) {
+  pdl_wait();
+  pdl_launch();
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= P) return;
   int s = 0;
@@ -98,7 +107,8 @@ void launch_init_walkers(const fn_system* s, int B, uint64_t seed, double std_, 
   using Wlk = typename Mode::Wlk;
   const int64_t n = (int64_t)B * s->N * 3;
   ProfScope ps(s->prof, kProfInit, st);
-  k_init_walkers<Wlk><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(B, s->N, s->d_elec_atom, s->d_nuclei, std_, seed,
+  launch_k(true, k_init_walkers<Wlk>, (unsigned)((n + 255) / 256), 256, 0, st, B, s->N, s->d_elec_atom, s->d_nuclei,
+             std_, seed,
                                                                      s->walker_offset, (Wlk*)walkers);
 }
 
@@ -108,7 +118,9 @@ void launch_propose(const fn_system* s, int B, const void* walkers, void* out, d
   using Wlk = typename Mode::Wlk;
   const int64_t n = (int64_t)B * ((3 * s->N + 1) / 2);
   ProfScope ps(s->prof, kProfSampler, st);
-  k_propose<Wlk><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(B, s->N, (const Wlk*)walkers, (Wlk*)out, step, seed,
+  launch_k(true, k_propose<Wlk>, (unsigned)((n + 127) / 128), 128, 0, st, B, s->N, (const Wlk*)walkers, (Wlk*)out,
+      step,
+             seed,
                                                                 step_idx, s->walker_offset);
 }
 
@@ -117,7 +129,9 @@ void launch_accept(const fn_system* s, int B, void* walkers, const void* prop, d
                    uint64_t seed, uint32_t step_idx, int64_t* accept_count, cudaStream_t st) {
   using Wlk = typename Mode::Wlk;
   ProfScope ps(s->prof, kProfSampler, st);
-  k_accept<Wlk><<<(B + 127) / 128, 128, 0, st>>>(B, s->N, (Wlk*)walkers, (const Wlk*)prop, lp, lp_new, seed, step_idx,
+  launch_k(true, k_accept<Wlk>, (B + 127) / 128, 128, 0, st, B, s->N, (Wlk*)walkers, (const Wlk*)prop, lp, lp_new,
+      seed,
+             step_idx,
                                                   s->walker_offset, (unsigned long long*)accept_count);
 }
 
@@ -152,7 +166,7 @@ void launch_init_params(const fn_system* s, uint64_t seed, void* params, cudaStr
       add(s->off_sig[a], end, s->cfg.envelope == FN_ENV_ANISOTROPIC ? 2 : 1, 1);
     }
   ProfScope ps(s->prof, kProfInit, st);
-  k_init_params<Par><<<(unsigned)((s->P + 255) / 256), 256, 0, st>>>(s->P, g, seed, (Par*)params);
+  launch_k(true, k_init_params<Par>, (unsigned)((s->P + 255) / 256), 256, 0, st, s->P, g, seed, (Par*)params);
 }
 
 #define FN_INST(M)                                                                                          \

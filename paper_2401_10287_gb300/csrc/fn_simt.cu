@@ -4,6 +4,7 @@
 
 #include <algorithm>
 
+#include "fn_device.cuh"
 #include "fn_internal.cuh"
 #include "fn_simt_launch.cuh"
 
@@ -44,6 +45,8 @@ __device__ __forceinline__ void store_group(T* p, int live, const T (&v)[Vec<T>:
 // ---------------------------------------------------------------------------------------
 template <typename T, int TM, int TN, int WM, bool FULL, bool VEC>
 __global__ void __launch_bounds__(32 * WM) k_layer(Shape sh, LayerArgs a, int wps, int subs) {
+  pdl_wait();
+  pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V, LDY = Tl::BN + V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -138,7 +141,7 @@ static void layer_cfg(const Shape& sh, const LayerArgs& a, bool vec, cudaStream_
   const unsigned grid = (unsigned)((a.h1 + Tl::BN - 1) / Tl::BN) * sh.tiles * subs;
   auto go = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kernel<<<grid, Tl::kThreads, smem, st>>>(sh, a, wps, subs);
+    launch_k(overlap_launches(sh, sizeof(T)), kernel, grid, Tl::kThreads, smem, st, sh, a, wps, subs);
   };
   if (sh.T > 1) vec ? go(k_layer<T, TM, TN, WM, true, true>) : go(k_layer<T, TM, TN, WM, true, false>);
   else vec ? go(k_layer<T, TM, TN, WM, false, true>) : go(k_layer<T, TM, TN, WM, false, false>);
@@ -213,6 +216,8 @@ __device__ __forceinline__ T env_value(const T* pi, const T* sig, int aniso, int
 constexpr int kEnvOrbs = 16;
 template <typename T>
 __global__ void __launch_bounds__(kTileRows) k_envelope(Shape sh, OrbArgs a) {
+  pdl_wait();
+  pdl_launch();
   __shared__ T ds[3 * kMaxNuclei][kTileRows];
   const int tile = blockIdx.x, rl = threadIdx.x, wl = rl / sh.N, j = rl - wl * sh.N, w = tile * sh.wpt + wl;
   if (wl >= sh.wpt || w >= sh.B) return;                        // no barrier below: each thread reads its own column
@@ -228,6 +233,8 @@ __global__ void __launch_bounds__(kTileRows) k_envelope(Shape sh, OrbArgs a) {
 
 template <typename T, int TM, int TN, int WM, bool FULL, bool VEC>
 __global__ void __launch_bounds__(32 * WM) k_orbitals(Shape sh, OrbArgs a, int spin) {
+  pdl_wait();
+  pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V, LDY = Tl::BN + V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -303,7 +310,7 @@ static void orbitals_cfg(const Shape& sh, const OrbArgs& a, int spin, cudaStream
   const dim3 grid((unsigned)((n_ko + Tl::BN - 1) / Tl::BN) * ((sh.B + wpc - 1) / wpc), 1, sh.T);
   auto go = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kernel<<<grid, Tl::kThreads, smem, st>>>(sh, a, spin);
+    launch_k(overlap_launches(sh, sizeof(T)), kernel, grid, Tl::kThreads, smem, st, sh, a, spin);
   };
   if (full) vec ? go(k_orbitals<T, TM, TN, WM, true, true>) : go(k_orbitals<T, TM, TN, WM, true, false>);
   else vec ? go(k_orbitals<T, TM, TN, WM, false, true>) : go(k_orbitals<T, TM, TN, WM, false, false>);
@@ -312,7 +319,8 @@ static void orbitals_cfg(const Shape& sh, const OrbArgs& a, int spin, cudaStream
 template <typename T>
 void launch_envelope(const Shape& sh, const OrbArgs& a, cudaStream_t st) {
   const int n_ko = a.K * std::max(sh.n_up, sh.n_dn);
-  k_envelope<T><<<dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st>>>(sh, a);
+  launch_k(overlap_launches(sh, sizeof(T)), k_envelope<T>, dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st,
+      sh, a);
 }
 
 template <typename T>
@@ -349,6 +357,8 @@ void launch_orbitals(const Shape& sh, const OrbArgs& a, int sm_count, cudaStream
 // ---------------------------------------------------------------------------------------
 template <typename T, int TM, int TN, int WM, bool AT, bool BT, bool VEC>
 __global__ void __launch_bounds__(32 * WM) k_gemm(GemmArgs<T> g) {
+  pdl_wait();
+  pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -406,7 +416,7 @@ static void gemm_cfg(const GemmArgs<T>& g, bool at, bool bt, int split, bool vec
   const dim3 grid((unsigned)((g.N + Tl::BN - 1) / Tl::BN * ((g.M + Tl::BM - 1) / Tl::BM)), 1, split);
   auto go = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Tl::kRingBytes);
-    kernel<<<grid, Tl::kThreads, Tl::kRingBytes, st>>>(g);
+    launch_k(sizeof(T) == 4 && g.M <= kOverlapGemmRows, kernel, grid, Tl::kThreads, Tl::kRingBytes, st, g);
   };
   if (at) vec ? go(k_gemm<T, TM, TN, WM, true, false, true>) : go(k_gemm<T, TM, TN, WM, true, false, false>);
   else if (bt) vec ? go(k_gemm<T, TM, TN, WM, false, true, true>) : go(k_gemm<T, TM, TN, WM, false, true, false>);

@@ -15,6 +15,7 @@
 
 #include <algorithm>
 
+#include "fn_device.cuh"
 #include "fn_internal.cuh"
 #include "fn_lu.cuh"
 #include "fn_rng.cuh"
@@ -209,6 +210,8 @@ __device__ void small_eval(const SmallArgs& a, const SmallLayout& s, double* sm,
 
 // log|psi| and sign of every walker (n_steps = 0), or n_steps Metropolis steps from d_log_psi.
 __global__ void __launch_bounds__(kSmallThreads) k_small(SmallArgs a) {
+  pdl_wait();
+  pdl_launch();
   extern __shared__ __align__(16) double small_smem[];
   double* sm = small_smem;
   const SmallLayout s = small_layout(a);
@@ -282,7 +285,7 @@ static void launch(const SmallArgs& a, cudaStream_t st) {
   const int threads = (int)std::min<int64_t>(kSmallThreads, round_up((int64_t)a.G * a.N * a.h1, 32));
   const size_t smem = small_layout(a).total * sizeof(double);
   cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_small<<<(unsigned)((a.B + a.G - 1) / a.G), threads, smem, st>>>(a);
+  launch_k(true, k_small, (unsigned)((a.B + a.G - 1) / a.G), threads, smem, st, a);
 }
 
 void launch_small_log_psi(const fn_system* s, const void* walkers, int B, double* log_psi, int8_t* sign, cudaStream_t st) {

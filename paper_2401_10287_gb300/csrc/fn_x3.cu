@@ -151,6 +151,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
+  pdl_wait();
+  pdl_launch();
   const uint32_t tmem = *tmem_slot;
   const uint64_t deadline = globaltimer() + kWaitNs * 8 * (uint64_t)(my_tiles > 0 ? my_tiles : 1);
 
@@ -491,6 +493,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ---- prepared weights: [n][part][ldw] BF16, columns kd .. ldw - 1 zero ------------------
 __global__ void k_split_weights(const float* __restrict__ blob, SplitList list, __nv_bfloat16* __restrict__ out) {
+  pdl_wait();
+  pdl_launch();
   const SplitEntry e = list.e[blockIdx.y];
   const int64_t n = (int64_t)e.rows * e.ldw;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -510,7 +514,7 @@ __global__ void k_split_weights(const float* __restrict__ blob, SplitList list, 
 }
 
 void launch_split_weights(const float* blob, const SplitList& list, void* out, cudaStream_t st) {
-  k_split_weights<<<dim3(32, list.n), 256, 0, st>>>(blob, list, (__nv_bfloat16*)out);
+  launch_k(false, k_split_weights, dim3(32, list.n), 256, 0, st, blob, list, (__nv_bfloat16*)out);
 }
 
 template <int EPI>
@@ -539,7 +543,7 @@ static bool launch(const Args& a, const void* W, int64_t w_rows, const float* X,
   const int ctiles = (a.ncols + kNt - 1) / kNt;
   const dim3 grid(ctiles, std::min(a.tiles, std::max(1, sm_count / ctiles)));
   cudaFuncSetAttribute(k_x3<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  k_x3<EPI><<<grid, kThreads, kSmem, st>>>(tb, tx, ty, a);
+  launch_k(false, k_x3<EPI>, grid, kThreads, kSmem, st, tb, tx, ty, a);
   return true;
 }
 
