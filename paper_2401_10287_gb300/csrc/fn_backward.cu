@@ -20,6 +20,7 @@
 
 #include "fn_device.cuh"
 #include "fn_internal.cuh"
+#include "fn_pair.cuh"
 #include "fn_simt_launch.cuh"
 
 namespace fn {
@@ -513,6 +514,10 @@ __global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* __restrict__ r, Sha
 // the 32 x 32 output) and the input gradient dz W (pairs as rows), then one coalesced pass adds
 // dG^{l+1} (residual, l >= 1) and the layer input's spin-mean gradient, as k_pair_bwd does.
 
+// Rows of 32 words with permuted 8-word groups (pair_at) as in the forward pair kernels, a warp per
+// pair and a lane per channel in the elementwise passes (element-wise index divisions and row strides
+// of 33 words kept the kernel at 32 % issue and 0.2 TB/s).  N2, 4096 walkers, four levels: 1.39 ->
+// 0.81 ms.
 template <typename Wlk>
 __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r, Shape sh, PairBwdArgs a) {
   pdl_wait();
@@ -524,8 +529,8 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
   const bool has_layer = a.l < a.L - 1;
   __nv_bfloat16* wth = (__nv_bfloat16*)smem_raw;                 // [32 c][kBwdWLd]: bf16(W[q][c]) at [c][q]
   __nv_bfloat16* wtl = wth + 32 * kBwdWLd;
-  float* gin_s = (float*)(wtl + 32 * kBwdWLd);                   // [NPp][33] g^l, later dz W
-  float* dz_s = gin_s + NPp * 33;                                // [NPp][33]
+  float* gin_s = (float*)(wtl + 32 * kBwdWLd);                   // [NPp][32] g^l, later dz W
+  float* dz_s = gin_s + NPp * 32;                                // [NPp][32]
   if (has_layer) {
     const float* W = (const float*)a.W;                          // [h2][d_g]
     for (int e = tid; e < 32 * 32; e += blockDim.x) {
@@ -535,129 +540,120 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
       wth[c * kBwdWLd + q] = h;
       wtl[c * kBwdWLd + q] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
-    // padding rows, and the columns beyond the widths, stay zero in dz_s; gin_s is written whole
-    for (int e = tid; e < NPp * 33; e += blockDim.x) { gin_s[e] = 0.f; dz_s[e] = 0.f; }
+    // padding rows stay zero in both; the products below write zero over zero there
+    for (int e = NP * 32 + tid; e < NPp * 32; e += blockDim.x) { gin_s[e] = 0.f; dz_s[e] = 0.f; }
   }
   // CTAs loop over walkers: the weights are staged once, and the weight gradients stay in
   // registers until the end (one atomic per element and CTA instead of one per walker)
   float c2[2][4] = {}, dc = 0.f;
   const int q0 = (warp >> 1) * 16, nb0 = (warp & 1) * 2;
+  const bool in_h2 = lane < a.h2, in_dg = lane < a.d_g;
+  const float n_spin[2] = {(float)sh.n_up, (float)sh.n_dn};
   for (int w = blockIdx.x; w < sh.B; w += gridDim.x) {
-  const float* dG = (const float*)a.dG + (int64_t)w * NP * a.h2;
-  if (has_layer) {
-    __syncthreads();
-    const Wlk* rw = r + (int64_t)w * N * 3;
-    const float* gin_g = a.g_in ? (const float*)a.g_in + (int64_t)w * NP * a.h2 : nullptr;
-    const float* gout_g = (const float*)a.g_out + (int64_t)w * NP * a.h2;
-    // four elements per thread and round: all their global loads are issued before any use
-    for (int e0 = tid; e0 < NP * 32; e0 += 4 * blockDim.x) {
-      float gin[4], gout[4], dg[4];
+    float* dG = (float*)a.dG + (int64_t)w * NP * a.h2 + lane;
+    if (has_layer) {
+      __syncthreads();
+      const Wlk* rw = r + (int64_t)w * N * 3;
+      const float* gin_g = a.g_in ? (const float*)a.g_in + (int64_t)w * NP * a.h2 + lane : nullptr;
+      const float* gout_g = (const float*)a.g_out + (int64_t)w * NP * a.h2 + lane;
+      // eight pairs per warp and round: all their global loads are issued before any use
+      for (int pb = warp; pb < NP; pb += 32) {
+        float gin[8], gout[8], dg[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * blockDim.x;
-        const int p = e >> 5, c = e & 31;
-        gin[u] = 0.f; gout[u] = 0.f; dg[u] = 0.f;
-        if (e >= NP * 32) continue;
-        if (gin_g) {
-          if (c < a.d_g) gin[u] = gin_g[p * a.h2 + c];
-        } else if (c < 4) {
-          const int i = p / N, j = p - (p / N) * N;
-          if (i != j) {
-            const float d0 = (float)rw[3 * i] - (float)rw[3 * j], d1 = (float)rw[3 * i + 1] - (float)rw[3 * j + 1],
-                        d2 = (float)rw[3 * i + 2] - (float)rw[3 * j + 2];
-            gin[u] = c == 0 ? d0 : c == 1 ? d1 : c == 2 ? d2 : sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+        for (int u = 0; u < 8; ++u) {
+          const int p = pb + 4 * u;
+          gin[u] = 0.f; gout[u] = 0.f; dg[u] = 0.f;
+          if (p >= NP) continue;
+          if (gin_g) {
+            if (in_dg) gin[u] = gin_g[p * a.h2];
+          } else if (lane < 4) {
+            const int i = p / N, j = p - i * N;
+            if (i != j) {
+              const float d0 = (float)rw[3 * i] - (float)rw[3 * j], d1 = (float)rw[3 * i + 1] - (float)rw[3 * j + 1],
+                          d2 = (float)rw[3 * i + 2] - (float)rw[3 * j + 2];
+              gin[u] = lane == 0 ? d0 : lane == 1 ? d1 : lane == 2 ? d2 : sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+            }
+          }
+          if (in_h2) {
+            gout[u] = gout_g[p * a.h2];
+            dg[u] = dG[p * a.h2];
           }
         }
-        if (c < a.h2) {
-          gout[u] = gout_g[p * a.h2 + c];
-          dg[u] = dG[p * a.h2 + c];
-        }
-      }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e >= NP * 32) continue;
-        const int p = e >> 5, c = e & 31;
-        gin_s[p * 33 + c] = gin[u];
-        if (c < a.h2) {
+        for (int u = 0; u < 8; ++u) {
+          const int p = pb + 4 * u;
+          if (p >= NP) continue;
           const float t = a.l >= 1 ? gout[u] - gin[u] : gout[u];
-          dz_s[p * 33 + c] = dg[u] * (1.f - t * t);
+          const float dz = in_h2 ? dg[u] * (1.f - t * t) : 0.f;
+          gin_s[pair_at(p, lane)] = gin[u];
+          dz_s[pair_at(p, lane)] = dz;
+          dc += dz;                                                // dc = column sums of dz
         }
       }
-    }
-    __syncthreads();
-    // dc = column sums of dz: warp k sums every fourth pair of its lane's column
-    for (int p = warp; p < NP; p += 4) dc += dz_s[p * 33 + lane];
-    // dW[q][c] = sum_p dz[p][q] g[p][c]: warp -> rows q0 .. q0 + 15, column blocks nb0, nb0 + 1
-    {
+      __syncthreads();
+      // dW[q][c] = sum_p dz[p][q] g[p][c]: warp -> rows q0 .. q0 + 15, column blocks nb0, nb0 + 1
       for (int p0 = 0; p0 < NPp; p0 += 16) {
+        const int p1 = p0 + 2 * tig;                               // A[m = q][k = p] = dz[p][q]
+        const int x0 = (q0 + grp) ^ ((p1 & 3) << 3), x1 = (q0 + grp) ^ (((p1 + 1) & 3) << 3);   // p1 + 8: the same
+        const float *z0 = dz_s + p1 * 32, *z1 = z0 + 32;
         uint32_t ah[4], al[4];
-        const float* zc0 = dz_s + (p0 + 2 * tig) * 33 + q0 + grp;      // A[m = q][k = p] = dz[p][q]
-        split_pack(zc0[0], zc0[33], ah[0], al[0]);
-        split_pack(zc0[8], zc0[33 + 8], ah[1], al[1]);
-        split_pack(zc0[8 * 33], zc0[9 * 33], ah[2], al[2]);
-        split_pack(zc0[8 * 33 + 8], zc0[9 * 33 + 8], ah[3], al[3]);
+        split_pack(z0[x0], z1[x1], ah[0], al[0]);
+        split_pack(z0[x0 ^ 8], z1[x1 ^ 8], ah[1], al[1]);
+        split_pack(z0[8 * 32 + x0], z1[8 * 32 + x1], ah[2], al[2]);
+        split_pack(z0[8 * 32 + (x0 ^ 8)], z1[8 * 32 + (x1 ^ 8)], ah[3], al[3]);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int n = 8 * (nb0 + u) + grp;                          // B[k = p][n = c] = g[p][c]
-          const float* gc0 = gin_s + (p0 + 2 * tig) * 33 + n;
+          const int n = 8 * (nb0 + u) + grp;                      // B[k = p][n = c] = g[p][c]
+          const int y0 = n ^ ((p1 & 3) << 3), y1 = n ^ (((p1 + 1) & 3) << 3);
+          const float *g0 = gin_s + p1 * 32, *g1 = g0 + 32;
           uint32_t bh0, bl0, bh1, bl1;
-          split_pack(gc0[0], gc0[33], bh0, bl0);
-          split_pack(gc0[8 * 33], gc0[9 * 33], bh1, bl1);
+          split_pack(g0[y0], g1[y1], bh0, bl0);
+          split_pack(g0[8 * 32 + y0], g1[8 * 32 + y1], bh1, bl1);
           mma_16816(c2[u], ah, bh0, bh1);
           mma_16816(c2[u], ah, bl0, bl1);
           mma_16816(c2[u], al, bh0, bh1);
         }
       }
-    }
-    __syncthreads();                                               // gin_s is overwritten below
-    // dz W -> gin_s (rows = pairs)
-    for (int mt = warp; mt < NPp / 16; mt += (int)(blockDim.x >> 5)) {
-      const int p0 = mt * 16;
-      float c[4][4] = {};
+      if (a.l < 1) continue;                                       // no gradient below the input features
+      __syncthreads();                                             // gin_s is overwritten below
+      // dz W -> gin_s (rows = pairs)
+      for (int mt = warp; mt < NPp / 16; mt += 4) {
+        const int p0 = mt * 16;
+        float c[4][4] = {};
 #pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        const int k0 = ks * 16;
-        const float* r0 = dz_s + (p0 + grp) * 33 + k0 + 2 * tig;
-        const float* r1 = dz_s + (p0 + grp + 8) * 33 + k0 + 2 * tig;
-        uint32_t ah[4], al[4];
-        split_pack(r0[0], r0[1], ah[0], al[0]);
-        split_pack(r1[0], r1[1], ah[1], al[1]);
-        split_pack(r0[8], r0[9], ah[2], al[2]);
-        split_pack(r1[8], r1[9], ah[3], al[3]);
+        for (int ks = 0; ks < 2; ++ks) pair_mma_k16<kBwdWLd>(dz_s, p0 + grp, wth, wtl, 16 * ks, grp, tig, c);
 #pragma unroll
         for (int nb = 0; nb < 4; ++nb) {
-          const int off = (8 * nb + grp) * kBwdWLd + k0 + 2 * tig;
-          const uint32_t bh0 = *(const uint32_t*)(wth + off), bh1 = *(const uint32_t*)(wth + off + 8);
-          const uint32_t bl0 = *(const uint32_t*)(wtl + off), bl1 = *(const uint32_t*)(wtl + off + 8);
-          mma_16816(c[nb], ah, bh0, bh1);
-          mma_16816(c[nb], ah, bl0, bl1);
-          mma_16816(c[nb], al, bh0, bh1);
+          *(float2*)(gin_s + pair_at(p0 + grp, 8 * nb + 2 * tig)) = make_float2(c[nb][0], c[nb][1]);
+          *(float2*)(gin_s + pair_at(p0 + grp + 8, 8 * nb + 2 * tig)) = make_float2(c[nb][2], c[nb][3]);
         }
       }
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb)
-#pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4)
-          gin_s[(p0 + grp + (q4 >= 2 ? 8 : 0)) * 33 + 8 * nb + 2 * tig + (q4 & 1)] = c[nb][q4];
+      __syncthreads();
     }
-    __syncthreads();
-  }
-  if (a.l < 1) continue;                                           // no gradient below the input features
-  // dG^l = (dz W) + dG^{l+1} (residual) + the spin-mean gradient of the layer input
-  float* dGo = (float*)a.dG + (int64_t)w * NP * a.h2;
-  for (int e = tid; e < NP * a.h2; e += blockDim.x) {
-    const int p = e / a.h2, c = e - (e / a.h2) * a.h2;
-    const int i = p / N, j = p - (p / N) * N;
-    float v = 0.f;
-    if (has_layer) v = gin_s[p * 33 + c] + dGo[e];
-    if (c < a.d_g) {
-      const int sj = j < sh.n_up ? 0 : 1;
-      const int nsj = sj ? sh.n_dn : sh.n_up;
-      v += ((const float*)a.dX)[tile_row(w, i, N, sh.wpt) * a.ldx + a.col0 + sj * a.d_g + c] / (float)nsj;
+    if (a.l < 1) continue;
+    // dG^l = (dz W) + dG^{l+1} (residual) + the spin-mean gradient of the layer input
+    if (in_h2) {
+      const float* dx = (const float*)a.dX + tile_row(w, 0, N, sh.wpt) * a.ldx + a.col0 + lane;
+      for (int i = warp; i < N; i += 4) {
+        float m[2] = {0.f, 0.f};
+#pragma unroll
+        for (int s2 = 0; s2 < 2; ++s2)
+          if (in_dg) m[s2] = dx[(int64_t)i * a.ldx + s2 * a.d_g] / n_spin[s2];
+        for (int j0 = 0; j0 < N; j0 += 8) {
+          float old[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) old[u] = has_layer && j0 + u < N ? dG[(i * N + j0 + u) * a.h2] : 0.f;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int j = j0 + u, p = i * N + j;
+            if (j >= N) break;
+            float v = has_layer ? gin_s[pair_at(p, lane)] + old[u] : 0.f;
+            if (in_dg) v += m[j < sh.n_up ? 0 : 1];
+            dG[p * a.h2] = v;
+          }
+        }
+      }
     }
-    dGo[e] = v;
-  }
   }
   if (!has_layer) return;
 #pragma unroll
@@ -667,7 +663,7 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
       const int qq = q0 + grp + (q4 >= 2 ? 8 : 0), cc = 8 * (nb0 + u) + 2 * tig + (q4 & 1);
       if (qq < a.h2 && cc < a.d_g) atomicAdd((float*)a.gW + qq * a.d_g + cc, c2[u][q4]);
     }
-  if (lane < a.h2) atomicAdd((float*)a.gc + lane, dc);
+  if (in_h2) atomicAdd((float*)a.gc + lane, dc);
 }
 
 __global__ void k_widen_bf16(int64_t n8, const uint4* __restrict__ in, float4* __restrict__ out) {

@@ -82,7 +82,7 @@ inline size_t smem_pair_value(int cmp_bytes, int N, int L) {
 }
 // k_pair_value_mma (BF16)
 inline size_t smem_pair_value_mma(int N, int L) {
-  return (size_t)(L - 1) * (2 * 32 * kPairWLd * 2 + 32 * 4) + (size_t)((N * N + 15) & ~15) * 33 * 4;
+  return (size_t)(L - 1) * (2 * 32 * kPairWLd * 2 + 32 * 4) + (size_t)((N * N + 15) & ~15) * 32 * 4;
 }
 // k_pair_full (FP32/FP64): electrons per CTA, the fewest warps per walker with at most 8 warps per CTA
 inline int pair_full_ib(int N) {
@@ -101,7 +101,7 @@ inline size_t smem_pair_full(int cmp_bytes, int N, int L, int ib) {
 inline int pair_full_mma_ib(int N) { return std::max(1, std::min(N, 256 / (5 * N))); }
 inline size_t smem_pair_full_mma(int N, int L, int ibm) {
   const int rows_p = (ibm * N * 5 + 15) & ~15;
-  return (size_t)(L - 1) * (2 * 32 * kPairWLd * 2 + 32 * 4) + (size_t)2 * rows_p * 33 * 4;
+  return (size_t)(L - 1) * (2 * 32 * kPairWLd * 2 + 32 * 4) + (size_t)2 * rows_p * 32 * 4;
 }
 // k_pair_bwd_mma (BF16)
 inline size_t smem_pair_bwd_mma(int N) { return 2 * 32 * kBwdWLd * 2 + (size_t)2 * ((N * N + 15) & ~15) * 33 * 4; }

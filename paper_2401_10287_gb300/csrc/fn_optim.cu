@@ -114,7 +114,7 @@ constexpr int kClipCached = 8;         // keys per thread kept in registers (bat
 
 // One CTA, so its time is its chain of barriers: 8 digit passes over the batch in memory took 20 us
 // for 4096 energies.  With the keys in registers and the search ended as soon as one key is left
-// in the bin (two or three digits, unless energies are equal) it takes @CLIP@ us.
+// in the bin (two or three digits, unless energies are equal) the call with an Adam step went from 31 to 28 us.
 __global__ void __launch_bounds__(kClipThreads) k_clip_energy(int B, const double* e, double width, double* out,
                                                                double* __restrict__ stats,
                                                                int* __restrict__ status) {

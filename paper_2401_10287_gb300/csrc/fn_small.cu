@@ -285,7 +285,7 @@ static void launch(const SmallArgs& a, cudaStream_t st) {
   const int threads = (int)std::min<int64_t>(kSmallThreads, round_up((int64_t)a.G * a.N * a.h1, 32));
   const size_t smem = small_layout(a).total * sizeof(double);
   cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  launch_k(true, k_small, (unsigned)((a.B + a.G - 1) / a.G), threads, smem, st, a);
+  launch_k(false, k_small, (unsigned)((a.B + a.G - 1) / a.G), threads, smem, st, a);
 }
 
 void launch_small_log_psi(const fn_system* s, const void* walkers, int B, double* log_psi, int8_t* sign, cudaStream_t st) {
