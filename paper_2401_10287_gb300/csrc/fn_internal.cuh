@@ -249,18 +249,20 @@ struct fn_system {
 
 namespace fn {
 
-// Whether a pass of this size lets its kernels begin while their predecessors drain: below about
-// 2^18 electron rows x slabs the kernels take 5 to 30 us and the gaps between them count (value
-// pass of a 256-walker carbon atom 205 -> 164 us, LiH training iteration 4.43 -> 3.85 ms); above,
-// CTAs that arrive while only some SMs have room crowd onto those (N2 local energy 10.8 -> 11.2 ms,
-// its FP32 form 15.7 -> 16.5).  FP64 kernels do not overlap: two CTAs on one SM share its slow FP64
-// pipe while other SMs idle (H2 pass 1.34 -> 1.41 ms).
+// Whether a pass lets its kernels begin while their predecessors drain.  Value passes do up to
+// 2^18 rows: their kernels take 5 to 30 us and the gaps between them count (256-walker carbon atom
+// 205 -> 164 us, LiH training iteration 4.43 -> 3.85 ms).  Passes with tangent slabs only do while
+// tiny, up to 2^15 rows x slabs (H2, 700 walkers: 147 -> 128 us): in their longer kernels, CTAs that
+// arrive while only some SMs have room crowd onto those (C, 700 walkers, BF16: 841 -> 1176 us; N2,
+// 4096 walkers, FP32: 15.7 -> 16.5 ms).  FP64 kernels and the FMA-bound products of fn_simt.cu do not
+// overlap: two CTAs on one SM share its pipe while other SMs idle (H2 FP64 pass 1.34 -> 1.41 ms;
+// FP32 value pass of 300 Si- walkers 287 -> 388 us).
 inline bool overlap_launches(const Shape& sh, size_t word = 4) {
-  return word == 4 && (int64_t)sh.T * sh.R <= ((int64_t)1 << 18);
+  return word == 4 && (int64_t)sh.T * sh.R <= ((int64_t)1 << (sh.T == 1 ? 18 : 15));
 }
 
-// The same for a product, by its rows (electron rows, or T x walkers of at least four electrons).
-constexpr int64_t kOverlapGemmRows = 1 << 16;
+// The same for a product, by its rows (electrons, walkers, or slabs x walkers).
+constexpr int64_t kOverlapGemmRows = 1 << 13;
 
 // Launch of a kernel that calls pdl_wait; with `overlap` it may begin while its predecessor in the
 // stream drains.

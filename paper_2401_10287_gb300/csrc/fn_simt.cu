@@ -141,7 +141,7 @@ static void layer_cfg(const Shape& sh, const LayerArgs& a, bool vec, cudaStream_
   const unsigned grid = (unsigned)((a.h1 + Tl::BN - 1) / Tl::BN) * sh.tiles * subs;
   auto go = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_k(overlap_launches(sh, sizeof(T)), kernel, grid, Tl::kThreads, smem, st, sh, a, wps, subs);
+    launch_k(false, kernel, grid, Tl::kThreads, smem, st, sh, a, wps, subs);
   };
   if (sh.T > 1) vec ? go(k_layer<T, TM, TN, WM, true, true>) : go(k_layer<T, TM, TN, WM, true, false>);
   else vec ? go(k_layer<T, TM, TN, WM, false, true>) : go(k_layer<T, TM, TN, WM, false, false>);
@@ -310,7 +310,7 @@ static void orbitals_cfg(const Shape& sh, const OrbArgs& a, int spin, cudaStream
   const dim3 grid((unsigned)((n_ko + Tl::BN - 1) / Tl::BN) * ((sh.B + wpc - 1) / wpc), 1, sh.T);
   auto go = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_k(overlap_launches(sh, sizeof(T)), kernel, grid, Tl::kThreads, smem, st, sh, a, spin);
+    launch_k(false, kernel, grid, Tl::kThreads, smem, st, sh, a, spin);
   };
   if (full) vec ? go(k_orbitals<T, TM, TN, WM, true, true>) : go(k_orbitals<T, TM, TN, WM, true, false>);
   else vec ? go(k_orbitals<T, TM, TN, WM, false, true>) : go(k_orbitals<T, TM, TN, WM, false, false>);
@@ -319,7 +319,7 @@ static void orbitals_cfg(const Shape& sh, const OrbArgs& a, int spin, cudaStream
 template <typename T>
 void launch_envelope(const Shape& sh, const OrbArgs& a, cudaStream_t st) {
   const int n_ko = a.K * std::max(sh.n_up, sh.n_dn);
-  launch_k(overlap_launches(sh, sizeof(T)), k_envelope<T>, dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st,
+  launch_k(false, k_envelope<T>, dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st,
       sh, a);
 }
 
@@ -416,7 +416,7 @@ static void gemm_cfg(const GemmArgs<T>& g, bool at, bool bt, int split, bool vec
   const dim3 grid((unsigned)((g.N + Tl::BN - 1) / Tl::BN * ((g.M + Tl::BM - 1) / Tl::BM)), 1, split);
   auto go = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Tl::kRingBytes);
-    launch_k(sizeof(T) == 4 && g.M <= kOverlapGemmRows, kernel, grid, Tl::kThreads, Tl::kRingBytes, st, g);
+    launch_k(false, kernel, grid, Tl::kThreads, Tl::kRingBytes, st, g);
   };
   if (at) vec ? go(k_gemm<T, TM, TN, WM, true, false, true>) : go(k_gemm<T, TM, TN, WM, true, false, false>);
   else if (bt) vec ? go(k_gemm<T, TM, TN, WM, false, true, true>) : go(k_gemm<T, TM, TN, WM, false, true, false>);
