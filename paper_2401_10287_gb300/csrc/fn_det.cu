@@ -1318,18 +1318,20 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
   const int nmax = std::max(s->n_up, s->n_dn), K = s->cfg.n_dets;
   ProfScope ps(s->prof, full ? kProfDetFull : kProfDetValue, st);
   if (full && nmax <= 4 && s->N <= 8) {
+    // FP64 in every mode.  A determinant that nearly vanishes beside a psi that does not leaves terms
+    // 1/d^2 that cancel to 1/d between lap_k and |g_k|^2; in FP32 they decided the error of the FP32
+    // energies of few-electron walkers (one such walker up to 0.99 of the 2-norm over 2500).  LiH-,
+    // 4096 walkers: 72 -> 189 us of a 1.8 ms call, error against 64 bits 1.0e-6 -> 0.4e-6 in the 2-norm.
     const int per_cta = 128 / (2 * K);
-    const size_t smem = smem_det_energy_small(sizeof(Det), s->N, K);
-    cudaFuncSetAttribute(k_det_energy_small<4, Det, Wlk, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_k(ov, k_det_energy_small<4, Det, Wlk, PhiT>,
-        (unsigned)((sh.B + per_cta - 1) / per_cta), 128, smem, st,
-               (const Wlk*)walkers, s->d_nuclei, sh, a);
+    const size_t smem = smem_det_energy_small(sizeof(double), s->N, K);
+    cudaFuncSetAttribute(k_det_energy_small<4, double, Wlk, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_k(ov, k_det_energy_small<4, double, Wlk, PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, smem, st,
+             (const Wlk*)walkers, s->d_nuclei, sh, a);
   } else if (full && std::is_same<Det, double>::value && std::is_same<PhiT, float>::value && nmax <= kGrpN &&
              det_grp_enabled()) {
     const size_t smem = smem_det_energy_grp(s->N, K);
     cudaFuncSetAttribute(k_det_energy_grp<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_k(ov, k_det_energy_grp<Wlk>, sh.B, 128, smem, st, (const Wlk*)walkers, s->d_nuclei, sh,
-        a);
+    launch_k(ov, k_det_energy_grp<Wlk>, sh.B, 128, smem, st, (const Wlk*)walkers, s->d_nuclei, sh, a);
   } else if (full) {
     const size_t smem = smem_det_energy(sizeof(Det), nmax, s->N, K,
                                         std::is_same<Det, double>::value && std::is_same<PhiT, float>::value);
@@ -1342,8 +1344,7 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
         st, sh, a);
   } else if (std::is_same<Det, double>::value && nmax <= 8) {
     const int per_cta = 128 / (2 * K);
-    launch_k(ov, k_det_seed_small<PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st,
-        sh, a);
+    launch_k(ov, k_det_seed_small<PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st, sh, a);
   } else {
     const int threads = (int)round_up(2 * K, 32);
     const size_t vsmem = smem_det_value(sizeof(Det), nmax, K, keep_inverse);
