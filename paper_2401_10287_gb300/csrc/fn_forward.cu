@@ -2,8 +2,8 @@
 // ("FermiNet Model" section; Eq. 4 envelope): SIMT kernels for FP64/FP32, the BF16-mode
 // kernels around the tensor-core ones of fn_layer_tc.cu, and the launch sequence:
 //   k_prep             parameter blob -> internal layouts (one launch, descriptor table)
-//   k_features_en      one-electron stream input [r_i - R_m, |r_i - R_m|] with tangents
-//   k_features_mean    spin means of the one-electron input
+//   k_features         one-electron stream input [r_i - R_m, |r_i - R_m|] with tangents, and
+//                      its spin means
 //   k_pair_full/value  two-electron stream, SIMT (a pair depends on r_i - r_j only: 5 jet
 //                      rows) and its spin means for every layer
 //   k_pair_*_mma       the same on warp-level BF16 MMAs with hi/lo splits (BF16 mode)
@@ -163,99 +163,85 @@ void launch_prep_params(const fn_system* s, const void* params, bool full, cudaS
 // ---------------------------------------------------------------------------------------
 // input features
 // ---------------------------------------------------------------------------------------
-template <typename Act, typename Wlk>
-__global__ void k_features_en(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh,
-                              Act* __restrict__ X0, int ldx) {
-  pdl_wait();
-  pdl_launch();
-  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)sh.B * sh.N) return;
-  const int w = (int)(gid / sh.N), i = (int)(gid % sh.N);
-  const int64_t row = tile_row(w, i, sh.N, sh.wpt);
-  const int64_t slab = sh.R * ldx;
-  const double rx = (double)r[gid * 3], ry = (double)r[gid * 3 + 1], rz = (double)r[gid * 3 + 2];
-  for (int m = 0; m < sh.M; ++m) {
-    const double d[3] = {rx - nuc[3 * m], ry - nuc[3 * m + 1], rz - nuc[3 * m + 2]};
-    const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    Act* base = X0 + row * ldx + 4 * m;
-    for (int a = 0; a < 3; ++a) st(base + a, d[a]);
-    st(base + 3, dist);
-    if (SplitValue<Act>::value) {
-      Act* lo = base + sh.T * slab;
-      for (int a = 0; a < 3; ++a) st_lo(lo + a, d[a]);
-      st_lo(lo + 3, dist);
-    }
-    if (sh.T == 1) continue;
-    for (int t = 1; t < sh.T; ++t) {
-      Act* o = base + t * slab;
-      const int e = (t - 1) / 3, c = (t - 1) % 3;
-      if (t == sh.T - 1) {
-        st(o, 0.0); st(o + 1, 0.0); st(o + 2, 0.0); st(o + 3, 2.0 / dist);
-      } else if (e == i) {
-        for (int a = 0; a < 3; ++a) st(o + a, a == c ? 1.0 : 0.0);
-        st(o + 3, d[c] / dist);
-      } else {
-        for (int a = 0; a < 4; ++a) st(o + a, 0.0);
-      }
-    }
+// One kernel for the layer-0 rows h0 = [r_i - R_m, |r_i - R_m|], their tangents, and the spin means
+// of both (Hbar0[t][w][spin * 4M + 4m + a]).  A thread takes one (electron, nucleus) of the CTA's
+// walkers: the FP64 root and quotients are formed once and shared through shared memory (two kernels
+// formed them twice with 4 warps per SM: 137 us for N2 at 4096 walkers with tangents, 27 us without),
+// and every group of four values leaves as one vector.
+constexpr int kFeatThreads = 256;
+template <typename Act> struct alignas(4 * sizeof(Act) > 16 ? 16 : 4 * sizeof(Act)) Act4 { Act v[4]; };
+
+template <typename Act>
+__device__ __forceinline__ void st4(Act* p, double a, double b, double c, double d) {
+  Act4<Act> o;
+  st(o.v, a); st(o.v + 1, b); st(o.v + 2, c); st(o.v + 3, d);
+  *(Act4<Act>*)p = o;
+}
+// the values and, in BF16 storage, their low parts `lo` elements further
+template <typename Act>
+__device__ __forceinline__ void st4_split(Act* p, int64_t lo, double a, double b, double c, double d) {
+  st4(p, a, b, c, d);
+  if constexpr (SplitValue<Act>::value) {
+    Act4<Act> o;
+    st_lo(o.v, a); st_lo(o.v + 1, b); st_lo(o.v + 2, c); st_lo(o.v + 3, d);
+    *(Act4<Act>*)(p + lo) = o;
   }
 }
 
-// Hbar0[t][w][spin * 4M + 4m + a]: mean over the electrons of one spin of h0.
 template <typename Act, typename Wlk>
-__global__ void k_features_mean(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh,
-                                Act* __restrict__ Hbar) {
+__global__ void __launch_bounds__(kFeatThreads) k_features(const Wlk* __restrict__ r, const double* __restrict__ nuc,
+                                                           Shape sh, Act* __restrict__ X0, int ldx,
+                                                           Act* __restrict__ Hbar, int wpb) {
   pdl_wait();
   pdl_launch();
-  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)sh.B * 2 * sh.M) return;
-  const int w = (int)(gid / (2 * sh.M)), spin = (int)((gid / sh.M) % 2), m = (int)(gid % sh.M);
-  const int lo = spin ? sh.n_up : 0, hi = spin ? sh.N : sh.n_up;
-  const int n_s = hi - lo;
-  const int width = 2 * 4 * sh.M;
-  const int64_t slab = (int64_t)sh.B * width;
-  Act* base = Hbar + (int64_t)w * width + spin * 4 * sh.M + 4 * m;
-  const double inv = n_s ? 1.0 / n_s : 0.0;
-  double v[4] = {0, 0, 0, 0}, lap = 0.0;
-  for (int e = lo; e < hi; ++e) {
-    const Wlk* re = r + ((int64_t)w * sh.N + e) * 3;
-    const double d[3] = {(double)re[0] - nuc[3 * m], (double)re[1] - nuc[3 * m + 1], (double)re[2] - nuc[3 * m + 2]};
-    const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    v[0] += d[0]; v[1] += d[1]; v[2] += d[2]; v[3] += dist;
-    lap += 2.0 / dist;
-    if (sh.T > 1)
-      for (int c = 0; c < 3; ++c) {
-        Act* o = base + (1 + 3 * e + c) * slab;
-        for (int a = 0; a < 3; ++a) st(o + a, a == c ? inv : 0.0);
-        st(o + 3, d[c] / dist * inv);
-        if (SplitValue<Act>::value) {
-          Act* ol = o + sh.T * slab;
-          for (int a = 0; a < 3; ++a) st_lo(ol + a, a == c ? inv : 0.0);
-          st_lo(ol + 3, d[c] / dist * inv);
-        }
-      }
-  }
-  for (int a = 0; a < 4; ++a) st(base + a, v[a] * inv);
-  if (SplitValue<Act>::value)
-    for (int a = 0; a < 4; ++a) st_lo(base + sh.T * slab + a, v[a] * inv);
-  if (sh.T == 1) return;
-  Act* o = base + (sh.T - 1) * slab;
-  st(o, 0.0); st(o + 1, 0.0); st(o + 2, 0.0); st(o + 3, lap * inv);
-  if (SplitValue<Act>::value) {
-    Act* ol = o + sh.T * slab;
-    st_lo(ol, 0.0); st_lo(ol + 1, 0.0); st_lo(ol + 2, 0.0); st_lo(ol + 3, lap * inv);
-  }
-  // slabs of the other spin's electrons are zero
-  const int olo = spin ? 0 : sh.n_up, ohi = spin ? sh.n_up : sh.N;
-  for (int e = olo; e < ohi; ++e)
+  __shared__ double4 sd[kMaxElectrons * kMaxNuclei];              // d, |d| per (walker, electron, nucleus)
+  const int N = sh.N, M = sh.M, w0 = blockIdx.x * wpb, nw = min(wpb, sh.B - w0), T = sh.T;
+  const int64_t xslab = sh.R * ldx, hslab = (int64_t)sh.B * 8 * M;
+  for (int e = threadIdx.x; e < nw * N * M; e += blockDim.x) {
+    const int m = e % M, wi = e / M, wl = wi / N, i = wi - wl * N, w = w0 + wl;
+    const Wlk* p = r + ((int64_t)w * N + i) * 3;
+    const double d0 = (double)p[0] - nuc[3 * m], d1 = (double)p[1] - nuc[3 * m + 1], d2 = (double)p[2] - nuc[3 * m + 2];
+    const double dist = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+    sd[e] = make_double4(d0, d1, d2, dist);
+    Act* x = X0 + tile_row(w, i, N, sh.wpt) * ldx + 4 * m;
+    st4_split(x, T * xslab, d0, d1, d2, dist);
+    if (T == 1) continue;
+    const int s = i < sh.n_up ? 0 : 1;
+    const double inv = 1.0 / (s ? sh.n_dn : sh.n_up);
+    const double q[3] = {d0 / dist, d1 / dist, d2 / dist};
+    Act* hb = Hbar + (int64_t)w * 8 * M + s * 4 * M + 4 * m;      // own spin's mean; the other's gets zero
+    Act* ho = Hbar + (int64_t)w * 8 * M + (1 - s) * 4 * M + 4 * m;
     for (int c = 0; c < 3; ++c) {
-      Act* q = base + (1 + 3 * e + c) * slab;
-      st(q, 0.0); st(q + 1, 0.0); st(q + 2, 0.0); st(q + 3, 0.0);
-      if (SplitValue<Act>::value) {
-        Act* ql = q + sh.T * slab;
-        st_lo(ql, 0.0); st_lo(ql + 1, 0.0); st_lo(ql + 2, 0.0); st_lo(ql + 3, 0.0);
-      }
+      const int t = 1 + 3 * i + c;
+      const double u0 = c == 0, u1 = c == 1, u2 = c == 2;
+      st4(x + t * xslab, u0, u1, u2, q[c]);
+      st4_split(hb + t * hslab, T * hslab, u0 * inv, u1 * inv, u2 * inv, q[c] * inv);
+      st4_split(ho + t * hslab, T * hslab, 0.0, 0.0, 0.0, 0.0);
     }
+    st4(x + (T - 1) * xslab, 0.0, 0.0, 0.0, 2.0 / dist);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nw * 2 * M; e += blockDim.x) {
+    const int m = e % M, ws = e / M, wl = ws >> 1, s = ws & 1, lo = s ? sh.n_up : 0, hi = s ? N : sh.n_up;
+    const double inv = hi > lo ? 1.0 / (hi - lo) : 0.0;
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0, lap = 0.0;
+    for (int i = lo; i < hi; ++i) {
+      const double4 d = sd[(wl * N + i) * M + m];
+      v0 += d.x; v1 += d.y; v2 += d.z; v3 += d.w;
+      if (T > 1) lap += 2.0 / d.w;
+    }
+    Act* hb = Hbar + (int64_t)(w0 + wl) * 8 * M + s * 4 * M + 4 * m;
+    st4_split(hb, T * hslab, v0 * inv, v1 * inv, v2 * inv, v3 * inv);
+    if (T > 1) st4_split(hb + (T - 1) * hslab, T * hslab, 0.0, 0.0, 0.0, lap * inv);
+  }
+  if (T == 1) return;
+  // the rows' slabs of other electrons' coordinates are zero
+  const int per_t = nw * N * M;
+  for (int e = threadIdx.x; e < (T - 2) * per_t; e += blockDim.x) {
+    const int t = e / per_t, k = e - t * per_t, m = k % M, wi = k / M, wl = wi / N, i = wi - wl * N;
+    if (t / 3 == i) continue;
+    st4(X0 + (1 + t) * xslab + tile_row(w0 + wl, i, N, sh.wpt) * ldx + 4 * m, 0.0, 0.0, 0.0, 0.0);
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -907,24 +893,26 @@ using simt::OrbArgs;
 // Envelope sum_m pi exp(-s_m) of orbital ko at electron position rj (Eq. 4), its gradient
 // along rj and its Laplacian.  Isotropic: s = sigma |d|; anisotropic: s = |Sigma d|, with
 // grad s = Sigma^T u / s and lap s = (|Sigma|_F^2 - |Sigma^T u|^2 / s^2) / s.
-template <typename Cmp, typename Wlk>
-__device__ __forceinline__ void env_jet(const OrbArgs& a, int spin, int ko, const Wlk* rj, const double* nuc, int M,
-                                        Cmp* env_out, Cmp* ge, Cmp* le_out) {
-  const Cmp* pi = (const Cmp*)a.pi[spin] + (int64_t)ko * M;
+// par: per nucleus pi, then sigma (1 or 9 words), consecutive words `ld` apart; dist: per nucleus d.
+template <typename Cmp>
+__device__ __forceinline__ void env_jet(int aniso, const Cmp* par, int ld, const Cmp* dist, int M, Cmp* env_out, Cmp* ge,
+                                        Cmp* le_out) {
   Cmp env = 0, le = 0;
   ge[0] = ge[1] = ge[2] = 0;
   for (int m = 0; m < M; ++m) {
-    const Cmp d[3] = {(Cmp)((double)rj[0] - nuc[3 * m]), (Cmp)((double)rj[1] - nuc[3 * m + 1]),
-                      (Cmp)((double)rj[2] - nuc[3 * m + 2])};
+    const Cmp d[3] = {dist[3 * m], dist[3 * m + 1], dist[3 * m + 2]};
+    const Cmp* pm = par + m * (aniso ? 10 : 2) * ld;
     Cmp s, gs[3], ls;
-    if (!a.aniso) {
-      const Cmp sg = ((const Cmp*)a.sig[spin])[(int64_t)ko * M + m];
-      const Cmp dist = f_sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      s = sg * dist;
-      for (int c = 0; c < 3; ++c) gs[c] = sg * d[c] / dist;
-      ls = (Cmp)2 * sg / dist;
+    if (!aniso) {
+      const Cmp sg = pm[ld];
+      const Cmp dist1 = f_sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+      s = sg * dist1;
+      for (int c = 0; c < 3; ++c) gs[c] = sg * d[c] / dist1;
+      ls = (Cmp)2 * sg / dist1;
     } else {
-      const Cmp* S = (const Cmp*)a.sig[spin] + ((int64_t)ko * M + m) * 9;
+      Cmp S[9];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) S[q] = pm[(1 + q) * ld];
       Cmp u[3];
       for (int x = 0; x < 3; ++x) u[x] = S[3 * x] * d[0] + S[3 * x + 1] * d[1] + S[3 * x + 2] * d[2];
       s = f_sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
@@ -934,7 +922,7 @@ __device__ __forceinline__ void env_jet(const OrbArgs& a, int spin, int ko, cons
       for (int y = 0; y < 3; ++y) { gs[y] = stu[y] / s; n2 += stu[y] * stu[y]; }
       ls = (frob - n2 / (s * s)) / s;
     }
-    const Cmp e = pi[m] * f_exp(-s);
+    const Cmp e = pm[0] * f_exp(-s);
     env += e;
     Cmp g2 = 0;
     for (int c = 0; c < 3; ++c) { ge[c] -= e * gs[c]; g2 += gs[c] * gs[c]; }
@@ -946,33 +934,62 @@ __device__ __forceinline__ void env_jet(const OrbArgs& a, int spin, int ko, cons
 
 // Envelope-derivative terms of the full pass: on the slabs of the row's own
 // coordinates phi += P_0 d_c env, on the Laplacian slab phi += 2 sum_c P_c d_c env + P_0 lap env.
+// A thread keeps one (electron, orbital) and walks over the walkers; the envelope parameters of the
+// CTA's orbitals sit in shared memory, transposed so that consecutive orbitals read consecutive
+// words, and a walker's electron-nucleus distances are formed once per CTA (as FP64 differences in
+// every thread they took half of the kernel's time).  N2, 4096 walkers: 0.36 -> @FX@ ms.
 template <typename Cmp, typename PhiT, typename Wlk>
-__global__ void k_orbital_fixup(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbArgs a,
-                                const Cmp* __restrict__ orbP) {
+__global__ void __launch_bounds__(256) k_orbital_fixup(const Wlk* __restrict__ r, const double* __restrict__ nuc,
+                                                       Shape sh, OrbArgs a, const Cmp* __restrict__ orbP, int slots) {
   pdl_wait();
   pdl_launch();
-  const int w = blockIdx.x / sh.N, j = blockIdx.x % sh.N;
-  const int spin = j < sh.n_up ? 0 : 1;
-  const int n_s = spin ? sh.n_dn : sh.n_up;
-  const int ko = threadIdx.x;
-  if (ko >= a.K * n_s) return;
-  const int jj = j - (spin ? sh.n_up : 0);
-  const int64_t row = tile_row(w, j, sh.N, sh.wpt);
-  const int ldp = a.K * sh.N, poff = spin ? a.K * sh.n_up : 0;
-  Cmp env, ge[3], le;
-  env_jet<Cmp, Wlk>(a, spin, ko, r + ((int64_t)w * sh.N + j) * 3, nuc, sh.M, &env, ge, &le);
-  const Cmp* pr = orbP + row * 4 * ldp + poff + ko;
-  const Cmp P0 = pr[0];
-  const int k = ko / n_s, i = ko % n_s;
-  const int64_t nn = (int64_t)n_s * n_s;
-  PhiT* base = (PhiT*)a.Phi + (int64_t)w * a.PW + (spin ? (int64_t)a.K * sh.T * sh.n_up * sh.n_up : 0) +
-               (int64_t)k * sh.T * nn + i * n_s + jj;
-  Cmp lap = P0 * le;
-  for (int c = 0; c < 3; ++c) {
-    base[(1 + 3 * j + c) * nn] += (PhiT)(P0 * ge[c]);
-    lap += (Cmp)2 * pr[(1 + c) * ldp] * ge[c];
+  extern __shared__ __align__(16) unsigned char fix_smem[];
+  const int M = sh.M, N = sh.N, nc = a.aniso ? 9 : 1, tid = threadIdx.x, nt = blockDim.x;
+  const int up_block = a.K * sh.n_up * sh.n_up, per_walker = up_block + a.K * sh.n_dn * sh.n_dn;
+  Cmp* ds = (Cmp*)fix_smem;                                     // [slots][N][3 M] distances of the walkers
+  Cmp* ps = ds + slots * 3 * N * M;                                     // [M][1 + nc][threads]: pi, sigma of the thread's orbital
+  const int slot = slots > 1 ? tid / per_walker : 0;
+  int rem = slots > 1 ? tid - slot * per_walker : blockIdx.x * nt + tid;
+  const bool live = rem < per_walker && slot < slots;
+  if (!live) rem = per_walker - 1;
+  const int spin = rem < up_block ? 0 : 1;
+  if (spin) rem -= up_block;
+  const int n_s = spin ? sh.n_dn : sh.n_up, Kn = a.K * n_s, jj = rem / Kn, ko = rem - jj * Kn;
+  const int j = (spin ? sh.n_up : 0) + jj, k = ko / n_s, i = ko - k * n_s;
+  for (int m = 0; m < M; ++m) {
+    ps[m * (1 + nc) * nt + tid] = ((const Cmp*)a.pi[spin])[(int64_t)ko * M + m];
+    for (int c = 0; c < nc; ++c)
+      ps[(m * (1 + nc) + 1 + c) * nt + tid] = ((const Cmp*)a.sig[spin])[((int64_t)ko * M + m) * nc + c];
   }
-  base[(sh.T - 1) * nn] += (PhiT)lap;
+  const int ldp = a.K * N, poff = spin ? a.K * sh.n_up : 0;
+  const int64_t nn = (int64_t)n_s * n_s;
+  const int64_t phi_off = (spin ? (int64_t)a.K * sh.T * sh.n_up * sh.n_up : 0) + (int64_t)k * sh.T * nn + i * n_s + jj;
+  for (int w0 = blockIdx.y * slots; w0 < sh.B; w0 += gridDim.y * slots) {
+    const int w = w0 + slot;
+    __syncthreads();
+    for (int e = tid; e < min(slots, sh.B - w0) * 3 * N * M; e += nt) {
+      const int el = e / (3 * M), q = e - el * 3 * M;
+      ds[e] = (Cmp)((double)r[((int64_t)w0 * N + el) * 3 + q % 3] - nuc[q]);
+    }
+    __syncthreads();
+    if (!live || w >= sh.B) continue;
+    const Cmp* pr = orbP + tile_row(w, j, N, sh.wpt) * 4 * ldp + poff + ko;
+    const Cmp P0 = pr[0], P1 = pr[ldp], P2 = pr[2 * ldp], P3 = pr[3 * ldp];
+    PhiT* base = (PhiT*)a.Phi + (int64_t)w * a.PW + phi_off;
+    PhiT old[4];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) old[c] = base[(1 + 3 * j + c) * nn];
+    old[3] = base[(sh.T - 1) * nn];
+    Cmp env, ge[3], le;
+    env_jet<Cmp>(a.aniso, ps + tid, nt, ds + (slot * N + j) * 3 * M, M, &env, ge, &le);
+    Cmp lap = P0 * le;
+    lap += (Cmp)2 * P1 * ge[0];
+    lap += (Cmp)2 * P2 * ge[1];
+    lap += (Cmp)2 * P3 * ge[2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) base[(1 + 3 * j + c) * nn] = old[c] + (PhiT)(P0 * ge[c]);
+    base[(sh.T - 1) * nn] = old[3] + (PhiT)lap;
+  }
 }
 
 // Envelope values of every (electron, own-spin orbital), one thread each (tensor-core pass).
@@ -1104,15 +1121,11 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
   const Wlk* r = (const Wlk*)walkers;
   // inputs
   {
-    const int64_t n = (int64_t)sh.B * sh.N;
     ProfScope ps(s->prof, kProfFeatures, st);
-    launch_k(ov, k_features_en<Act, Wlk>, (unsigned)((n + 127) / 128), 128, 0, st, r, s->d_nuclei,
-        sh, (Act*)ws.X[0],
-                                                                           s->layer[0].ldx);
-    const int64_t m = (int64_t)sh.B * 2 * sh.M;
-    launch_k(ov, k_features_mean<Act, Wlk>, (unsigned)((m + 127) / 128), 128, 0, st, r,
-        s->d_nuclei, sh,
-               (Act*)ws.Hbar[0]);
+    // walkers of a CTA: one item per thread, fewer while SMs would have no CTA
+    const int wpb = std::max(1, std::min(kFeatThreads / (sh.N * sh.M), (sh.B + s->sm_count - 1) / s->sm_count));
+    launch_k(ov, k_features<Act, Wlk>, (unsigned)((sh.B + wpb - 1) / wpb), kFeatThreads, 0, st, r, s->d_nuclei, sh,
+             (Act*)ws.X[0], s->layer[0].ldx, (Act*)ws.Hbar[0], wpb);
   }
   {
     PairArgs pa{};
@@ -1281,10 +1294,17 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
     }
     if (!ok) const_cast<fn_system*>(s)->host_error = FN_ERR_CUDA;
     if (full) {
-      const int ko_max = s->cfg.n_dets * std::max(s->n_up, s->n_dn);
+      const int items = s->cfg.n_dets * (s->n_up * s->n_up + s->n_dn * s->n_dn), words = s->M * (oa.aniso ? 10 : 2);
+      int threads = 256;                                        // (two CTAs per SM at least)
+      while (threads > 64 && sizeof(Cmp) * words * threads > 96 * 1024) threads /= 2;
+      const int gx = (items + threads - 1) / threads;
+      const int slots = std::max(1, threads / items);           // walkers side by side where one is few orbitals
+      const size_t smem = sizeof(Cmp) * ((size_t)3 * s->N * s->M * slots + (size_t)words * threads);
+      const int gy = std::max(1, std::min((sh.B + slots - 1) / slots, (8 * s->sm_count + gx - 1) / gx));
+      auto kernel = k_orbital_fixup<Cmp, typename Mode::PhiT, Wlk>;
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       ProfScope ps(s->prof, kProfOrbFix, st);
-      launch_k(ov, k_orbital_fixup<Cmp, typename Mode::PhiT, Wlk>, (unsigned)((int64_t)sh.B * sh.N),
-                 (unsigned)round_up(ko_max, 32), 0, st, r, s->d_nuclei, sh, oa, (const Cmp*)ws.orbP);
+      launch_k(ov, kernel, dim3(gx, gy), threads, smem, st, r, s->d_nuclei, sh, oa, (const Cmp*)ws.orbP, slots);
     }
   }
 }

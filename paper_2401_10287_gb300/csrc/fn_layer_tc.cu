@@ -1762,10 +1762,16 @@ bool launch_orbitals_tc(const Shape& sh, const void* HL, int h1, const void* W16
   CUtensorMap ta[2], tb;
   tc::TcArgs a{};
   const int ns[2] = {sh.n_up, sh.n_dn};
+  a.ctiles_up = (K * sh.n_up + nt - 1) / nt;
+  const int ctiles_dn = (K * sh.n_dn + nt - 1) / nt, ctiles = a.ctiles_up + ctiles_dn;
+  // As many walker tiles of one spin in a row tile as fit; fewer while the row tiles still find a
+  // CTA each (C, 256 walkers, value pass, 11 tiles: two or three to a row tile 166 us, one 157 us;
+  // Si-, 1031 walkers, full pass: one to a row tile makes a second round, 0.44 against 0.26 ms).
+  const int per_col = std::max(1, sm_count() / ctiles);
   for (int q = 0; q < 2; ++q) {
-    a.group[q] = a.rtiles[q] = 0;
     if (!ns[q]) continue;
     a.group[q] = std::min(sh.tiles, 128 / (sh.wpt * ns[q]));
+    while (a.group[q] > 1 && (sh.tiles + a.group[q] - 2) / (a.group[q] - 1) <= per_col) --a.group[q];
     a.rtiles[q] = (sh.tiles + a.group[q] - 1) / a.group[q];
     if (!make_spin_map(&ta[q], (const __nv_bfloat16*)HL + (int64_t)(q ? sh.n_up : 0) * h1, h1, ns[q], sh, a.group[q]))
       return false;
@@ -1783,8 +1789,6 @@ bool launch_orbitals_tc(const Shape& sh, const void* HL, int h1, const void* W16
   a.nuclei = nuclei;
   a.K = K;
   a.aniso = aniso;
-  a.ctiles_up = (K * sh.n_up + nt - 1) / nt;
-  const int ctiles_dn = (K * sh.n_dn + nt - 1) / nt;
   a.Phi = (float*)Phi;
   a.PW = PW;
   a.orbP = orbP;
@@ -1795,7 +1799,7 @@ bool launch_orbitals_tc(const Shape& sh, const void* HL, int h1, const void* W16
   const bool full = sh.T > 1;
   a.tmem_cols = pow2_cols(3 * nt);
   launch_tc<tc::kEpiOrbital>(ta[0], ta[1], tb, a,
-                             persistent_grid(a.ctiles_up + ctiles_dn, std::max(a.rtiles[0], a.rtiles[1])), full, st);
+                             persistent_grid(ctiles, std::max(a.rtiles[0], a.rtiles[1])), full, st);
   return true;
 }
 
