@@ -24,6 +24,7 @@
 #include "fn_internal.cuh"
 #include "fn_lu.cuh"
 #include "fn_small.cuh"
+#include "fn_tc.cuh"
 
 namespace fn {
 
@@ -431,84 +432,68 @@ __global__ void __launch_bounds__(128) k_det_energy(const Wlk* __restrict__ r, c
 // One CTA of 128 threads per walker, in 16 groups of 8 lanes; lane r of a group holds row r
 // of one (determinant, spin) block.  Every lane works in every phase, so no thread waits on
 // a barrier while a few others factorise, and no thread holds a whole matrix in registers:
-//   1. Gauss-Jordan elimination with partial pivoting on [A | I] in FP64 registers, the pivot
-//      row found by a group reduction and broadcast by shuffles.  The rows are not swapped:
+//   1. Gauss-Jordan elimination with partial pivoting, in place, in FP64 registers, the pivot
+//      row found by a group reduction and broadcast by shuffles.  (Column c of the row takes the
+//      inverse's column of the pivot row once c is eliminated: the numbers of the elimination of
+//      [A | I] with two thirds of its FP64 operations and shuffles.)  The rows are not swapped:
 //      the lane that supplies column c's pivot ends with row c of C = A^-1.  The unused rows
 //      receive the updates of an LU factorisation, so the pivots are those of the one-thread
 //      LU (log|det| agrees with it to rounding, 1e-14 in log|psi| measured).  The same lanes
 //      form the Laplacian trace tr(C lap A) in FP64 and store C as double-FP32 rows.
-//   2. Tangent items (block, coordinate): lane r forms row r of B = C d_t A in double-FP32
+//   2. Tangent items (block, two coordinates): lane r forms row r of B = C d_t A in double-FP32
 //      arithmetic (the operations of the one-thread items: from the same C they give the
 //      same entries), then g = tr B and q = tr(B^2) from the rows staged in shared memory
-//      and a double-FP32 reduction over the group.
+//      and a double-FP32 reduction over the group.  The two coordinates are the two words of
+//      packed FP32 instructions: half the issue slots for the same roundings.
+//      N2, 4096 walkers: [A | I] and one coordinate per instruction 2.30 ms, this 1.74 (Si-, 1031
+//      walkers: 1.24 -> 0.84); what is left is FP64 and the chains of the double-FP32 sums.
 //   3. The determinant terms are combined and E_L assembled as in k_det_energy.
 constexpr int kGrpN = 8;                 // rows per group (largest block of this kernel)
 constexpr int kGrpCP = kGrpN + 1;        // padded row of a staged C copy (floats)
-constexpr int kGrpBS = 2 * kGrpN + 1;    // padded row of a staged B row (high, low words)
+constexpr int kGrpBS = kGrpN + 1;        // padded row of a staged B row (pairs: two coordinates)
 
 __host__ __device__ inline size_t smem_det_energy_grp(int N, int K) {
   const int NM = 2 * K, NC = 3 * N;
   return sizeof(double) * ((size_t)2 * NM * NC + 3 * NM + (size_t)K * NC + 2 * K + 128) +
-         sizeof(float) * ((size_t)NM * 2 * kGrpN * kGrpCP + 16 * 8 * kGrpBS);
+         sizeof(float) * ((size_t)NM * 2 * kGrpN * kGrpCP + 2 * 16 * 8 * kGrpBS);
+}
+
+// (s, e) = a - np, the rounding error of the difference in e; np holds the negated second term
+// (packed FP32 has no negated operand: products are formed negated and subtracted, the same roundings).
+__device__ __forceinline__ void ff2_two_diff(uint64_t a, uint64_t np, uint64_t& s, uint64_t& e) {
+  s = tc::sub_f2(a, np);
+  const uint64_t bb = tc::sub_f2(s, a);
+  e = tc::sub_f2(tc::sub_f2(a, tc::sub_f2(s, bb)), tc::add_f2(np, bb));
 }
 
 // (h, l) += the (h, l) of the lane `off` away (double-FP32 sum, error-free on the high words)
-__device__ __forceinline__ void ff_add_xor(float& h, float& l, int off) {
-  const float oh = __shfl_xor_sync(0xffffffffu, h, off), ol = __shfl_xor_sync(0xffffffffu, l, off);
-  float s, e;
-  ff_two_sum(h, oh, s, e);
+__device__ __forceinline__ void ff2_add_xor(uint64_t& h, uint64_t& l, int off) {
+  const uint64_t oh = __shfl_xor_sync(0xffffffffu, h, off), ol = __shfl_xor_sync(0xffffffffu, l, off);
+  const uint64_t s = tc::add_f2(h, oh), bb = tc::sub_f2(s, h);
+  const uint64_t e = tc::add_f2(tc::sub_f2(h, tc::sub_f2(s, bb)), tc::sub_f2(oh, bb));
   h = s;
-  l = __fadd_rn(__fadd_rn(l, ol), e);
+  l = tc::add_f2(tc::add_f2(l, ol), e);
 }
 
-// Row r of B = C D for an M x M block: M double-FP32 accumulators (the operations of
-// tangent_item_ff's inner loop, in the same order).
-template <int M>
-__device__ __forceinline__ void ff_row(const float* __restrict__ chr, const float* __restrict__ clr,
-                                       const float* __restrict__ D, float (&bh)[kGrpN], float (&bl)[kGrpN]) {
-#pragma unroll
-  for (int j = 0; j < M; ++j) { bh[j] = 0.f; bl[j] = 0.f; }
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    const float ch = chr[m], cl = clr[m];
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const float d = __ldg(D + m * M + j);
-      const float p = __fmul_rn(ch, d);
-      const float pe = __fmaf_rn(ch, d, -p);
-      float s, e;
-      ff_two_sum(bh[j], p, s, e);
-      bh[j] = s;
-      bl[j] = __fmaf_rn(cl, d, __fadd_rn(bl[j], __fadd_rn(e, pe)));
-    }
-  }
-}
-
-// The same row for two consecutive tangent slabs of a block (D1 = D0 + M^2): the C row is
-// read once and the two sets of accumulators are independent (twice the instruction-level
-// parallelism of ff_row).
+// Row r of B = C D for two consecutive tangent slabs of an M x M block (D1 = D0 + M^2), the slabs in
+// the words of a pair: M double-FP32 accumulators each, the operations and order of
+// tangent_item_ff's inner loop.
 template <int M>
 __device__ __forceinline__ void ff_row2(const float* __restrict__ chr, const float* __restrict__ clr,
-                                        const float* __restrict__ D0, float (&bh0)[kGrpN], float (&bl0)[kGrpN],
-                                        float (&bh1)[kGrpN], float (&bl1)[kGrpN]) {
+                                        const float* __restrict__ D0, uint64_t (&bh)[kGrpN], uint64_t (&bl)[kGrpN]) {
   const float* D1 = D0 + M * M;
 #pragma unroll
-  for (int j = 0; j < M; ++j) { bh0[j] = 0.f; bl0[j] = 0.f; bh1[j] = 0.f; bl1[j] = 0.f; }
-#pragma unroll
   for (int m = 0; m < M; ++m) {
-    const float ch = chr[m], cl = clr[m];
+    const float c = chr[m], l = clr[m];
+    const uint64_t ch = tc::pack_f2(c, c), nch = tc::pack_f2(-c, -c), cl = tc::pack_f2(l, l);
 #pragma unroll
     for (int j = 0; j < M; ++j) {
-      const float d0 = __ldg(D0 + m * M + j), d1 = __ldg(D1 + m * M + j);
-      const float p0 = __fmul_rn(ch, d0), p1 = __fmul_rn(ch, d1);
-      const float pe0 = __fmaf_rn(ch, d0, -p0), pe1 = __fmaf_rn(ch, d1, -p1);
-      float s0, e0, s1, e1;
-      ff_two_sum(bh0[j], p0, s0, e0);
-      ff_two_sum(bh1[j], p1, s1, e1);
-      bh0[j] = s0;
-      bh1[j] = s1;
-      bl0[j] = __fmaf_rn(cl, d0, __fadd_rn(bl0[j], __fadd_rn(e0, pe0)));
-      bl1[j] = __fmaf_rn(cl, d1, __fadd_rn(bl1[j], __fadd_rn(e1, pe1)));
+      const uint64_t d = tc::pack_f2(__ldg(D0 + m * M + j), __ldg(D1 + m * M + j));
+      const uint64_t np = tc::mul_f2(nch, d), pe = tc::fma_f2(ch, d, np);
+      uint64_t sum, e;
+      ff2_two_diff(bh[j], np, sum, e);
+      bh[j] = sum;
+      bl[j] = tc::fma_f2(cl, d, tc::add_f2(bl[j], tc::add_f2(e, pe)));
     }
   }
 }
@@ -535,7 +520,7 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
   double* rho = lapk + K;                                 // [K]
   double* red = rho + K;                                  // [128]
   float* Cs = (float*)(red + 128);                        // [NM][2][8][9]: rows of C, high then low words
-  float* Bs = Cs + NM * 2 * kGrpN * kGrpCP;               // [16 groups][8 rows][17]: B rows of an item
+  uint64_t* Bs = (uint64_t*)(Cs + NM * 2 * kGrpN * kGrpCP);               // [16 groups][8 rows][9 pairs]: B rows of an item
   const float* Phi = (const float*)a.Phi + (int64_t)w * a.PW;
   const int64_t blk_off[2] = {0, (int64_t)K * T * ns[0] * ns[0]};
   const int lane = tid & 31, gid = tid >> 3, rr = tid & 7;
@@ -547,12 +532,9 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
     const bool live = p < NM;
     const int n = live ? ns[p & 1] : 0;
     const float* Ab = Phi + blk_off[p & 1] + (int64_t)(p >> 1) * T * n * n;     // value slab of the block
-    double av[kGrpN], vv[kGrpN];
+    double av[kGrpN];
 #pragma unroll
-    for (int j = 0; j < kGrpN; ++j) {
-      av[j] = (rr < n && j < n) ? widen<double, float>(Ab[rr * n + j]) : 0.0;
-      vv[j] = j == rr ? 1.0 : 0.0;
-    }
+    for (int j = 0; j < kGrpN; ++j) av[j] = (rr < n && j < n) ? widen<double, float>(Ab[rr * n + j]) : 0.0;
     bool used = rr >= n, singular = false;
     int mycol = -1, pc[kGrpN];
     double mant = 1.0;
@@ -571,12 +553,9 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
       }
       pc[c] = li;
       if (col && key == 0ull) singular = true;
-      double pa[kGrpN], pv[kGrpN];
+      double pa[kGrpN];
 #pragma unroll
-      for (int j = 0; j < kGrpN; ++j) {
-        pa[j] = j >= c ? __shfl_sync(0xffffffffu, av[j], gbase + li) : 0.0;
-        pv[j] = __shfl_sync(0xffffffffu, vv[j], gbase + li);
-      }
+      for (int j = 0; j < kGrpN; ++j) pa[j] = __shfl_sync(0xffffffffu, av[j], gbase + li);
       if (col && !singular) {
         const double piv = pa[c];
         const double rp = 1.0 / piv;
@@ -586,20 +565,15 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
         int e2;
         mant = frexp(mant, &e2);
         expo += e2;
-        // (only the columns right of c of the A part are read again)
         if (rr == li) {
 #pragma unroll
-          for (int j = c + 1; j < kGrpN; ++j) av[j] = pa[j] * rp;
-#pragma unroll
-          for (int j = 0; j < kGrpN; ++j) vv[j] = pv[j] * rp;
+          for (int j = 0; j < kGrpN; ++j) av[j] = j == c ? rp : pa[j] * rp;
           used = true;
           mycol = c;
         } else {
           const double f = av[c] * rp;
 #pragma unroll
-          for (int j = c + 1; j < kGrpN; ++j) av[j] -= f * pa[j];
-#pragma unroll
-          for (int j = 0; j < kGrpN; ++j) vv[j] -= f * pv[j];
+          for (int j = 0; j < kGrpN; ++j) av[j] = j == c ? -f : av[j] - f * pa[j];
         }
       }
     }
@@ -632,6 +606,10 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
       float* ch = Cs + ((int64_t)(p * 2) * kGrpN + row) * kGrpCP;
       float* cl = ch + kGrpN * kGrpCP;
       const float* Dl = Phi + blk_off[p & 1] + (int64_t)(p >> 1) * T * n * n + (int64_t)(T - 1) * n * n;
+      double* vv = (double*)Bs + (gid * 8 + rr) * kGrpBS;       // the row in the order of its columns
+#pragma unroll
+      for (int m = 0; m < kGrpN; ++m)
+        if (m < n) vv[pc[m]] = av[m];
 #pragma unroll
       for (int m = 0; m < kGrpN; ++m) {
         if (m < n) {
@@ -659,10 +637,10 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
     const int tr0 = live ? 2 * (it - p * NP2) : 0;
     const bool two = tr0 + 1 < NC;
     const int n = live ? ns[p & 1] : 0;
-    float bh0[kGrpN], bl0[kGrpN], bh1[kGrpN], bl1[kGrpN];
+    uint64_t bh[kGrpN], bl[kGrpN];                        // (zero bits: 0.f, 0.f)
 #pragma unroll
-    for (int j = 0; j < kGrpN; ++j) { bh0[j] = 0.f; bl0[j] = 0.f; bh1[j] = 0.f; bl1[j] = 0.f; }
-    float* brow = Bs + (gid * 8 + rr) * kGrpBS;
+    for (int j = 0; j < kGrpN; ++j) { bh[j] = 0; bl[j] = 0; }
+    uint64_t* brow = Bs + (gid * 8 + rr) * kGrpBS;
     {
       // the orbital tangents are read once, from DRAM: start the pair of blocks this group
       // takes two steps later on its way into L2 (up to four 128-byte lines)
@@ -675,66 +653,68 @@ __global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict
       }
     }
     if (rr < n) {
-      // (a block's last odd coordinate runs its pair on the same slab twice and keeps one)
+      // (a block's last odd coordinate is the second word of its pair and keeps no other)
       const float* D = Phi + blk_off[p & 1] + (int64_t)(p >> 1) * T * n * n + (int64_t)(1 + tr0 - (two ? 0 : 1)) * n * n;
       const float* chr = Cs + ((int64_t)(p * 2) * kGrpN + rr) * kGrpCP;
       const float* clr = chr + kGrpN * kGrpCP;
       switch (n) {
-        case 1: ff_row2<1>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        case 2: ff_row2<2>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        case 3: ff_row2<3>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        case 4: ff_row2<4>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        case 5: ff_row2<5>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        case 6: ff_row2<6>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        case 7: ff_row2<7>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-        default: ff_row2<8>(chr, clr, D, bh0, bl0, bh1, bl1); break;
-      }
-      if (!two) {
-#pragma unroll
-        for (int j = 0; j < kGrpN; ++j) { bh0[j] = bh1[j]; bl0[j] = bl1[j]; }
+        case 1: ff_row2<1>(chr, clr, D, bh, bl); break;
+        case 2: ff_row2<2>(chr, clr, D, bh, bl); break;
+        case 3: ff_row2<3>(chr, clr, D, bh, bl); break;
+        case 4: ff_row2<4>(chr, clr, D, bh, bl); break;
+        case 5: ff_row2<5>(chr, clr, D, bh, bl); break;
+        case 6: ff_row2<6>(chr, clr, D, bh, bl); break;
+        case 7: ff_row2<7>(chr, clr, D, bh, bl); break;
+        default: ff_row2<8>(chr, clr, D, bh, bl); break;
       }
     }
-    // g: this row's diagonal entry; q: sum_j B[rr][j] B[j][rr]; the rows of the first slab,
-    // then of the second, pass through the group's staging rows
-    float g0h = 0.f, g0l = 0.f, q0h = 0.f, q0l = 0.f, g1h = 0.f, g1l = 0.f, q1h = 0.f, q1l = 0.f;
-    const float* bcol = Bs + (gid * 8) * kGrpBS + 2 * rr;
+    // g: this row's diagonal entry; q: sum_j B[rr][j] B[j][rr]; the high words, then the low words,
+    // pass through the group's staging rows
+    uint64_t gh = 0, gl = 0, qh = 0, ql = 0, ch[kGrpN], cl[kGrpN];
+    const uint64_t* bcol = Bs + (gid * 8) * kGrpBS + rr;
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
-      float(&bh)[kGrpN] = half ? bh1 : bh0;
-      float(&bl)[kGrpN] = half ? bl1 : bl0;
       if (rr < n) {
 #pragma unroll
-        for (int j = 0; j < kGrpN; ++j) {
-          brow[2 * j] = bh[j];
-          brow[2 * j + 1] = bl[j];
-        }
+        for (int j = 0; j < kGrpN; ++j) brow[j] = half ? bl[j] : bh[j];
       }
       __syncwarp();
-      float gh = 0.f, gl = 0.f, qh = 0.f, ql = 0.f;
       if (rr < n) {
-        gh = bcol[rr * kGrpBS];
-        gl = bcol[rr * kGrpBS + 1];
+        (half ? gl : gh) = bcol[rr * kGrpBS];
 #pragma unroll
         for (int j = 0; j < kGrpN; ++j)
-          if (j < n) ff_fma_acc(bh[j], bl[j], bcol[j * kGrpBS], bcol[j * kGrpBS + 1], 1.f, qh, ql);
+          if (j < n) (half ? cl : ch)[j] = bcol[j * kGrpBS];
       }
       __syncwarp();
-      if (half) { g1h = gh; g1l = gl; q1h = qh; q1l = ql; } else { g0h = gh; g0l = gl; q0h = qh; q0l = ql; }
+    }
+    if (rr < n) {
+      const uint64_t minus = tc::pack_f2(-1.f, -1.f);
+#pragma unroll
+      for (int j = 0; j < kGrpN; ++j)
+        if (j < n) {                                      // ff_fma_acc of both words
+          const uint64_t nb = tc::mul_f2(bh[j], minus), np = tc::mul_f2(nb, ch[j]);
+          const uint64_t pe = tc::fma_f2(bh[j], cl[j], tc::fma_f2(bl[j], ch[j], tc::fma_f2(bh[j], ch[j], np)));
+          uint64_t sum, e;
+          ff2_two_diff(qh, np, sum, e);
+          qh = sum;
+          ql = tc::add_f2(ql, tc::add_f2(pe, e));
+        }
     }
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) {
-      ff_add_xor(g0h, g0l, off);
-      ff_add_xor(q0h, q0l, off);
-      ff_add_xor(g1h, g1l, off);
-      ff_add_xor(q1h, q1l, off);
+      ff2_add_xor(gh, gl, off);
+      ff2_add_xor(qh, ql, off);
     }
     if (live && rr == 0) {
-      gt[p * NC + tr0] = make_float2(g0h, g0l);
-      qt[p * NC + tr0] = make_float2(q0h, q0l);
-      if (two) {
-        gt[p * NC + tr0 + 1] = make_float2(g1h, g1l);
-        qt[p * NC + tr0 + 1] = make_float2(q1h, q1l);
-      }
+      float h0, h1, l0, l1;
+      tc::unpack_f2(gh, h0, h1);
+      tc::unpack_f2(gl, l0, l1);
+      if (two) gt[p * NC + tr0] = make_float2(h0, l0);
+      gt[p * NC + tr0 + (two ? 1 : 0)] = make_float2(h1, l1);
+      tc::unpack_f2(qh, h0, h1);
+      tc::unpack_f2(ql, l0, l1);
+      if (two) qt[p * NC + tr0] = make_float2(h0, l0);
+      qt[p * NC + tr0 + (two ? 1 : 0)] = make_float2(h1, l1);
     }
   }
   __syncthreads();
