@@ -24,8 +24,12 @@
  *     reported by fn_sync() as FN_ERR_NUMERIC.
  *   - Precision modes fix the dtypes:
  *       FN_FP64        params double, walkers double, all arithmetic FP64;
- *       FN_FP32        params float,  walkers float,  all arithmetic FP32
- *                      (energies accumulated and returned in FP64);
+ *       FN_FP32        params float,  walkers float,  arithmetic to FP32 accuracy:
+ *                      FP32 sums and products (the tangent pass with h1 a
+ *                      multiple of 128 forms them on the tensor cores, each
+ *                      operand split into three BF16 parts), the determinant
+ *                      stage of few electrons in FP64; energies accumulated
+ *                      and returned in FP64;
  *       FN_BF16_MIXED  params float,  walkers float; stream-layer and
  *                      Laplacian-tangent contractions on tcgen05 tensor cores
  *                      with BF16 operands and FP32 accumulation; elementwise

@@ -10,6 +10,7 @@
 //   k_spin_means_bf16  spin means of a BF16 stream-layer output (next mean-field input)
 //   simt::launch_gemm / launch_layer / launch_orbitals (fn_simt.cu)  FP32/FP64 mean-field
 //                      term U [hbar_up, hbar_dn] + b, stream layer and orbitals
+//   x3 kernels (fn_x3.cu)  the same for FP32 tangent passes with h1 a multiple of 128
 //   k_envelope_values  envelope values per (electron, orbital) for the tensor-core orbitals
 //   k_orbital_fixup    envelope-derivative terms of the full pass's orbitals
 #include <algorithm>
@@ -166,7 +167,7 @@ void launch_prep_params(const fn_system* s, const void* params, bool full, cudaS
 // One kernel for the layer-0 rows h0 = [r_i - R_m, |r_i - R_m|], their tangents, and the spin means
 // of both (Hbar0[t][w][spin * 4M + 4m + a]).  A thread takes one (electron, nucleus) of the CTA's
 // walkers: the FP64 root and quotients are formed once and shared through shared memory (two kernels
-// formed them twice with 4 warps per SM: 137 us for N2 at 4096 walkers with tangents, 27 us without),
+// formed them twice with 4 warps per SM: N2 at 4096 walkers with tangents 137 us, now 51),
 // and every group of four values leaves as one vector.
 constexpr int kFeatThreads = 256;
 template <typename Act> struct alignas(4 * sizeof(Act) > 16 ? 16 : 4 * sizeof(Act)) Act4 { Act v[4]; };
@@ -937,7 +938,7 @@ __device__ __forceinline__ void env_jet(int aniso, const Cmp* par, int ld, const
 // A thread keeps one (electron, orbital) and walks over the walkers; the envelope parameters of the
 // CTA's orbitals sit in shared memory, transposed so that consecutive orbitals read consecutive
 // words, and a walker's electron-nucleus distances are formed once per CTA (as FP64 differences in
-// every thread they took half of the kernel's time).  N2, 4096 walkers: 0.36 -> @FX@ ms.
+// every thread they took half of the kernel's time).  N2, 4096 walkers: 0.36 -> 0.25 ms.
 template <typename Cmp, typename PhiT, typename Wlk>
 __global__ void __launch_bounds__(256) k_orbital_fixup(const Wlk* __restrict__ r, const double* __restrict__ nuc,
                                                        Shape sh, OrbArgs a, const Cmp* __restrict__ orbP, int slots) {
