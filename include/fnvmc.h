@@ -28,7 +28,8 @@
  *                      FP32 sums and products (the tangent pass with h1 a
  *                      multiple of 128 forms them on the tensor cores, each
  *                      operand split into three BF16 parts), the determinant
- *                      stage of few electrons in FP64; energies accumulated
+ *                      stage of few electrons, and of gradients with at most
+ *                      8 electrons a spin, in FP64; energies accumulated
  *                      and returned in FP64;
  *       FN_BF16_MIXED  params float,  walkers float; stream-layer and
  *                      Laplacian-tangent contractions on tcgen05 tensor cores

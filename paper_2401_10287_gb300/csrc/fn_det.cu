@@ -13,7 +13,8 @@
 //       grad log|psi| = sum_k rho_k g_k,
 //       lap log|psi| = sum_k rho_k (lap_k + |g_k|^2) - |grad log|psi||^2,
 //   * E_L = -1/2 (|grad|^2 + lap) + V_ee + V_ne + V_nn (Eqs. 2-3).
-// All of it runs in the Det type (FP64 in the FP64 and BF16-mixed modes).
+// All of it runs in the Det type (FP64 in the FP64 and BF16-mixed modes); FP32 mode takes FP64 for
+// the energies of few electrons and for the gradient's seeds of blocks of at most 8 x 8.
 #include <algorithm>
 #include <climits>
 #include <cstdlib>
@@ -924,10 +925,12 @@ __global__ void __launch_bounds__(128, 3) k_det_value_small(Shape sh, DetArgs a)
   }
 }
 
-// Gradient's value pass, FP64 blocks of at most 8 x 8: log|psi| as in k_det_value_small, and the
-// backward seed rho_k A^{-T}.  One thread inverts one block in registers (Gauss-Jordan in place,
-// partial pivoting by predicated row swaps; the column permutation of the inverse goes into
-// the store addresses), 128 / (2K) walkers per CTA.  The factors in shared memory with two
+// Gradient's value pass, blocks of at most 8 x 8 in FP64 (in every mode): log|psi| as in
+// k_det_value_small, and the backward seed rho_k A^{-T}.  One thread inverts one block in registers
+// (Gauss-Jordan in place, partial pivoting by predicated row swaps; the column permutation of the
+// inverse goes into the store addresses), 128 / (2K) walkers per CTA.  FP32 mode takes it because rho
+// from FP32 logarithms of D_k is off by 6e-8 |log D_k| and the inverse by its own roundings (N2, 1024
+// walkers, worst of 20 gradients: 1.4e-5 of the norm with the FP32 stage, 1.2e-5 with this).  The factors in shared memory with two
 // substitutions per column took 488 us for the 131072 7 x 7 blocks of 4096 N2 walkers, bound by the
 // latency of 8 warps per SM; in registers they take 269 us (n^3 multiply-adds are about 80 us of the
 // FP64 pipe, the rest is the predicated swaps and scattered 8-byte stores).
@@ -979,8 +982,8 @@ struct GjStep<NN, NN> {
 };
 
 // out[i n + j] = (A^{-1})[j][i]; det A = mant 2^expo (mant = 0 and a zero inverse if singular)
-template <int NN, typename PhiT>
-__device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, double* __restrict__ out, double* mant_out,
+template <int NN, typename PhiT, typename Out>
+__device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, Out* __restrict__ out, double* mant_out,
                                             int* expo_out) {
   double a[NN][NN], mant = 1.0;
   int piv[NN], expo = 0;
@@ -988,7 +991,8 @@ __device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, double*
 #pragma unroll
   for (int i = 0; i < NN; ++i)
 #pragma unroll
-    for (int j = 0; j < NN; ++j) a[i][j] = widen<double, PhiT>(Ag[i * NN + j]);
+    for (int j = 0; j < NN; ++j)   // (FP32 mode keeps subnormal entries, which the bitwise widening drops)
+      a[i][j] = sizeof(Out) == 4 ? (double)Ag[i * NN + j] : widen<double, PhiT>(Ag[i * NN + j]);
   GjStep<NN, 0>::run(a, piv, mant, expo, singular);
   // the row swaps of A are column swaps of its inverse, undone last to first: column c of `a` is
   // column col[c] of A^{-1}
@@ -1008,12 +1012,12 @@ __device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, double*
 #pragma unroll
   for (int c = 0; c < NN; ++c)
 #pragma unroll
-    for (int j = 0; j < NN; ++j) out[col[c] * NN + j] = singular ? 0.0 : a[j][c];
+    for (int j = 0; j < NN; ++j) out[col[c] * NN + j] = (Out)(singular ? 0.0 : a[j][c]);
   *mant_out = singular ? 0.0 : mant;
   *expo_out = singular ? 0 : expo;
 }
 
-template <typename PhiT>
+template <typename PhiT, typename Out>
 __global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) {
   pdl_wait();
   pdl_launch();
@@ -1023,24 +1027,24 @@ __global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) 
   const int wl = threadIdx.x / NM, p = threadIdx.x % NM, w0 = blockIdx.x * per_cta, w = w0 + wl;
   const int ns[2] = {sh.n_up, sh.n_dn};
   const int64_t dn_off = (int64_t)K * ns[0] * ns[0], per = dn_off + (int64_t)K * ns[1] * ns[1];
-  double* io = (double*)a.inv_out;
+  Out* io = (Out*)a.inv_out;
   if (wl < per_cta && w < sh.B) {
     const int k = p >> 1, sp = p & 1, n = ns[sp];
     const int64_t off = (sp ? dn_off : 0) + (int64_t)k * n * n;
     const PhiT* A = (const PhiT*)a.Phi + (int64_t)w * a.PW + off;
-    double* out = io + (int64_t)w * per + off;
+    Out* out = io + (int64_t)w * per + off;
     double* m = mt2 + threadIdx.x;
     int* e = ex2 + threadIdx.x;
     switch (n) {
       case 0: *m = 1.0; *e = 0; break;
-      case 1: invert_regs<1, PhiT>(A, out, m, e); break;
-      case 2: invert_regs<2, PhiT>(A, out, m, e); break;
-      case 3: invert_regs<3, PhiT>(A, out, m, e); break;
-      case 4: invert_regs<4, PhiT>(A, out, m, e); break;
-      case 5: invert_regs<5, PhiT>(A, out, m, e); break;
-      case 6: invert_regs<6, PhiT>(A, out, m, e); break;
-      case 7: invert_regs<7, PhiT>(A, out, m, e); break;
-      default: invert_regs<8, PhiT>(A, out, m, e); break;
+      case 1: invert_regs<1, PhiT, Out>(A, out, m, e); break;
+      case 2: invert_regs<2, PhiT, Out>(A, out, m, e); break;
+      case 3: invert_regs<3, PhiT, Out>(A, out, m, e); break;
+      case 4: invert_regs<4, PhiT, Out>(A, out, m, e); break;
+      case 5: invert_regs<5, PhiT, Out>(A, out, m, e); break;
+      case 6: invert_regs<6, PhiT, Out>(A, out, m, e); break;
+      case 7: invert_regs<7, PhiT, Out>(A, out, m, e); break;
+      default: invert_regs<8, PhiT, Out>(A, out, m, e); break;
     }
   }
   __syncthreads();
@@ -1070,10 +1074,10 @@ __global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) 
   // scale by rho_k, consecutive elements per lane (the inverses of this CTA are in L2)
   const int nw = min(per_cta, sh.B - w0);
   for (int v = 0; v < nw; ++v) {
-    double* o = io + (int64_t)(w0 + v) * per;
+    Out* o = io + (int64_t)(w0 + v) * per;
     for (int e = threadIdx.x; e < (int)per; e += blockDim.x) {
       const int k = e < dn_off ? e / (ns[0] * ns[0]) : (e - (int)dn_off) / (ns[1] * ns[1]);
-      o[e] *= rho[v * K + k];
+      o[e] = (Out)(rho[v * K + k] * (double)o[e]);
     }
   }
 }
@@ -1322,9 +1326,9 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
     const int per_cta = 128 / (2 * K);
     launch_k(ov, k_det_value_small<Det, PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0,
         st, sh, a);
-  } else if (std::is_same<Det, double>::value && nmax <= 8) {
+  } else if (nmax <= 8) {
     const int per_cta = 128 / (2 * K);
-    launch_k(ov, k_det_seed_small<PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st, sh, a);
+    launch_k(ov, k_det_seed_small<PhiT, Det>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st, sh, a);
   } else {
     const int threads = (int)round_up(2 * K, 32);
     const size_t vsmem = smem_det_value(sizeof(Det), nmax, K, keep_inverse);

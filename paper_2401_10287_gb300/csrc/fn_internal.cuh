@@ -115,7 +115,7 @@ inline size_t smem_det_energy(int det_bytes, int nmax, int N, int K, bool split 
                               2 * K + 128) + sizeof(int) * (size_t)nmax * ST +
          (split ? sizeof(float) * 2 * (size_t)nmax * nmax * ST : 0);
 }
-// k_det_value (value passes with more than 8 electrons of a spin, and the gradient's pass with inverses)
+// k_det_value (value passes and gradients with more than 8 electrons of a spin)
 inline size_t smem_det_value(int det_bytes, int nmax, int K, bool inv) {
   const int threads = (int)round_up(2 * K, 32);
   return (size_t)det_bytes * ((size_t)(inv ? 2 : 1) * nmax * nmax * threads + (size_t)nmax * threads + 5 * K) +

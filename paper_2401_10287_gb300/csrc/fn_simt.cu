@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(32 * WM) k_layer(Shape sh, LayerArgs a, int wp
   pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V, LDY = Tl::BN + V;
+  constexpr bool TWO = sizeof(T) == 4 && !FULL;                 // (with tangents the registers hold h and sum z^2)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* ys = (T*)(smem_raw + Tl::kRingBytes);                      // [BM][LDY] staged outputs
   // column tiles run fastest, so that the CTAs that share input rows run together
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(32 * WM) k_layer(Shape sh, LayerArgs a, int wp
     if (++lk == nk) { lk = 0; Xl += xslab; }
   };
   T hv[FULL ? TM : 1][FULL ? TN : 1], sq[FULL ? TM : 1][FULL ? TN : 1];
-  auto done = [&](const Acc<T, TM, TN>& acc, int t) {
+  auto done = [&](const Acc<T, TM, TN, TWO>& acc, int t) {
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int rl = r0 + 4 * i;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(32 * WM) k_layer(Shape sh, LayerArgs a, int wp
       // the barrier of the next slab's first stage orders these reads before the next staging
     }
   };
-  stream<Tl, T, TM, TN>(smem_raw, nk, sh.T, load, done);
+  stream<Tl, T, TM, TN, TWO>(smem_raw, nk, sh.T, load, done);
 }
 
 template <typename T, int TM, int TN, int WM>
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(32 * WM) k_orbitals(Shape sh, OrbArgs a, int s
   pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V, LDY = Tl::BN + V;
+  constexpr bool TWO = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* ys = (T*)(smem_raw + Tl::kRingBytes);                      // [BM][LDY]
   T* ds = ys + Tl::BM * LDY;                                    // value pass: [BM][3 M] electron - nucleus
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(32 * WM) k_orbitals(Shape sh, OrbArgs a, int s
         rows, (const T*)a.wT[spin], n_ko, n0, n_ko);
   };
   const int r0 = lane_row0<Tl>(), poff = spin ? a.K * sh.n_up : 0, ldp = a.K * sh.N;
-  auto done = [&](const Acc<T, TM, TN>& acc, int) {
+  auto done = [&](const Acc<T, TM, TN, TWO>& acc, int) {
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int rl = r0 + 4 * i;
@@ -297,7 +299,7 @@ __global__ void __launch_bounds__(32 * WM) k_orbitals(Shape sh, OrbArgs a, int s
       Phi[wl * a.PW + ((int64_t)k * sh.T + t) * nn + i * n_s + jj] = ys[(wl * n_s + jj) * LDY + c];
     }
   };
-  stream<Tl, T, TM, TN>(smem_raw, nk, 1, load, done);
+  stream<Tl, T, TM, TN, TWO>(smem_raw, nk, 1, load, done);
 }
 
 template <typename T, int TM, int TN, int WM>
@@ -361,6 +363,7 @@ __global__ void __launch_bounds__(32 * WM) k_gemm(GemmArgs<T> g) {
   pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V;
+  constexpr bool TWO = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nct = (g.N + Tl::BN - 1) / Tl::BN, n0 = (blockIdx.x % nct) * Tl::BN;
   const int64_t m0 = (int64_t)(blockIdx.x / nct) * Tl::BM;
@@ -375,7 +378,7 @@ __global__ void __launch_bounds__(32 * WM) k_gemm(GemmArgs<T> g) {
         g.lda, (kb0 + s) * Tl::BK, g.K, rows, g.B, g.ldb, n0, g.N);
   };
   const int r0 = lane_row0<Tl>();
-  auto done = [&](const Acc<T, TM, TN>& acc, int) {
+  auto done = [&](const Acc<T, TM, TN, TWO>& acc, int) {
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int rl = r0 + 4 * i;
@@ -407,7 +410,7 @@ __global__ void __launch_bounds__(32 * WM) k_gemm(GemmArgs<T> g) {
       }
     }
   };
-  stream<Tl, T, TM, TN>(smem_raw, nk, 1, load, done);
+  stream<Tl, T, TM, TN, TWO>(smem_raw, nk, 1, load, done);
 }
 
 template <typename T, int TM, int TN, int WM>

@@ -105,21 +105,26 @@ __device__ __forceinline__ void load_stage(unsigned char* stage, RowSrc rows_src
   }
 }
 
-template <typename T, int TM, int TN> struct Acc;
+template <typename T, int TM, int TN, bool TWO> struct Acc;
 
-// FP32: accumulators as pairs of adjacent columns
-template <int TM, int TN>
-struct Acc<float, TM, TN> {
-  uint64_t v[TM][TN / 2];
+// FP32: accumulators as pairs of adjacent columns.  TWO: sums in two levels, each stage's products
+// from zero in v and then added to s, so that a contraction of k terms rounds like one of 16 and one
+// of k / 16 terms instead of one chain of k.  The value passes need it: the determinants multiply the
+// roundings of their matrices by the inverse, and one chain over k = 128 .. 256 was most of the
+// error of an FP32 gradient.  One packed addition per 16 FMAs; the first product of a stage is a
+// multiplication, so nothing is cleared between stages.
+template <int TM, int TN, bool TWO>
+struct Acc<float, TM, TN, TWO> {
+  uint64_t v[TM][TN / 2], s[TWO ? TM : 1][TWO ? TN / 2 : 1];
   __device__ __forceinline__ void clear() {
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int p = 0; p < TN / 2; ++p) v[i][p] = 0ull;
+      for (int p = 0; p < TN / 2; ++p) (TWO ? s[TWO ? i : 0][TWO ? p : 0] : v[i][p]) = 0ull;
   }
   __device__ __forceinline__ float get(int i, int j) const {
     float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v[i][j >> 1]));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(TWO ? s[TWO ? i : 0][TWO ? j >> 1 : 0] : v[i][j >> 1]));
     return (j & 1) ? hi : lo;
   }
   // sa: this lane's row 0 of the stage's A tile; sb: this lane's column 0 of the B tile
@@ -145,16 +150,25 @@ struct Acc<float, TM, TN> {
           const float s = kk ? a[i].y : a[i].x;
           asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(s));
 #pragma unroll
-          for (int p = 0; p < TN / 2; ++p)
-            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v[i][p]) : "l"(aa), "l"(b[p]));
+          for (int p = 0; p < TN / 2; ++p) {
+            if (TWO && k == 0 && kk == 0)
+              asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v[i][p]) : "l"(aa), "l"(b[p]));
+            else
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v[i][p]) : "l"(aa), "l"(b[p]));
+          }
         }
       }
     }
+    if constexpr (TWO)
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int p = 0; p < TN / 2; ++p) asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s[i][p]) : "l"(v[i][p]));
   }
 };
 
-template <int TM, int TN>
-struct Acc<double, TM, TN> {
+template <int TM, int TN, bool TWO>
+struct Acc<double, TM, TN, TWO> {
   double v[TM][TN];
   __device__ __forceinline__ void clear() {
 #pragma unroll
@@ -199,8 +213,8 @@ template <typename Tl> __device__ __forceinline__ int lane_col(int j) {
 
 // Streams stages 0 .. n_stages - 1 through the ring: load(stage index, buffer) issues one
 // stage's copies, done(acc, slab) is called after every `nk` stages with the finished
-// accumulators (cleared afterwards).
-template <typename Tl, typename T, int TM, int TN, typename Load, typename Done>
+// accumulators (cleared afterwards).  TWO: two-level FP32 sums.
+template <typename Tl, typename T, int TM, int TN, bool TWO, typename Load, typename Done>
 __device__ __forceinline__ void stream(unsigned char* ring, int nk, int n_slabs, Load load, Done done) {
   const int total = nk * n_slabs;
 #pragma unroll
@@ -208,7 +222,7 @@ __device__ __forceinline__ void stream(unsigned char* ring, int nk, int n_slabs,
     if (s < total) load(s, ring + s * Tl::kStageBytes);
     cp_commit();
   }
-  Acc<T, TM, TN> acc;
+  Acc<T, TM, TN, TWO> acc;
   acc.clear();
   const int a_off = lane_row0<Tl>() * kRowPad, b_off = Tl::kABytes + lane_col<Tl>(0) * (int)sizeof(T);
   int buf = 0, kb = 0, slab = 0;
