@@ -189,6 +189,15 @@ __device__ __forceinline__ void st4_split(Act* p, int64_t lo, double a, double b
   }
 }
 
+// BF16 storage: zero low parts of a tangent's values.  The layer product takes the low parts of a
+// tangent from the k-block of the pair columns on, and where the width of h is not a multiple of 64
+// that block begins in h, whose tangents have none: what an earlier call of another batch size left
+// there would be added.
+template <typename Act>
+__device__ __forceinline__ void st4_zero_lo(Act* p, int64_t lo) {
+  if constexpr (SplitValue<Act>::value) st4(p + lo, 0.0, 0.0, 0.0, 0.0);
+}
+
 template <typename Act, typename Wlk>
 __global__ void __launch_bounds__(kFeatThreads) k_features(const Wlk* __restrict__ r, const double* __restrict__ nuc,
                                                            Shape sh, Act* __restrict__ X0, int ldx,
@@ -216,10 +225,12 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(const Wlk* __restrict
       const int t = 1 + 3 * i + c;
       const double u0 = c == 0, u1 = c == 1, u2 = c == 2;
       st4(x + t * xslab, u0, u1, u2, q[c]);
+      st4_zero_lo(x + t * xslab, T * xslab);
       st4_split(hb + t * hslab, T * hslab, u0 * inv, u1 * inv, u2 * inv, q[c] * inv);
       st4_split(ho + t * hslab, T * hslab, 0.0, 0.0, 0.0, 0.0);
     }
     st4(x + (T - 1) * xslab, 0.0, 0.0, 0.0, 2.0 / dist);
+    st4_zero_lo(x + (T - 1) * xslab, T * xslab);
   }
   __syncthreads();
   for (int e = threadIdx.x; e < nw * 2 * M; e += blockDim.x) {
@@ -241,7 +252,9 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(const Wlk* __restrict
   for (int e = threadIdx.x; e < (T - 2) * per_t; e += blockDim.x) {
     const int t = e / per_t, k = e - t * per_t, m = k % M, wi = k / M, wl = wi / N, i = wi - wl * N;
     if (t / 3 == i) continue;
-    st4(X0 + (1 + t) * xslab + tile_row(w0 + wl, i, N, sh.wpt) * ldx + 4 * m, 0.0, 0.0, 0.0, 0.0);
+    Act* x = X0 + (1 + t) * xslab + tile_row(w0 + wl, i, N, sh.wpt) * ldx + 4 * m;
+    st4(x, 0.0, 0.0, 0.0, 0.0);
+    st4_zero_lo(x, T * xslab);
   }
 }
 
@@ -838,6 +851,16 @@ __global__ void __launch_bounds__(256) k_pair_full_mma(const Wlk* __restrict__ r
         __nv_bfloat16* o = Xl + t * slab + ei * ldx;
         st2(o, m0, m1);
         st2_lo(o + lo_slab, m0, m1);
+      }
+    }
+    // the low parts of the tangents of h that share the first k-block of the pair columns are zero
+    // (as in k_features, which writes those of layer 0): 8 columns per lane
+    const int z8 = l > 0 ? (a.col0[l] & 63) >> 3 : 0;
+    if (z8) {
+      __nv_bfloat16* Z = (__nv_bfloat16*)a.X[l] + (a.col0[l] & ~63) + xrow0 * ldx + lo_slab + slab;
+      for (int e = threadIdx.x; e < n_i * (sh.T - 1) * z8; e += blockDim.x) {
+        const int c8 = e % z8, q = e / z8, ei = q % n_i, t = q / n_i;
+        *(uint4*)(Z + t * slab + ei * ldx + 8 * c8) = make_uint4(0u, 0u, 0u, 0u);
       }
     }
     if (l == a.L - 1) break;
