@@ -54,7 +54,7 @@ void launch_energy_weights(const fn_system* s, int B, const double* e_local, dou
 
 // ---- column sums (atomic) -------------------------------------------------------------
 template <typename T, typename Cmp>
-__global__ void k_colsum(const T* __restrict__ src, int64_t rows, int64_t lds, int cols, Cmp* __restrict__ dst) {
+__global__ void k_colsum(const T* src, int64_t rows, int64_t lds, int cols, Cmp* __restrict__ dst) {
   pdl_wait();
   pdl_launch();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -90,7 +90,7 @@ static void colsum(const fn_system* s, cudaStream_t st, const T* src, int64_t ro
 // as zero.  32 x 32 tiles pass through shared memory, so the row-major reads and the
 // transposed writes are both coalesced.
 template <typename Tin>
-__global__ void k_bf16_copy_T(Shape sh, const Tin* __restrict__ in, int64_t ld_in, int cols,
+__global__ void k_bf16_copy_T(Shape sh, const Tin* in, int64_t ld_in, int cols,
                               __nv_bfloat16* __restrict__ out, int64_t ld_out, __nv_bfloat16* __restrict__ outT) {
   pdl_wait();
   pdl_launch();
@@ -118,7 +118,7 @@ __global__ void k_bf16_copy_T(Shape sh, const Tin* __restrict__ in, int64_t ld_i
 // The transposed copy alone of a BF16 matrix, in 64 x 64 tiles: 16-byte loads of 8 columns and
 // 16-byte stores of 8 rows (the 2-byte accesses of the kernel above take 51 us for the 58368 x 320
 // input of an N2 layer at 4096 walkers, 75 MB in all).
-__global__ void __launch_bounds__(256) k_bf16_T(Shape sh, const __nv_bfloat16* __restrict__ in, int64_t ld_in, int cols,
+__global__ void __launch_bounds__(256) k_bf16_T(Shape sh, const __nv_bfloat16* in, int64_t ld_in, int cols,
                                                 __nv_bfloat16* __restrict__ outT) {
   pdl_wait();
   pdl_launch();
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(256) k_bf16_T(Shape sh, const __nv_bfloat16* _
     const int64_t r = r0 + k;
     const int rr = (int)(r % kTileRows), q = (int)(r / kTileRows), wl = rr / sh.N;
     const bool valid = wl < sh.wpt && q * sh.wpt + wl < sh.B && c < cols;
-    const uint4 v = valid ? __ldg((const uint4*)(in + r * ld_in + c)) : make_uint4(0u, 0u, 0u, 0u);
+    const uint4 v = valid ? *(const uint4*)(in + r * ld_in + c) : make_uint4(0u, 0u, 0u, 0u);
     const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int m = 0; m < 4; ++m) *(uint32_t*)&tile[k][8 * (e & 7) + 2 * m] = u[m];
@@ -194,7 +194,7 @@ struct OrbBwdArgs {
 // zeroes the other spin's columns there, and accumulates the envelope gradients in
 // registers (MM >= the number of nuclei bounds the unrolled per-nucleus arrays).
 template <typename Cmp, typename Det, typename Wlk, int MM>
-__global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbBwdArgs a) {
+__global__ void k_orb_bwd(const Wlk* r, const double* __restrict__ nuc, Shape sh, OrbBwdArgs a) {
   pdl_wait();
   pdl_launch();
   const int spin = blockIdx.y;
@@ -313,7 +313,7 @@ __global__ void k_orb_bwd(const Wlk* __restrict__ r, const double* __restrict__ 
 
 // ---- stream layers -------------------------------------------------------------------
 template <typename Cmp>
-__global__ void k_bwd_tanh(Shape sh, int h1, const Cmp* __restrict__ dH, const Cmp* __restrict__ act,
+__global__ void k_bwd_tanh(Shape sh, int h1, const Cmp* dH, const Cmp* act,
                            Cmp* __restrict__ dZ, Cmp* __restrict__ dZw) {
   pdl_wait();
   pdl_launch();
@@ -334,8 +334,8 @@ __global__ void k_bwd_tanh(Shape sh, int h1, const Cmp* __restrict__ dH, const C
 // BF16 mode: dz leaves only as the operands of the tensor-core products, row-major and transposed
 // BF16 (rows without an electron are zero), and as the walker sums.  One 128-row tile (whole
 // walkers) x 32 columns per CTA; separate tanh, copy and clear passes moved dz four times.
-__global__ void __launch_bounds__(256) k_bwd_tanh_bf16(Shape sh, int h1, const float* __restrict__ dH,
-                                                       const float* __restrict__ act, __nv_bfloat16* __restrict__ out,
+__global__ void __launch_bounds__(256) k_bwd_tanh_bf16(Shape sh, int h1, const float* dH,
+                                                       const float* act, __nv_bfloat16* __restrict__ out,
                                                        __nv_bfloat16* __restrict__ outT, float* __restrict__ dZw) {
   pdl_wait();
   pdl_launch();
@@ -381,8 +381,8 @@ __global__ void __launch_bounds__(256) k_bwd_tanh_bf16(Shape sh, int h1, const f
 // Four columns per thread where the width allows (the divisions and index arithmetic of one
 // element per thread took 77 us for 176 MB).
 template <typename Cmp, int V>
-__global__ void k_bwd_dh(Shape sh, int h1, int ldx, int d_h, const Cmp* __restrict__ dX,
-                         const Cmp* __restrict__ dHbar, Cmp* __restrict__ dH) {
+__global__ void k_bwd_dh(Shape sh, int h1, int ldx, int d_h, const Cmp* dX,
+                         const Cmp* dHbar, Cmp* __restrict__ dH) {
   pdl_wait();
   pdl_launch();
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -418,7 +418,7 @@ struct PairBwdArgs {
 };
 
 template <typename Cmp, typename Wlk>
-__global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* __restrict__ r, Shape sh, PairBwdArgs a) {
+__global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* r, Shape sh, PairBwdArgs a) {
   pdl_wait();
   pdl_launch();
   __shared__ Cmp red[4][32][33];
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(128) k_pair_bwd(const Wlk* __restrict__ r, Sha
 // of 33 words kept the kernel at 32 % issue and 0.2 TB/s).  N2, 4096 walkers, four levels: 1.39 ->
 // 0.81 ms.
 template <typename Wlk>
-__global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r, Shape sh, PairBwdArgs a) {
+__global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* r, Shape sh, PairBwdArgs a) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -666,11 +666,11 @@ __global__ void __launch_bounds__(128) k_pair_bwd_mma(const Wlk* __restrict__ r,
   if (in_h2) atomicAdd((float*)a.gc + lane, dc);
 }
 
-__global__ void k_widen_bf16(int64_t n8, const uint4* __restrict__ in, float4* __restrict__ out) {
+__global__ void k_widen_bf16(int64_t n8, const uint4* in, float4* __restrict__ out) {
   pdl_wait();
   pdl_launch();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint4 v = __ldg(in + i);
+    const uint4 v = in[i];
     out[2 * i] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
                              __uint_as_float(v.y & 0xffff0000u));
     out[2 * i + 1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
@@ -680,7 +680,7 @@ __global__ void k_widen_bf16(int64_t n8, const uint4* __restrict__ in, float4* _
 
 // ---- internal layout -> blob order ---------------------------------------------------
 template <typename Par, typename Cmp>
-__global__ void k_unprep(Par* __restrict__ blob, const CopyDesc* __restrict__ descs, const Cmp* __restrict__ gradc) {
+__global__ void k_unprep(Par* __restrict__ blob, const CopyDesc* __restrict__ descs, const Cmp* gradc) {
   pdl_wait();
   pdl_launch();
   const CopyDesc d = descs[blockIdx.y];

@@ -278,7 +278,7 @@ __device__ __forceinline__ bool tangent_item_split(const float* Ch, const float*
 // g_t = tr(C d_t A), q_t = tr((C d_t A)^2) and tr(C lap A); then the determinant terms
 // are combined and E_L assembled.
 template <typename Det, typename Wlk, typename PhiT>
-__global__ void __launch_bounds__(128) k_det_energy(const Wlk* __restrict__ r, const double* __restrict__ nuc,
+__global__ void __launch_bounds__(128) k_det_energy(const Wlk* r, const double* __restrict__ nuc,
                                                     Shape sh, DetArgs a) {
   pdl_wait();
   pdl_launch();
@@ -489,7 +489,7 @@ __device__ __forceinline__ void ff_row2(const float* __restrict__ chr, const flo
     const uint64_t ch = tc::pack_f2(c, c), nch = tc::pack_f2(-c, -c), cl = tc::pack_f2(l, l);
 #pragma unroll
     for (int j = 0; j < M; ++j) {
-      const uint64_t d = tc::pack_f2(__ldg(D0 + m * M + j), __ldg(D1 + m * M + j));
+      const uint64_t d = tc::pack_f2(D0[m * M + j], D1[m * M + j]);
       const uint64_t np = tc::mul_f2(nch, d), pe = tc::fma_f2(ch, d, np);
       uint64_t sum, e;
       ff2_two_diff(bh[j], np, sum, e);
@@ -500,7 +500,7 @@ __device__ __forceinline__ void ff_row2(const float* __restrict__ chr, const flo
 }
 
 template <typename Wlk>
-__global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* __restrict__ r, const double* __restrict__ nuc,
+__global__ void __launch_bounds__(128, 4) k_det_energy_grp(const Wlk* r, const double* __restrict__ nuc,
                                                            Shape sh, DetArgs a) {
   pdl_wait();
   pdl_launch();
@@ -1091,7 +1091,7 @@ __global__ void __launch_bounds__(128, 2) k_det_seed_small(Shape sh, DetArgs a) 
 // the K terms and assembles E_L.  128 / (2K) walkers share a CTA, so a small walker does not
 // occupy a CTA of idle threads.
 template <int NMAX, typename Det, typename Wlk, typename PhiT>
-__global__ void __launch_bounds__(128) k_det_energy_small(const Wlk* __restrict__ r, const double* __restrict__ nuc,
+__global__ void __launch_bounds__(128) k_det_energy_small(const Wlk* r, const double* __restrict__ nuc,
                                                           Shape sh, DetArgs a) {
   pdl_wait();
   pdl_launch();

@@ -10,6 +10,10 @@ namespace fn {
 // touches memory, and lets the next kernel of the stream begin only after that: when a kernel
 // runs, everything before its predecessor is complete, so its prologue (barriers, tensor
 // memory, weights prepared at least two kernels earlier) may overlap the predecessor's tail.
+// A kernel that started early was alive while its inputs were written, so they are not read-only for
+// its lifetime: what earlier kernels of the stream write is read with ordinary loads, never with __ldg
+// or through a `const * __restrict__` parameter (which may become loads of read-only data).  The handle's
+// own uploads (nuclei, atoms, copy descriptors, Hartree-Fock orbitals) may be.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

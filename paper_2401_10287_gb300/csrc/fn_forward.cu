@@ -29,7 +29,7 @@ namespace fn {
 // ---------------------------------------------------------------------------------------
 
 template <typename Par, typename Cmp>
-__global__ void k_prep(const Par* __restrict__ blob, const CopyDesc* __restrict__ descs, int n_desc,
+__global__ void k_prep(const Par* blob, const CopyDesc* __restrict__ descs, int n_desc,
                        Cmp* __restrict__ prep, __nv_bfloat16* __restrict__ prep16) {
   pdl_wait();
   pdl_launch();
@@ -199,7 +199,7 @@ __device__ __forceinline__ void st4_zero_lo(Act* p, int64_t lo) {
 }
 
 template <typename Act, typename Wlk>
-__global__ void __launch_bounds__(kFeatThreads) k_features(const Wlk* __restrict__ r, const double* __restrict__ nuc,
+__global__ void __launch_bounds__(kFeatThreads) k_features(const Wlk* r, const double* __restrict__ nuc,
                                                            Shape sh, Act* __restrict__ X0, int ldx,
                                                            Act* __restrict__ Hbar, int wpb) {
   pdl_wait();
@@ -345,7 +345,7 @@ __device__ __forceinline__ void pair_matvec(const Cmp* __restrict__ sWl, const C
 // (-d/dr_i / n_spin) to the layer input, adjacent columns from adjacent threads.
 
 template <typename Act, typename Cmp, typename Wlk>
-__global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Shape sh, PairArgs a, int ib) {
+__global__ void __launch_bounds__(256) k_pair_full(const Wlk* r, Shape sh, PairArgs a, int ib) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(256) k_pair_full(const Wlk* __restrict__ r, Sh
 // memory between layers; per layer the spin means over j are summed per
 // (i, spin, channel), then every pair is advanced through the next pair layer.
 template <typename Act, typename Cmp, typename Wlk>
-__global__ void __launch_bounds__(512) k_pair_value(const Wlk* __restrict__ r, Shape sh, PairArgs a) {
+__global__ void __launch_bounds__(512) k_pair_value(const Wlk* r, Shape sh, PairArgs a) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(512) k_pair_value(const Wlk* __restrict__ r, S
 // The value slab adds its low part (slab T of Y); every mean is stored as a hi/lo pair
 // (the low part of slab t in slab T + t of Hbar).  One thread per (slab, walker, spin, 8
 // columns); a warp reads 512 contiguous bytes of a row.
-__global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* __restrict__ Y, int ldy, int h1,
+__global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* Y, int ldy, int h1,
                                   __nv_bfloat16* __restrict__ Hbar) {
   pdl_wait();
   pdl_launch();
@@ -558,7 +558,7 @@ __global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* __restrict__ Y,
         uint4 u[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          u[k] = i0 + k < hi ? __ldg((const uint4*)(base + (int64_t)(i0 + k) * ldy)) : make_uint4(0u, 0u, 0u, 0u);
+          u[k] = i0 + k < hi ? *(const uint4*)(base + (int64_t)(i0 + k) * ldy) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           if (i0 + k >= hi) break;
@@ -589,7 +589,7 @@ __global__ void k_spin_means_bf16(Shape sh, const __nv_bfloat16* __restrict__ Y,
 }
 
 // The same in FP32 (after the FP32 tensor-core layer): one thread per (slab, walker, spin, 4 columns).
-__global__ void k_spin_means_f32(Shape sh, const float* __restrict__ Y, int ldy, int h1, float* __restrict__ Hbar) {
+__global__ void k_spin_means_f32(Shape sh, const float* Y, int ldy, int h1, float* __restrict__ Hbar) {
   pdl_wait();
   pdl_launch();
   const int g4 = h1 >> 2;
@@ -607,7 +607,7 @@ __global__ void k_spin_means_f32(Shape sh, const float* __restrict__ Y, int ldy,
       float4 u[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        u[k] = i0 + k < hi ? __ldg((const float4*)(base + (int64_t)(i0 + k) * ldy)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        u[k] = i0 + k < hi ? *(const float4*)(base + (int64_t)(i0 + k) * ldy) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int k = 0; k < 4; ++k) { acc.x += u[k].x; acc.y += u[k].y; acc.z += u[k].z; acc.w += u[k].w; }
     }
@@ -644,7 +644,7 @@ __device__ __forceinline__ void stage_pair_weights_bf16(const PairArgs& a, __nv_
 // conflict-free pairs (a row stride of 33 words cost a third of the wavefronts).
 // N2, 4096 walkers: 213 -> 194 us.
 template <typename Wlk>
-__global__ void __launch_bounds__(128) k_pair_value_mma(const Wlk* __restrict__ r, Shape sh, PairArgs a) {
+__global__ void __launch_bounds__(128) k_pair_value_mma(const Wlk* r, Shape sh, PairArgs a) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(128) k_pair_value_mma(const Wlk* __restrict__ 
 // slots: its loops carry pairs and pointers by increments instead of dividing and multiplying
 // for each.  N2, 4096 walkers: 1.58 -> 1.14 ms.
 template <typename Wlk>
-__global__ void __launch_bounds__(256) k_pair_full_mma(const Wlk* __restrict__ r, Shape sh, PairArgs a, int ib) {
+__global__ void __launch_bounds__(256) k_pair_full_mma(const Wlk* r, Shape sh, PairArgs a, int ib) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -963,8 +963,8 @@ __device__ __forceinline__ void env_jet(int aniso, const Cmp* par, int ld, const
 // words, and a walker's electron-nucleus distances are formed once per CTA (as FP64 differences in
 // every thread they took half of the kernel's time).  N2, 4096 walkers: 0.36 -> 0.25 ms.
 template <typename Cmp, typename PhiT, typename Wlk>
-__global__ void __launch_bounds__(256) k_orbital_fixup(const Wlk* __restrict__ r, const double* __restrict__ nuc,
-                                                       Shape sh, OrbArgs a, const Cmp* __restrict__ orbP, int slots) {
+__global__ void __launch_bounds__(256) k_orbital_fixup(const Wlk* r, const double* __restrict__ nuc,
+                                                       Shape sh, OrbArgs a, const Cmp* orbP, int slots) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char fix_smem[];
@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(256) k_orbital_fixup(const Wlk* __restrict__ r
 
 // Envelope values of every (electron, own-spin orbital), one thread each (tensor-core pass).
 template <typename Wlk>
-__global__ void k_envelope_values(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh, OrbArgs a,
+__global__ void k_envelope_values(const Wlk* r, const double* __restrict__ nuc, Shape sh, OrbArgs a,
                                   float* __restrict__ envv) {
   pdl_wait();
   pdl_launch();
@@ -1069,7 +1069,7 @@ __global__ void k_envelope_values(const Wlk* __restrict__ r, const double* __res
 // Grid: (ceil(K (n_up^2 + n_dn^2) / 256), rows striding over the walkers).  Shared memory
 // per spin s: sigma [M][9 or 1][K n_s], then pi [M][K n_s].
 template <typename Wlk>
-__global__ void k_envelope_values_smem(const Wlk* __restrict__ r, const double* __restrict__ nuc, Shape sh,
+__global__ void k_envelope_values_smem(const Wlk* r, const double* __restrict__ nuc, Shape sh,
                                        OrbArgs a, float* __restrict__ envv) {
   pdl_wait();
   pdl_launch();

@@ -805,8 +805,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
         res[pc][1] = make_uint4(0u, 0u, 0u, 0u);
         if (pc < npieces && has_res) {
           const int cb = (2 * (pc >> 1) + ehalf) * 32 + (pc & 1) * 16;
-          res[pc][0] = __ldg(xres + cb / 8);
-          res[pc][1] = __ldg(xres + cb / 8 + 1);
+          res[pc][0] = xres[cb / 8];
+          res[pc][1] = xres[cb / 8 + 1];
         }
       }
       cp_async_wait_all();

@@ -31,7 +31,7 @@ struct AdamCoef {
 };
 
 template <typename P>
-__global__ void k_adam(int64_t n, P* __restrict__ p, const P* __restrict__ g, P* __restrict__ m,
+__global__ void k_adam(int64_t n, P* __restrict__ p, const P* g, P* __restrict__ m,
                        P* __restrict__ v, AdamCoef<P> c, int* __restrict__ status) {
   pdl_wait();
   pdl_launch();
@@ -51,7 +51,7 @@ __global__ void k_adam(int64_t n, P* __restrict__ p, const P* __restrict__ g, P*
 }
 
 template <typename P>
-__global__ void k_sgd(int64_t n, P* __restrict__ p, const P* __restrict__ g, P lr, int* __restrict__ status) {
+__global__ void k_sgd(int64_t n, P* __restrict__ p, const P* g, P lr, int* __restrict__ status) {
   pdl_wait();
   pdl_launch();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -258,7 +258,7 @@ void launch_clip_energy(const fn_system* s, int B, const double* e, double width
 // statistics or the weights are formed.  One CTA, FP64, fixed summation order.
 constexpr int kStatThreads = 1024;
 
-__global__ void __launch_bounds__(kStatThreads) k_energy_moments(int B, const double* __restrict__ e,
+__global__ void __launch_bounds__(kStatThreads) k_energy_moments(int B, const double* e,
                                                                   double* __restrict__ mom) {
   pdl_wait();
   pdl_launch();
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kStatThreads) k_energy_moments(int B, const do
   }
 }
 
-__global__ void k_energy_stats(const double* __restrict__ mom, double* __restrict__ stats, int* __restrict__ status) {
+__global__ void k_energy_stats(const double* mom, double* __restrict__ stats, int* __restrict__ status) {
   pdl_wait();
   pdl_launch();
   const double n = mom[0], mean = mom[1] / n;
@@ -297,7 +297,7 @@ __global__ void k_energy_stats(const double* __restrict__ mom, double* __restric
   if (!isfinite(mean) || !isfinite(var)) atomicOr(status, kStatusNonFinite);
 }
 
-__global__ void k_energy_weights_from(int B, const double* __restrict__ e, const double* __restrict__ mom,
+__global__ void k_energy_weights_from(int B, const double* e, const double* mom,
                                       double* __restrict__ w) {
   pdl_wait();
   pdl_launch();

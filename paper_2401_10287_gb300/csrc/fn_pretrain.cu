@@ -18,8 +18,8 @@ constexpr int kHfPerFunction = 18;   // centre[3], powers[3], exponents[6], weig
 
 // One warp per walker, one lane per electron (N <= 32).
 template <typename Det, typename PhiT, typename Wlk>
-__global__ void k_pretrain_seed(const Wlk* __restrict__ r, Shape sh, const double* __restrict__ hf, int nbf,
-                                const PhiT* __restrict__ Phi, int64_t PW, int K, Det* __restrict__ dPhi,
+__global__ void k_pretrain_seed(const Wlk* r, Shape sh, const double* __restrict__ hf, int nbf,
+                                const PhiT* Phi, int64_t PW, int K, Det* __restrict__ dPhi,
                                 double* __restrict__ cw, double* __restrict__ wloss) {
   pdl_wait();
   pdl_launch();
@@ -74,7 +74,7 @@ __global__ void k_pretrain_seed(const Wlk* __restrict__ r, Shape sh, const doubl
   }
 }
 
-__global__ void k_pretrain_loss(int B, const double* __restrict__ wloss, double* __restrict__ out) {
+__global__ void k_pretrain_loss(int B, const double* wloss, double* __restrict__ out) {
   pdl_wait();
   pdl_launch();
   __shared__ double red[1024];

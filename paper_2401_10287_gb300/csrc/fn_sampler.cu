@@ -32,7 +32,7 @@ __global__ void k_init_walkers(int B, int N, const int* __restrict__ atom, const
 // One thread per Box-Muller pair, i.e. per two coordinates of a walker: the FP64 logarithm, root,
 // sine and cosine are most of the kernel.
 template <typename Wlk>
-__global__ void k_propose(int B, int N, const Wlk* __restrict__ r, Wlk* __restrict__ out, double step,
+__global__ void k_propose(int B, int N, const Wlk* r, Wlk* __restrict__ out, double step,
                           uint64_t seed, uint32_t step_idx, uint64_t walker_offset) {
   pdl_wait();
   pdl_launch();
@@ -50,8 +50,8 @@ __global__ void k_propose(int B, int N, const Wlk* __restrict__ r, Wlk* __restri
 }
 
 template <typename Wlk>
-__global__ void k_accept(int B, int N, Wlk* __restrict__ r, const Wlk* __restrict__ prop, double* __restrict__ lp,
-                         const double* __restrict__ lp_new, uint64_t seed, uint32_t step_idx,
+__global__ void k_accept(int B, int N, Wlk* __restrict__ r, const Wlk* prop, double* __restrict__ lp,
+                         const double* lp_new, uint64_t seed, uint32_t step_idx,
                          uint64_t walker_offset, unsigned long long* __restrict__ accepted) {
   pdl_wait();
   pdl_launch();
