@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(32 * WM) k_gemm(GemmArgs<T> g) {
   pdl_launch();
   using Tl = Tile<T, TM, TN, WM>;
   constexpr int V = Tl::V, G = TN / V;
-  constexpr bool TWO = sizeof(T) == 4;
+  constexpr bool TWO = sizeof(T) == 4 && !AT && !BT;             // the value pass's products
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nct = (g.N + Tl::BN - 1) / Tl::BN, n0 = (blockIdx.x % nct) * Tl::BN;
   const int64_t m0 = (int64_t)(blockIdx.x / nct) * Tl::BM;
