@@ -49,7 +49,10 @@
  *     the same bits.  FN_DET_KERNEL=thread selects, for the BF16 local-energy
  *     determinant stage with blocks of 5 to 8 electrons, one thread per block
  *     instead of 8-lane groups; the results agree to rounding.  Both are read
- *     at every launch.
+ *     at every launch.  FN_LAYER_KERNEL=fma, read when a system is created, keeps
+ *     its FP32 energies with h1 a multiple of 128 off the tensor cores (the FMA
+ *     kernels of the other widths; also taken where those cannot run); the
+ *     results agree to FP32 rounding.
  */
 #ifndef FNVMC_H
 #define FNVMC_H

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <thread>
@@ -11,6 +12,7 @@
 
 #include "fn_internal.cuh"
 #include "fn_small.cuh"
+#include "fn_x3.cuh"
 
 namespace fn {
 
@@ -447,6 +449,10 @@ fn_status fn_create_system(const double* h_nuclei, const double* h_charges, int 
   if (cfg->precision == FN_BF16_MIXED && !tc_available()) {
     set_error("the driver does not provide cuTensorMapEncodeTiled"); fn_destroy_system(s); return FN_ERR_UNSUPPORTED;
   }
+  // FP32 energies of these widths take the tensor cores where those kernels can run, else the FMA pipe,
+  // which covers every width
+  const char* layer = std::getenv("FN_LAYER_KERNEL");
+  if (s->prep.total3 > 0 && ((layer && std::strcmp(layer, "fma") == 0) || !x3::available())) s->prep.total3 = 0;
   *out = s;
   return FN_OK;
 }

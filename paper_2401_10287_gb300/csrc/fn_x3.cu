@@ -517,17 +517,23 @@ void launch_split_weights(const float* blob, const SplitList& list, void* out, c
   launch_k(false, k_split_weights, dim3(32, list.n), 256, 0, st, blob, list, (__nv_bfloat16*)out);
 }
 
+// The register split needs the full launch allocation: a kernel compiled to another count cannot run.
+template <int EPI>
+static bool registers_fit() {
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, k_x3<EPI>) == cudaSuccess) return fa.numRegs == kLaunchRegs;
+  cudaGetLastError();
+  return false;
+}
+
+bool available() {
+  static const bool ok = tc_available() && registers_fit<kLayer>() && registers_fit<kPlain>() && registers_fit<kOrbital>();
+  return ok;
+}
+
 template <int EPI>
 static bool launch(const Args& a, const void* W, int64_t w_rows, const float* X, int64_t ldx, float* Y, int64_t y_cols, int64_t y_rows, int64_t ldy,
                    int sm_count, cudaStream_t st) {
-  // the register split needs the full launch allocation (checked once per kernel)
-  static const bool regs_ok = [] {
-    cudaFuncAttributes fa;
-    const bool ok = cudaFuncGetAttributes(&fa, k_x3<EPI>) == cudaSuccess && fa.numRegs == kLaunchRegs;
-    cudaGetLastError();
-    return ok;
-  }();
-  if (!regs_ok) return false;
   CUtensorMap tb, tx, ty;
   if (!make_map(&tb, W, 3 * (int64_t)a.ldw, w_rows, 3 * (int64_t)a.ldw, kNt)) return false;
   if (Y) {

@@ -32,6 +32,9 @@ struct SplitList {
   int n;
 };
 
+// Whether these kernels can run: the driver encodes tensor maps and every kernel has the registers
+// its split needs.  Decided when a handle is created; without them FP32 passes stay on the FMA pipe.
+bool available();
 void launch_split_weights(const float* blob, const SplitList& list, void* out, cudaStream_t st);
 // false: a tensor map could not be built (nothing launched)
 bool launch_layer(const Shape& sh, const float* X, int ldx, int k_self, const void* W, int ldw, const float* Mterm,
