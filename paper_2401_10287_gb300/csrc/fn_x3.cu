@@ -1,23 +1,29 @@
-// FP32 products on the 5th-generation tensor cores, without loss of precision: the stream
-// layers, the mean-field term and the orbitals of the FP32 local-energy pass.
+// FP32 products on the 5th-generation tensor cores, to FP32 accuracy: the stream layers, the mean-field
+// term and the orbitals of the FP32 local-energy pass.
 //
 // Every FP32 operand is the exact sum of three BF16 parts, x = x0 + x1 + x2 (8 significant
-// bits each).  Of the nine partial products six are kept, x0 w0, x0 w1, x1 w0, x0 w2, x1 w1,
-// x2 w0; the dropped ones are below 2^-25 of the product.  The tensor core adds in FP32 but
-// truncates, so the leading products x0 w0 have an accumulator of their own and the five
-// small ones another: one truncated addition per 16 k instead of one rounded addition per k.
-// Measured against FP64 (1024 x 128, k = 320, tanh-like rows, weights N(0, 1/k)): relative
-// RMS error 2.9e-7, the sequential FP32 FMA chain 3.2e-7; k = 64: 0.8e-7 and 1.5e-7.
+// bits each; rows by truncation, weights by rounding).  Of the nine partial products six are kept,
+// x0 w0, x0 w1, x1 w0, x0 w2, x1 w1, x2 w0.  Truncated rows leave |x1| < 2^-7 |x| and |x2| < 2^-15 |x|,
+// rounded weights |w1| <= 2^-8 |w| and |w2| <= 2^-17 |w|, so the three dropped products are below 2^-22.4
+// of the product (8 million normal pairs: at most 2^-22.6, root mean square 2^-25.7, with the sign of
+// the row's remainder); one FP32 rounding is up to 2^-24.  The tensor core adds in FP32 but truncates,
+// so the leading products x0 w0 have an accumulator of their own and the five small ones another: one
+// truncated addition per 16 k instead of one rounded addition per k.  Measured against FP64 (1024 x
+// 128, k = 320, tanh-like rows, weights N(0, 1/k)): relative RMS error 2.9e-7, the sequential
+// FP32 FMA chain 3.2e-7; k = 64: 0.8e-7 and 1.5e-7.
 //
-// One CTA of 512 threads per SM:
-//   warp 0        TMA: the three parts of a k-block's weights (3 x nt x 64, prepared in BF16)
-//   warp 1        allocates tensor memory; one lane issues five tcgen05.mma per 16 k: x0 times
-//                 the stacked [w0; w1] (N = 2 nt: both accumulators), x1 w0, x1 w1, x2 w0, x0 w2
-//   warps 4..7    read the FP32 rows of the next k-block (any row addresses: gathered electrons
-//                 of one spin), split them and write the parts into the swizzled operand tiles
-//   warps 8..15   epilogue: a TMEM lane quarter and nt / 2 columns each; a warp first moves its
-//                 sums to registers and hands the accumulators back, so that the MMAs of the
-//                 next item run under the rest
+// Infinities: the leading part of an infinite operand is infinite and its further parts are NaN
+// (inf - inf), so an infinite leading sum is the result, as in FP32.
+//
+// One CTA of 640 threads per SM:
+//   warp 0         TMA: the three parts of a k-block's weights (3 x nt x 64, prepared in BF16)
+//   warp 1         allocates tensor memory; one lane issues five tcgen05.mma per 16 k: x0 times
+//                  the stacked [w0; w1] (N = 2 nt: both accumulators), x1 w0, x1 w1, x2 w0, x0 w2
+//   warps 4..11    read the FP32 rows of the next k-block (any row addresses: gathered electrons
+//                  of one spin), split them and write the parts into the swizzled operand tiles
+//   warps 12..19   epilogue: a TMEM lane quarter and nt / 2 columns each; a warp first moves its
+//                  sums to registers and hands the accumulators back, so that the MMAs of the
+//                  next item run under the rest
 // Two stages of 2 x 48 KB operand tiles.  Activations stay FP32 in memory and are split in the
 // kernel: stored parts would move 6 instead of 4 bytes an element.
 //
@@ -335,6 +341,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       fence_after();
       float z[4][16];
       const uint32_t acc = tmem + lane_base + (uint32_t)(buf * 2 * kNt + c0);
+      uint64_t odd = 0;                          // becomes NaN with the first value that is not finite
 #pragma unroll
       for (int pc = 0; pc < 4; ++pc) {
         uint32_t u[16], s[16];
@@ -342,7 +349,25 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_ld16_nowait(acc + kNt + 16 * pc, s);
         tmem_wait_ld32(u, s);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) z[pc][j] = __uint_as_float(u[j]) + __uint_as_float(s[j]);
+        for (int j = 0; j < 16; j += 2) {
+          const uint64_t v = add_f2(pack_f2(__uint_as_float(u[j]), __uint_as_float(u[j + 1])),
+                                    pack_f2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])));
+          odd = fma_f2(v, 0ull, odd);
+          unpack_f2(v, z[pc][j], z[pc][j + 1]);
+        }
+      }
+      float odd0, odd1;
+      unpack_f2(odd, odd0, odd1);
+      if (__any_sync(0xffffffffu, !(odd0 + odd1 == 0.f))) {
+        // An infinite operand has its value in the leading products; its further parts are NaN.
+#pragma unroll
+        for (int pc = 0; pc < 4; ++pc) {
+          uint32_t u[16];
+          tmem_ld16(acc + 16 * pc, u);
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (isinf(__uint_as_float(u[j]))) z[pc][j] = __uint_as_float(u[j]);
+        }
       }
       fence_before();
       __syncwarp();
@@ -504,7 +529,8 @@ __global__ void k_split_weights(const float* __restrict__ blob, SplitList list, 
     if (k < e.len1) v = blob[e.src1 + r * e.src_ld + k];
     else if (k < e.kd) v = blob[e.src2 + r * e.src_ld + (k - e.len1)];
     __nv_bfloat16* o = out + e.dst + r * 3 * e.ldw + k;
-    const __nv_bfloat16 p0 = __float2bfloat16_rn(v);
+    __nv_bfloat16 p0 = __float2bfloat16_rn(v);
+    if (__hisinf(p0) && !isinf(v)) p0 = __float2bfloat16_rz(v);   // the largest finite values stay finite
     const float r1 = v - __bfloat162float(p0);
     const __nv_bfloat16 p1 = __float2bfloat16_rn(r1);
     o[0] = p0;
