@@ -336,7 +336,7 @@ static const char* shared_memory_overflow(const fn_system* s, size_t limit, size
 template <class Mode>
 static void launch_mcmc(const fn_system* s, void* walkers, double* lp, int B, int n_steps, double step_size,
                         uint64_t seed, uint64_t step_offset, int64_t* accept, cudaStream_t st) {
-  if (small_covers(s)) {
+  if (small_covers(s, B)) {
     launch_small_mcmc(s, walkers, lp, B, n_steps, step_size, seed, step_offset, accept, st);
     return;
   }

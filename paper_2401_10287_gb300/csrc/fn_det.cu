@@ -1339,7 +1339,7 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
 
 template <class Mode>
 void launch_log_psi(const fn_system* s, const void* walkers, int B, double* log_psi, int8_t* sign, cudaStream_t st) {
-  if (small_covers(s)) {
+  if (small_covers(s, B)) {
     launch_small_log_psi(s, walkers, B, log_psi, sign, st);
     return;
   }

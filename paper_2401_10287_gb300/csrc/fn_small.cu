@@ -276,9 +276,21 @@ static SmallArgs small_args(const fn_system* s) {
   return a;
 }
 
-bool small_covers(const fn_system* s) {
+// Where it is the faster path (log|psi| and a Metropolis step, against the general kernels, FP64; networks
+// 2 x 16 / 8, 2 x 32 / 8, 4 x 48 / 16, 3 x 64 / 16 and / 32 with 1 to 16 determinants): one or two electrons
+// at every batch (65536 walkers: 1.01 to 2.7 x).  With more, dot products without register tiling lose once
+// the general kernels have CTAs enough: LiH 1.03 to 1.2 x at 2048 to 4096 walkers, 0.75 to 0.92 at 65536;
+// C 1.04 to 1.26 at 2048, 0.63 to 0.94 at 65536; O 1.17 to 1.4 at 1024, 0.88 to 1.05 at 2048, 0.62 to 0.86 at
+// 65536.  At 16 columns the general tiles are half padding: up to four electrons win at every batch (1.15 x),
+// C at 16384 (1.06), O at 4096 (1.08).
+static bool small_wins(int N, int h1, int B) {
+  if (N <= (h1 <= 16 ? 4 : 2)) return true;
+  return (int64_t)B * N <= (h1 <= 16 ? 65536 : 12288);
+}
+
+bool small_covers(const fn_system* s, int B) {
   if (s->cfg.precision != FN_FP64 || s->N > 8 || s->cfg.h1 > 64 || s->cfg.n_dets > 16) return false;
-  return small_layout(small_args(s)).total * sizeof(double) <= 96 * 1024;
+  return small_wins(s->N, s->cfg.h1, B) && small_layout(small_args(s)).total * sizeof(double) <= 96 * 1024;
 }
 
 static void launch(const SmallArgs& a, cudaStream_t st) {
