@@ -441,6 +441,29 @@ void launch_gemm(GemmArgs<T> g, bool at, bool bt, int max_split, int sm_count, c
     *split = (int)std::max<int64_t>(1, std::min<int64_t>({want, (int64_t)max_split, nk / 4}));
     return tile_cost<Tl>(tiles * *split, sm_count, fill, rate) / *split;
   };
+  // FP64: each SM quarter has a pipe of its own that one warp saturates, so a product takes as long as
+  // the busiest SM's warps per quarter; K is split as that comes out shortest, with as few parts as give
+  // it to 2 %.  (Just enough CTAs for the SMs left quarters idle and some SMs with two: the weight
+  // gradients of a 320 x 256 layer ran 160 CTAs of two warps.  Products of the N2 gradient, 1618 walkers:
+  // 39.6 -> 28.6 ms; mean field with one part, 1618 and 3000 rows: 1.26 and 2.15 ms as before.)
+  auto pick64 = [&](auto tile, int* split) {
+    using Tl = decltype(tile);
+    const int64_t tiles = ((g.M + Tl::BM - 1) / Tl::BM) * ((g.N + Tl::BN - 1) / Tl::BN);
+    const int64_t nk = (g.K + Tl::BK - 1) / Tl::BK;
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>({(int64_t)max_split, nk / 4, 256}));
+    constexpr int warps = Tl::kThreads / 32;
+    double best = 0.0;
+    for (int64_t s = 1; s <= most; ++s) {
+      const int64_t per_sm = (tiles * s + sm_count - 1) / sm_count;
+      const double per_quarter = std::max(1.0, per_sm * warps / 4.0);
+      const double cost = per_quarter * (Tl::BM * Tl::BN / warps) * (double)((nk + s - 1) / s);
+      if (s == 1 || cost < 0.98 * best) {
+        best = cost;
+        *split = (int)s;
+      }
+    }
+    return best;
+  };
   int sb, ss;
   if constexpr (sizeof(T) == 4) {
     const double big = pick(Tile<T, 8, 8, 4>{}, 2, 1.0, &sb), small = pick(Tile<T, 4, 4, 2>{}, 4, 0.5, &ss);
@@ -448,7 +471,7 @@ void launch_gemm(GemmArgs<T> g, bool at, bool bt, int max_split, int sm_count, c
     if (big <= small) gemm_cfg<T, 8, 8, 4>(g, at, bt, sb, vec, st);
     else gemm_cfg<T, 4, 4, 2>(g, at, bt, ss, vec, st);
   } else {
-    const double big = pick(Tile<T, 4, 4, 8>{}, 1, 1.0, &sb), small = pick(Tile<T, 4, 4, 2>{}, 1, 1.0, &ss);
+    const double big = pick64(Tile<T, 4, 4, 8>{}, &sb), small = pick64(Tile<T, 4, 4, 2>{}, &ss);
     g.atomic = g.atomic || (big <= small ? sb : ss) > 1;
     if (big <= small) gemm_cfg<T, 4, 4, 8>(g, at, bt, sb, vec, st);
     else gemm_cfg<T, 4, 4, 2>(g, at, bt, ss, vec, st);
