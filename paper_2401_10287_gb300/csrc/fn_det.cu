@@ -992,7 +992,7 @@ __device__ __forceinline__ void invert_regs(const PhiT* __restrict__ Ag, Out* __
   for (int i = 0; i < NN; ++i)
 #pragma unroll
     for (int j = 0; j < NN; ++j)   // (FP32 mode keeps subnormal entries, which the bitwise widening drops)
-      a[i][j] = sizeof(Out) == 4 ? (double)Ag[i * NN + j] : widen<double, PhiT>(Ag[i * NN + j]);
+      a[i][j] = sizeof(Out) == 4 ? widen_all<double, PhiT>(Ag[i * NN + j]) : widen<double, PhiT>(Ag[i * NN + j]);
   GjStep<NN, 0>::run(a, piv, mant, expo, singular);
   // the row swaps of A are column swaps of its inverse, undone last to first: column c of `a` is
   // column col[c] of A^{-1}
@@ -1128,7 +1128,7 @@ __global__ void __launch_bounds__(128) k_det_energy_small(const Wlk* r, const do
       for (int i = 0; i < NMAX; ++i)
 #pragma unroll
         for (int j = 0; j < NMAX; ++j)
-          if (i < n && j < n) M[i][j] = widen<Det, PhiT>(blk[i * n + j]);
+          if (i < n && j < n) M[i][j] = widen_all<Det, PhiT>(blk[i * n + j]);
 #pragma unroll
       for (int i = 0; i < NMAX; ++i) M[i][NMAX + i] = (i < n) ? (Det)1 : (Det)0;
       Det sgn = 1, mant = 1;
@@ -1183,7 +1183,7 @@ __global__ void __launch_bounds__(128) k_det_energy_small(const Wlk* r, const do
             Det s = 0;
 #pragma unroll
             for (int m = 0; m < NMAX; ++m)
-              if (m < n && j < n) s += M[i][NMAX + m] * widen<Det, PhiT>(D[m * n + j]);
+              if (m < n && j < n) s += M[i][NMAX + m] * widen_all<Det, PhiT>(D[m * n + j]);
             Bm[i][j] = s;
           }
         Det g = 0, q = 0;
@@ -1206,7 +1206,7 @@ __global__ void __launch_bounds__(128) k_det_energy_small(const Wlk* r, const do
       for (int i = 0; i < NMAX; ++i)
 #pragma unroll
         for (int j = 0; j < NMAX; ++j)
-          if (i < n && j < n) l += M[j][NMAX + i] * widen<Det, PhiT>(DL[i * n + j]);
+          if (i < n && j < n) l += M[j][NMAX + i] * widen_all<Det, PhiT>(DL[i * n + j]);
       *lt = singular ? (Det)0 : l;
       *qs = singular ? (Det)0 : qsum;
     }

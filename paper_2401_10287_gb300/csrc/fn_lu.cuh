@@ -21,6 +21,16 @@ template <> __device__ __forceinline__ double widen<double, float>(float f) {
   return __hiloint2double((int)hi, (int)lo);
 }
 
+// The same with FP32 subnormals kept: they are scaled into the normal range (exactly) first.
+template <typename Det, typename PhiT> __device__ __forceinline__ Det widen_all(PhiT v) { return (Det)v; }
+template <> __device__ __forceinline__ double widen_all<double, float>(float f) {
+  const bool sub = (__float_as_uint(f) & 0x7F800000u) == 0u;
+  const uint32_t u = __float_as_uint(sub ? f * 0x1p64f : f);
+  const uint32_t ex = (u >> 23) & 0xFFu, sign = u & 0x80000000u, man = u & 0x7FFFFFu;
+  const uint32_t ex64 = ex == 0 ? 0u : (ex == 0xFFu ? 0x7FFu : ex + (sub ? 832u : 896u));
+  return __hiloint2double((int)(sign | (ex64 << 20) | (man >> 3)), (int)(man << 29));
+}
+
 // Pivot search key: |v| as an unsigned integer (the bit patterns of non-negative IEEE
 // numbers order like their values), so the comparisons leave the FP64 pipe alone.
 __device__ __forceinline__ unsigned long long abs_key(double v) {
