@@ -213,8 +213,6 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
   for (int l = 0; l < L; ++l) {
     o_X[l] = take((size_t)Tx * sh.R * s->layer[l].ldx * sizeof(Act));
     o_Hbar[l] = take((size_t)Tx * B * 2 * s->layer[l].d_h * sizeof(Act));
-    o_act[l] = take((size_t)sh.R * h1 * sizeof(Cmp));
-    o_gp[l] = take((size_t)B * N * N * h2 * sizeof(Cmp));
     max_ldx = std::max(max_ldx, s->layer[l].ldx);
     max_dh = std::max(max_dh, s->layer[l].d_h);
   }
@@ -227,6 +225,11 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
   const size_t o_walk2 = take((size_t)B * N * 3 * sizeof(Wlk));
   const size_t o_lp2 = take((size_t)B * sizeof(double));
   const size_t o_scr = take((size_t)B * sizeof(double) * 2);
+  const size_t o_kept = off;                     // activations of the gradient's value pass
+  for (int l = 0; l < L; ++l) {
+    o_act[l] = take((size_t)sh.R * h1 * sizeof(Cmp));
+    o_gp[l] = take((size_t)B * N * N * h2 * sizeof(Cmp));
+  }
   const size_t o_dX = take((size_t)sh.R * max_ldx * sizeof(Cmp));
   const size_t o_dH = take((size_t)sh.R * h1 * sizeof(Cmp));
   const size_t o_dZ = take((size_t)sh.R * h1 * sizeof(Cmp));
@@ -236,8 +239,11 @@ static size_t workspace_layout(fn_system* s, int B, Workspace* ws) {
   const size_t o_dPhi = take((size_t)B * phi_walker_stride(s, 1) * sizeof(Det));
   const size_t o_gradc = take((size_t)s->prep.total * sizeof(Cmp));
   const size_t o_dP = take((size_t)sh.R * s->cfg.n_dets * N * sizeof(Cmp));
-  const size_t o_orbP = take((size_t)sh.R * 4 * s->cfg.n_dets * N * sizeof(Cmp));
-  // FP32/FP64: the envelope values of the full pass take dP's place (a buffer of the gradient)
+  // FP32/FP64: the projections and envelope values of the full pass take the place of gradient buffers
+  // (dX .. dPhi and the kept activations in front of them, and dP): a gradient writes all of them that it reads
+  const size_t orbP_bytes = (size_t)sh.R * 4 * s->cfg.n_dets * N * sizeof(Cmp);
+  const bool shared = !pairs && orbP_bytes <= o_gradc - o_kept;
+  const size_t o_orbP = shared ? o_kept : take(orbP_bytes);
   const size_t o_envv = take(Mode::kMode == FN_BF16_MIXED ? (size_t)sh.R * s->cfg.n_dets * N * sizeof(float) : 0);
   const bool bf16 = Mode::kMode == FN_BF16_MIXED;
   int max_k = 0;

@@ -205,8 +205,9 @@ struct Workspace {
   void* dPhi = nullptr;          // [B][orbital block, value slab] (Det)
   void* gradc = nullptr;         // prepared-layout gradient accumulator (Cmp)
   void* dP = nullptr;            // [R][K (n_up + n_dn)] gradient wrt orbital projections (Cmp)
-  void* orbP = nullptr;          // [R][4][K N] projections for the orbital envelope fix-up (Cmp)
-  void* envv = nullptr;          // envelope values (Cmp): BF16 mode [R][K N], else [K N][R]
+  void* orbP = nullptr;          // [R][4][K N] projections for the orbital envelope fix-up (Cmp); FP32/FP64: in
+                                 // the place of act .. dPhi where it fits
+  void* envv = nullptr;          // envelope values (Cmp): BF16 mode [R][K N], else [K N][R] in the place of dP
   // BF16-mode backward operands for the tensor-core GEMMs
   void* g16 = nullptr;           // [R][max(h1, ldWT)] bf16 copy of dZ or dP
   void* t16a = nullptr;          // [max(k_self, h1)][R] bf16 transposed activations (X_l^T, h_L^T)
