@@ -14,8 +14,8 @@
 //                  BF16 MMAs over all pairs of a walker)
 // In BF16 mode the large GEMMs run on the tensor cores (fn_layer_tc.cu): row-major
 // products directly, weight gradients as split-K products over the electron rows on
-// transposed BF16 copies; FP32 and FP64 take the register-tiled GEMM (fn_simt.cu).  Parameter gradients accumulate in the internal layout and
-// are scattered back to the blob order at the end.
+// transposed BF16 copies; FP32 and FP64 take the register-tiled GEMM (fn_simt.cu).  Parameter
+// gradients accumulate in the internal layout and are scattered back to the blob order at the end.
 #include <algorithm>
 
 #include "fn_device.cuh"
@@ -152,8 +152,7 @@ static void bf16_T(const fn_system* s, cudaStream_t st, const Shape& sh, const v
                    __nv_bfloat16* outT) {
   ProfScope ps(s->prof, kProfBwdMisc, st);
   launch_k(overlap_launches(sh), k_bf16_T, dim3((cols + 63) / 64, (unsigned)(sh.R / 64)), 256, 0, st, sh,
-      (const __nv_bfloat16*)in,
-             ld_in, cols, outT);
+           (const __nv_bfloat16*)in, ld_in, cols, outT);
 }
 
 template <typename Tin>
@@ -162,7 +161,7 @@ static void bf16_copy_T(const fn_system* s, cudaStream_t st, const Shape& sh, co
   ProfScope ps(s->prof, kProfBwdMisc, st);
   dim3 grid((cols + 31) / 32, (unsigned)(sh.R / 32));
   launch_k(overlap_launches(sh), k_bf16_copy_T<Tin>, grid, dim3(32, 8), 0, st, sh, in, ld_in, cols, out, ld_out,
-      outT);
+           outT);
 }
 
 // K splits of a weight-gradient GEMM (K = all rows): about two CTAs per SM, >= 4 k-blocks each.
@@ -706,6 +705,7 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
   const int64_t R = sh.R;
   const int ldp = K * N;
   constexpr int kAnySplit = 1 << 20;             // weight gradients: as many K splits as fill the chip
+  const bool ov = overlap_launches(sh, sizeof(Cmp));
   cudaMemsetAsync(gradc, 0, sizeof(Cmp) * pl.total, st);
   cudaMemsetAsync(ws.dH, 0, sizeof(Cmp) * R * h1, st);
   // orbitals + envelopes: P = h_L w (both spins, every row), then the envelope kernel turns
@@ -751,14 +751,10 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
     const int threads = (int)std::min<int64_t>(1024, round_up((int64_t)K * std::max(s->n_up, s->n_dn), 32));
     dim3 grid((sh.B + a.chunk - 1) / a.chunk, 2);
     ProfScope ps(s->prof, kProfBwdOrb, st);
-    if (s->M <= 2) launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, 2>, grid, threads, 0, st, r, s->d_nuclei,
-        sh, a);
-    else if (s->M <= 4) launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, 4>, grid, threads, 0, st, r,
-        s->d_nuclei, sh, a);
-    else if (s->M <= 8) launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, 8>, grid, threads, 0, st, r,
-        s->d_nuclei, sh, a);
-    else launch_k(overlap_launches(sh, sizeof(Cmp)), k_orb_bwd<Cmp, Det, Wlk, kMaxNuclei>, grid, threads, 0, st, r, s->d_nuclei,
-        sh, a);
+    if (s->M <= 2) launch_k(ov, k_orb_bwd<Cmp, Det, Wlk, 2>, grid, threads, 0, st, r, s->d_nuclei, sh, a);
+    else if (s->M <= 4) launch_k(ov, k_orb_bwd<Cmp, Det, Wlk, 4>, grid, threads, 0, st, r, s->d_nuclei, sh, a);
+    else if (s->M <= 8) launch_k(ov, k_orb_bwd<Cmp, Det, Wlk, 8>, grid, threads, 0, st, r, s->d_nuclei, sh, a);
+    else launch_k(ov, k_orb_bwd<Cmp, Det, Wlk, kMaxNuclei>, grid, threads, 0, st, r, s->d_nuclei, sh, a);
   }
   const int ns[2] = {s->n_up, s->n_dn};
   __nv_bfloat16* g16 = (__nv_bfloat16*)ws.g16;
@@ -814,18 +810,16 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       // operands of the tensor-core products: dZ row-major and transposed, X_l transposed
       {
         ProfScope ps(s->prof, kProfBwdMisc, st);
-        launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_tanh_bf16, dim3(h1 / 32, sh.tiles), 256, 0, st, sh, h1, dH,
-            (const float*)ws.act[l], g16,
-                   t16b, dZw);
+        launch_k(ov, k_bwd_tanh_bf16, dim3(h1 / 32, sh.tiles), 256, 0, st, sh, h1, dH, (const float*)ws.act[l], g16,
+                 t16b, dZw);
       }
       bf16_T(s, st, sh, ws.X[l], d.ldx, d.k_self, t16a);
     } else {
       cudaMemsetAsync(dZ, 0, sizeof(Cmp) * R * h1, st);
       const int64_t n = (int64_t)sh.B * h1;
       ProfScope ps(s->prof, kProfBwdMisc, st);
-      launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_tanh<Cmp>, (unsigned)((n + 255) / 256), 256, 0, st, sh, h1, dH,
-          (const Cmp*)ws.act[l], dZ,
-                 dZw);
+      launch_k(ov, k_bwd_tanh<Cmp>, (unsigned)((n + 255) / 256), 256, 0, st, sh, h1, dH, (const Cmp*)ws.act[l], dZ,
+               dZw);
     }
     // dV_self (internal [k_self][h1]) += X^T dZ
     {
@@ -845,9 +839,8 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       if constexpr (kTc) {
         // the means in FP32 (2 d_h is a multiple of 8), in the buffer their gradient fills below
         const int64_t n8 = (int64_t)sh.B * 2 * d.d_h / 8;
-        launch_k(overlap_launches(sh, sizeof(Cmp)), k_widen_bf16, (unsigned)std::min<int64_t>((n8 + 255) / 256, 8 * s->sm_count),
-            256, 0, st, n8,
-                   (const uint4*)ws.Hbar[l], (float4*)dHbar);
+        launch_k(ov, k_widen_bf16, (unsigned)std::min<int64_t>((n8 + 255) / 256, 8 * s->sm_count), 256, 0, st, n8,
+                 (const uint4*)ws.Hbar[l], (float4*)dHbar);
         Hb = dHbar;
       }
       simt::launch_gemm<Cmp>({2 * d.d_h, h1, sh.B, Hb, 2 * d.d_h, dZw, h1, gradc + pl.UT[l], h1, nullptr, 0, 1}, true, false,
@@ -874,10 +867,8 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       const unsigned blocks = (unsigned)((n + 255) / 256);
       ProfScope ps(s->prof, kProfBwdMisc, st);
       if constexpr (sizeof(Cmp) == 4)
-        if (V == 4) launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_dh<Cmp, 4>, blocks, 256, 0, st, sh, h1, d.ldx, d.d_h, dX,
-            dHbar, dH);
-      if (V == 1) launch_k(overlap_launches(sh, sizeof(Cmp)), k_bwd_dh<Cmp, 1>, blocks, 256, 0, st, sh, h1, d.ldx, d.d_h, dX,
-          dHbar, dH);
+        if (V == 4) launch_k(ov, k_bwd_dh<Cmp, 4>, blocks, 256, 0, st, sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
+      if (V == 1) launch_k(ov, k_bwd_dh<Cmp, 1>, blocks, 256, 0, st, sh, h1, d.ldx, d.d_h, dX, dHbar, dH);
     }
     // two-electron stream level l
     if (L > 1) {
@@ -894,17 +885,15 @@ void launch_backward(const fn_system* s, const void* walkers, const Shape& sh, c
       if (Mode::kMode == FN_BF16_MIXED) {
         const size_t smem = smem_pair_bwd_mma(N);
         cudaFuncSetAttribute(k_pair_bwd_mma<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_k(overlap_launches(sh, sizeof(Cmp)), k_pair_bwd_mma<Wlk>, (unsigned)std::min(sh.B, 6 * s->sm_count), 128, smem,
-            st, r, sh, a);
+        launch_k(ov, k_pair_bwd_mma<Wlk>, (unsigned)std::min(sh.B, 6 * s->sm_count), 128, smem, st, r, sh, a);
       } else {
-        launch_k(overlap_launches(sh, sizeof(Cmp)), k_pair_bwd<Cmp, Wlk>, sh.B, 128, 0, st, r, sh, a);
+        launch_k(ov, k_pair_bwd<Cmp, Wlk>, sh.B, 128, 0, st, r, sh, a);
       }
     }
   }
   dim3 grid(32, s->n_descs);
   ProfScope ps(s->prof, kProfBwdMisc, st);
-  launch_k(overlap_launches(sh, sizeof(Cmp)), k_unprep<Par, Cmp>, grid, 256, 0, st, (Par*)grad, (const CopyDesc*)s->d_descs,
-      gradc);
+  launch_k(ov, k_unprep<Par, Cmp>, grid, 256, 0, st, (Par*)grad, (const CopyDesc*)s->d_descs, gradc);
 }
 
 #define FN_INST(M)                                                                                           \

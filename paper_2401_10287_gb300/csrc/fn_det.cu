@@ -1320,12 +1320,10 @@ void launch_det_energy(const fn_system* s, const void* walkers, const Shape& sh,
     const size_t smem = smem_det_energy(sizeof(Det), nmax, s->N, K,
                                         std::is_same<Det, double>::value && std::is_same<PhiT, float>::value);
     cudaFuncSetAttribute(k_det_energy<Det, Wlk, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_k(ov, k_det_energy<Det, Wlk, PhiT>, sh.B, 128, smem, st, (const Wlk*)walkers,
-        s->d_nuclei, sh, a);
+    launch_k(ov, k_det_energy<Det, Wlk, PhiT>, sh.B, 128, smem, st, (const Wlk*)walkers, s->d_nuclei, sh, a);
   } else if (!keep_inverse && nmax <= 8) {
     const int per_cta = 128 / (2 * K);
-    launch_k(ov, k_det_value_small<Det, PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0,
-        st, sh, a);
+    launch_k(ov, k_det_value_small<Det, PhiT>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st, sh, a);
   } else if (nmax <= 8) {
     const int per_cta = 128 / (2 * K);
     launch_k(ov, k_det_seed_small<PhiT, Det>, (unsigned)((sh.B + per_cta - 1) / per_cta), 128, 0, st, sh, a);

@@ -145,8 +145,7 @@ void launch_prep_params(const fn_system* s, const void* params, bool full, cudaS
   dim3 grid(32, s->n_descs);
   ProfScope ps(s->prof, kProfPrep, st);
   launch_k(true, k_prep<Par, Cmp>, grid, 256, 0, st, (const Par*)params, (const CopyDesc*)s->d_descs, s->n_descs,
-                                         (Cmp*)s->ws.prep,
-                                         (__nv_bfloat16*)s->ws.prep16);
+           (Cmp*)s->ws.prep, (__nv_bfloat16*)s->ws.prep16);
   if (!use_x3<Mode>(s, full)) return;
   x3::SplitList list{};
   const int L = s->cfg.n_layers, h1 = s->cfg.h1, K = s->cfg.n_dets, ns[2] = {s->n_up, s->n_dn};
@@ -1175,11 +1174,10 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         cudaFuncSetAttribute(k_pair_full_mma<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_m);
         launch_k(ov, k_pair_full_mma<Wlk>, (unsigned)blocks_m, 256, smem_m, st, r, sh, pa, ibm);
       } else {
-      const size_t smem = smem_pair_full(sizeof(Cmp), sh.N, L, ib);
-      const int64_t blocks = (int64_t)sh.B * ((sh.N + ib - 1) / ib);
-      cudaFuncSetAttribute(k_pair_full<Act, Cmp, Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      launch_k(ov, k_pair_full<Act, Cmp, Wlk>, (unsigned)blocks, 32 * warps, smem, st, r, sh, pa,
-          ib);
+        const size_t smem = smem_pair_full(sizeof(Cmp), sh.N, L, ib);
+        const int64_t blocks = (int64_t)sh.B * ((sh.N + ib - 1) / ib);
+        cudaFuncSetAttribute(k_pair_full<Act, Cmp, Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        launch_k(ov, k_pair_full<Act, Cmp, Wlk>, (unsigned)blocks, 32 * warps, smem, st, r, sh, pa, ib);
       }
     } else {
       if (Mode::kMode == FN_BF16_MIXED) {
@@ -1241,9 +1239,8 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         ProfScope pm(s->prof, kProfSpinMeans, st);
         const int64_t n = (int64_t)sh.T * sh.B * 2 * (h1 / 8);
         const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)s->sm_count * 64);
-        launch_k(ov, k_spin_means_bf16, blocks, 256, 0, st, sh, (const __nv_bfloat16*)la.Y,
-            la.ldy, h1,
-                                                  (__nv_bfloat16*)la.Hbar_out);
+        launch_k(ov, k_spin_means_bf16, blocks, 256, 0, st, sh, (const __nv_bfloat16*)la.Y, la.ldy, h1,
+                 (__nv_bfloat16*)la.Hbar_out);
       }
       continue;
     }
@@ -1255,8 +1252,7 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         ProfScope pm(s->prof, kProfSpinMeans, st);
         const int64_t n = (int64_t)sh.T * sh.B * 2 * (h1 / 4);
         const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)s->sm_count * 64);
-        launch_k(ov, k_spin_means_f32, blocks, 256, 0, st, sh, (const float*)la.Y, la.ldy, h1,
-            (float*)la.Hbar_out);
+        launch_k(ov, k_spin_means_f32, blocks, 256, 0, st, sh, (const float*)la.Y, la.ldy, h1, (float*)la.Hbar_out);
       }
       continue;
     }
@@ -1288,13 +1284,11 @@ void launch_forward(const fn_system* s, const void* walkers, const Shape& sh, bo
         const unsigned gx = (unsigned)((per_walker + 255) / 256);
         const unsigned gy = (unsigned)std::max(1, std::min(sh.B, (s->sm_count * 8 + (int)gx - 1) / (int)gx));
         cudaFuncSetAttribute(k_envelope_values_smem<Wlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)env_smem);
-        launch_k(ov, k_envelope_values_smem<Wlk>, dim3(gx, gy), 256, env_smem, st, r, s->d_nuclei,
-            sh, oa,
-                   (float*)ws.envv);
+        launch_k(ov, k_envelope_values_smem<Wlk>, dim3(gx, gy), 256, env_smem, st, r, s->d_nuclei, sh, oa,
+                 (float*)ws.envv);
       } else {
-        launch_k(ov, k_envelope_values<Wlk>, (unsigned)((n_env + 255) / 256), 256, 0, st, r,
-            s->d_nuclei, sh, oa,
-                   (float*)ws.envv);
+        launch_k(ov, k_envelope_values<Wlk>, (unsigned)((n_env + 255) / 256), 256, 0, st, r, s->d_nuclei, sh, oa,
+                 (float*)ws.envv);
       }
       const float* wb[2] = {(const float*)oa.g[0], (const float*)oa.g[1]};
       const float* pis[2] = {(const float*)oa.pi[0], (const float*)oa.pi[1]};

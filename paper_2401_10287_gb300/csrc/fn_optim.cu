@@ -85,7 +85,7 @@ void launch_adam(const fn_system* s, void* params, const void* grad, void* m, vo
   c.d2 = (P)(1.0 - pow(beta2, (double)t));
   ProfScope ps(s->prof, kProfOptim, st);
   launch_k(true, k_adam<P>, elementwise_grid(s, s->P), 256, 0, st, s->P, (P*)params, (const P*)grad, (P*)m, (P*)v, c,
-                                                        s->ws.status);
+           s->ws.status);
 }
 
 template <class Mode>
@@ -93,7 +93,7 @@ void launch_sgd(const fn_system* s, void* params, const void* grad, double lr, c
   using P = typename Mode::Par;
   ProfScope ps(s->prof, kProfOptim, st);
   launch_k(true, k_sgd<P>, elementwise_grid(s, s->P), 256, 0, st, s->P, (P*)params, (const P*)grad, (P)lr,
-      s->ws.status);
+           s->ws.status);
 }
 
 // ---- local-energy clipping ------------------------------------------------------------------

@@ -95,10 +95,9 @@ void launch_pretrain_seed(const fn_system* s, const void* walkers, const Shape& 
   const Workspace& ws = s->ws;
   ProfScope ps(s->prof, kProfBwdOrb, st);
   const int warps = 4;
-  launch_k(overlap_launches(sh), k_pretrain_seed<Det, PhiT, Wlk>, (unsigned)((sh.B + warps - 1) / warps),
-      32 * warps, 0, st,
-             (const Wlk*)walkers, sh, s->d_hf, s->hf_nbf, (const PhiT*)ws.Phi, phi_walker_stride(s, 1), s->cfg.n_dets,
-      (Det*)ws.dPhi, ws.scratch_d, ws.scratch_d + sh.B);
+  launch_k(overlap_launches(sh), k_pretrain_seed<Det, PhiT, Wlk>, (unsigned)((sh.B + warps - 1) / warps), 32 * warps,
+           0, st, (const Wlk*)walkers, sh, s->d_hf, s->hf_nbf, (const PhiT*)ws.Phi, phi_walker_stride(s, 1),
+           s->cfg.n_dets, (Det*)ws.dPhi, ws.scratch_d, ws.scratch_d + sh.B);
   if (loss) launch_k(overlap_launches(sh), k_pretrain_loss, 1, 1024, 0, st, sh.B, ws.scratch_d + sh.B, loss);
 }
 

@@ -108,8 +108,7 @@ void launch_init_walkers(const fn_system* s, int B, uint64_t seed, double std_, 
   const int64_t n = (int64_t)B * s->N * 3;
   ProfScope ps(s->prof, kProfInit, st);
   launch_k(true, k_init_walkers<Wlk>, (unsigned)((n + 255) / 256), 256, 0, st, B, s->N, s->d_elec_atom, s->d_nuclei,
-             std_, seed,
-                                                                     s->walker_offset, (Wlk*)walkers);
+           std_, seed, s->walker_offset, (Wlk*)walkers);
 }
 
 template <class Mode>
@@ -119,9 +118,7 @@ void launch_propose(const fn_system* s, int B, const void* walkers, void* out, d
   const int64_t n = (int64_t)B * ((3 * s->N + 1) / 2);
   ProfScope ps(s->prof, kProfSampler, st);
   launch_k(true, k_propose<Wlk>, (unsigned)((n + 127) / 128), 128, 0, st, B, s->N, (const Wlk*)walkers, (Wlk*)out,
-      step,
-             seed,
-                                                                step_idx, s->walker_offset);
+           step, seed, step_idx, s->walker_offset);
 }
 
 template <class Mode>
@@ -130,9 +127,7 @@ void launch_accept(const fn_system* s, int B, void* walkers, const void* prop, d
   using Wlk = typename Mode::Wlk;
   ProfScope ps(s->prof, kProfSampler, st);
   launch_k(true, k_accept<Wlk>, (B + 127) / 128, 128, 0, st, B, s->N, (Wlk*)walkers, (const Wlk*)prop, lp, lp_new,
-      seed,
-             step_idx,
-                                                  s->walker_offset, (unsigned long long*)accept_count);
+           seed, step_idx, s->walker_offset, (unsigned long long*)accept_count);
 }
 
 template <class Mode>

@@ -321,8 +321,7 @@ static void orbitals_cfg(const Shape& sh, const OrbArgs& a, int spin, cudaStream
 template <typename T>
 void launch_envelope(const Shape& sh, const OrbArgs& a, cudaStream_t st) {
   const int n_ko = a.K * std::max(sh.n_up, sh.n_dn);
-  launch_k(false, k_envelope<T>, dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st,
-      sh, a);
+  launch_k(false, k_envelope<T>, dim3(sh.tiles, (n_ko + kEnvOrbs - 1) / kEnvOrbs), kTileRows, 0, st, sh, a);
 }
 
 template <typename T>
