@@ -250,19 +250,22 @@ struct fn_system {
 
 namespace fn {
 
-// Whether a pass lets its kernels begin while their predecessors drain.  Value passes do up to
-// 2^18 rows: their kernels take 5 to 30 us and the gaps between them count (256-walker carbon atom
-// 205 -> 164 us, LiH training iteration 4.43 -> 3.85 ms).  Passes with tangent slabs only do while
-// tiny, up to 2^15 rows x slabs (H2, 700 walkers: 147 -> 128 us): in their longer kernels, CTAs that
-// arrive while only some SMs have room crowd onto those (C, 700 walkers, BF16: 841 -> 1176 us; N2,
-// 4096 walkers, FP32: 15.7 -> 16.5 ms).  FP64 kernels and the FMA-bound products of fn_simt.cu do not
-// overlap: two CTAs on one SM share its pipe while other SMs idle (H2 FP64 pass 1.34 -> 1.41 ms;
-// FP32 value pass of 300 Si- walkers 287 -> 388 us).
+// Whether a pass lets its kernels begin while their predecessors drain.  Value passes do up to 2^18 rows:
+// their kernels take 5 to 30 us and the gaps between them count.  BF16 log|psi| of N2 and C (4 x 256), LiH
+// (4 x 128) and H2 (2 x 32), time without overlap over time with it: 1.11 to 1.41 at 1000 to 4000 rows, 1.00
+// to 1.09 at 65536, 0.97 (N2) to 1.05 (H2) at 131072; above 2^18 rows overlap costs 0 to 5 %.  Passes with
+// tangent slabs only do while tiny, up to 2^15 rows x slabs (without: 1.03 to 1.17 x at 2000 to 8000,
+// 0.92 for N2 at 16016 to 1.16 for H2 at 32768): in their longer kernels, CTAs that arrive while only some
+// SMs have room crowd onto those (overlap at 32768 to 524288 rows x slabs: N2 1.02 to 1.09 x, C 1.11 to
+// 1.38 x slower; H2 and LiH 0.90 to 1.10).  FP64 kernels and the FMA-bound products of fn_simt.cu do not overlap: two
+// CTAs on one SM share its pipe while other SMs idle (H2 FP64 pass 1.34 -> 1.41 ms; FP32 value pass of 300
+// Si- walkers 287 -> 388 us); the other kernels of an FP32 value pass gain up to 5 % at 1000 rows, nothing above.
 inline bool overlap_launches(const Shape& sh, size_t word = 4) {
   return word == 4 && (int64_t)sh.T * sh.R <= ((int64_t)1 << (sh.T == 1 ? 18 : 15));
 }
 
-// The same for a product, by its rows (electrons, walkers, or slabs x walkers).
+// The same for a product, by its rows (electrons, walkers, or slabs x walkers): calls whose products do not
+// overlap take 1.03 to 1.15 x as long below 8192 rows; with overlap at every size 0.97 to 1.01 x.
 constexpr int64_t kOverlapGemmRows = 1 << 13;
 
 // Launch of a kernel that calls pdl_wait; with `overlap` it may begin while its predecessor in the

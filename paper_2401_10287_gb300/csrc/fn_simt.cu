@@ -149,7 +149,12 @@ static void layer_cfg(const Shape& sh, const LayerArgs& a, bool vec, cudaStream_
 }
 
 // Cost of a tile shape: CTAs on the busiest SM (at least the number that fills its FMA
-// pipe) x tile area / the shape's relative FMA rate.
+// pipe) x tile area / the shape's relative FMA rate.  FP32: the small tile has a quarter of the sums per
+// loaded operand, taken as half the rate.  Time with one tile only over the rule's, FP32 log|psi|: large
+// 1.48 to 2.2 up to 8192 rows, 1.00 to 1.26 at 65536; small 1.00 to 1.02 up to 4096 rows, 1.09 for N2 (4 x 256) at
+// 32760 rows and more, 0.93 to 0.95 for LiH (4 x 128) and 0.88 for C (3 x 64) at 65536, 0.89 for N2 at 16380.
+// FP64, where either tile saturates the pipe: large 1.2 to 1.8 up to 8192 rows (idle SMs), small 1.00 to 1.14; one warp
+// more or less per SM decides, which the equal rates count.
 template <typename Tl>
 static double tile_cost(int64_t ctas, int sm_count, int fill, double rate) {
   const int64_t per_sm = std::max<int64_t>((ctas + sm_count - 1) / sm_count, fill);
