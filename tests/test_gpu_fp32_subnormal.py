@@ -10,7 +10,7 @@ import pytest
 import torch
 
 import workloads as W
-from oracle import ansatz, mcmc
+from oracle import ansatz
 from gpu_helpers import make_pair, need_gpu, oracle_params, to_dev
 
 pytestmark = pytest.mark.gpu
